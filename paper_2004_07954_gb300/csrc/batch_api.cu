@@ -155,6 +155,7 @@ BatchArgs args_of(const wenozn_batch_params* bp, const Ptrs& p, int64_t cells, i
     a.gamma = bp->gamma;
     a.eps4 = 4.0 * bp->eps;
     a.kappa = zn_kappa(bp->A);
+    a.wide = wide_const(bp->eps, bp->A);
     a.cfl = bp->cfl;
     a.t_final = bp->t_final;
     return a;

@@ -171,13 +171,14 @@ __device__ __forceinline__ void split_cell_gen(const double* Uc, int split, doub
 // (cell_diffs).  Fh is in the sweep direction's frame.
 template <int NV>
 __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base, int stride,
-                                               double gm1, double eps4, double kappa, double* Fh) {
+                                               double gm1, const WideConst& wc, double eps4, double kappa,
+                                               double* Fh) {
     const int NC = s.NC;
     if (NV == 1) {
         Fh[0] = zn_split_flux(s.hp[base], s.hp[base + stride], s.hp[base + 2 * stride],
                               s.hp[base + 3 * stride], s.hp[base + 4 * stride],
                               s.hm[base + stride], s.hm[base + 2 * stride], s.hm[base + 3 * stride],
-                              s.hm[base + 4 * stride], s.hm[base + 5 * stride], eps4, kappa);
+                              s.hm[base + 4 * stride], s.hm[base + 5 * stride], wc, eps4, kappa);
         return;
     }
     // Roe average between the stencil's cells 2 and 3
@@ -239,8 +240,8 @@ __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base
     double gh[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-        const double fm = zn_flux_d(-Dm[3][k], -Dm[2][k], -Dm[1][k], -Dm[0][k], C[k], eps4, kappa);
-        gh[k] = zn_flux_d(Dp[0][k], Dp[1][k], Dp[2][k], Dp[3][k], fm, eps4, kappa);
+        const double fm = zn_flux_wide<true>(Dm[3][k], Dm[2][k], Dm[1][k], Dm[0][k], C[k], wc, eps4, kappa);
+        gh[k] = zn_flux_wide(Dp[0][k], Dp[1][k], Dp[2][k], Dp[3][k], fm, wc, eps4, kappa);
     }
     // back-projection F^ = R g^ with the right eigenvectors (columns)
     //   r_{u-c} = (1, u-c, [v,] H-uc), r_u = (1, u, [v,] q^2/2), r_shear = (0, 0, 1, v),

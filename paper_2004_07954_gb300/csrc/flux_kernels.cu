@@ -105,7 +105,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, int ta, int tc, dou
             interface_flux_gen<NV, GEN == 1>(sp, sidx(l, jl), kStride, gm1, a.eps4, a.kappa, a.weights,
                                              a.split, alpha_f, Fh);
         else
-            interface_flux<NV>(sp, sidx(l, jl), kStride, gm1, a.eps4, a.kappa, Fh);
+            interface_flux<NV>(sp, sidx(l, jl), kStride, gm1, a.wide, a.eps4, a.kappa, Fh);
         // store, undoing the direction frame
         if (DIR == 0) {
             const int64_t base = int64_t(line) * (a.nx + 1) + j;

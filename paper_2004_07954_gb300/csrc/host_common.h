@@ -81,6 +81,7 @@ inline FluxArgs flux_args(const wenozn_problem& p, const double* U, const unsign
     fa.ny = p.ny;
     fa.eps4 = 4.0 * p.eps;
     fa.kappa = zn_kappa(p.A);
+    fa.wide = wide_const(p.eps, p.A);
     fa.gamma = p.gamma;
     fa.adv_speed = p.adv_speed;
     fa.Fout = nullptr;

@@ -39,6 +39,7 @@ struct FluxArgs {
     int nx, ny, bc;                        // bc of the sweep direction (0 periodic, 1 outflow, 2 reflective)
     int weights, split;                    // weight function and flux splitting (wenozn.h enums)
     double eps4, kappa, gamma, adv_speed;  // eps4 = 4 eps, kappa = 2 / sqrt(A) (see zn_parts)
+    WideConst wide;                        // the same constants for the integer evaluation
 };
 // Admissible constants of the weights: with 1e-60 <= eps <= 1 and 1e-6 <= A <= 1e6 the
 // reconstruction's common denominator is a positive normal number and its range guard
@@ -100,6 +101,7 @@ struct BatchArgs {
     int stage;                 // 0, 1, 2
     int bc;                    // ghost map of every instance
     double gamma, eps4, kappa, cfl;
+    WideConst wide;
     double t_final;            // > 0: no instance steps past it
 };
 struct BatchShape { int tile, threads; };

@@ -1,0 +1,122 @@
+"""The integer evaluation of the reconstruction (csrc/wide_weights.cuh): compiled for the host
+against the binary128 oracle, and on the GPU at the edges of its range.
+
+Tolerance, from the operations: the numerator's operands are exact or off by 2^-58 of the
+largest difference Dmax, every weight a_k by less than 2^-53 relative, so f^ - c is off by less
+than 2^-52 Dmax before its rounding to 53 bits (|f^ - c| <= 7/6 Dmax), and the centre value is
+added with one more rounding: |error| <= 2^-51 (Dmax + |f^|)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2004_07954_gb300", "csrc")
+SHIM = """
+#include "wide_weights.cuh"
+extern "C" long wide_line(const double* f, long n, int side, double eps, double A, double* out) {
+    const wz::WideConst c = wz::wide_const(eps, A);
+    long refused = 0;
+    for (long j = 0; j <= n; ++j) {
+        const double* s = f + j;
+        double v[5], corr;
+        for (int k = 0; k < 5; ++k) v[k] = side > 0 ? s[k] : s[5 - k];
+        if (!wz::wide_correction(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], c, corr)) ++refused, corr = 0.0;
+        out[j] = v[2] + corr;
+    }
+    return refused;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def wide(tmp_path_factory):
+    d = tmp_path_factory.mktemp("wide")
+    src, so = str(d / "shim.cpp"), str(d / "shim.so")
+    with open(src, "w") as fh:
+        fh.write(SHIM)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, src, "-o", so],
+                   check=True)
+    L = ctypes.CDLL(so)
+    P = ctypes.c_void_p
+    L.wide_line.argtypes = [P, ctypes.c_long, ctypes.c_int, ctypes.c_double, ctypes.c_double, P]
+    L.wide_line.restype = ctypes.c_long
+
+    def line(f, side, eps=1e-40, A=10.0):
+        out = np.empty(f.size - 5)
+        refused = L.wide_line(f.ctypes.data, f.size - 6, side, eps, A, out.ctypes.data)
+        return out, refused
+
+    return line
+
+
+def _lines(n=600):
+    g = np.random.default_rng(7)
+    x = np.arange(n + 6) / n
+    smooth = np.sin(2 * np.pi * x) + 0.3 * np.cos(17 * x)
+    jumps = smooth + (x > 0.3) - 2.0 * (x > 0.31) + 1e3 * (x > 0.7)
+    return {
+        "random": g.normal(size=n + 6),
+        "smooth": smooth,
+        "jumps": jumps,
+        "steps": np.round(g.normal(size=n + 6)),                       # flat pieces, exact zeros
+        "noise beside jumps": np.where(x < 0.5, 1.0, -2.0) + 1e-15 * g.normal(size=n + 6),
+        "ranges": g.normal(size=n + 6) * 10.0 ** g.uniform(-30, 0, size=n + 6),
+        "flat": np.full(n + 6, 0.7),
+        "zeros": np.where(g.random(n + 6) < 0.5, 0.0, -0.0),
+    }
+
+
+def _bound(f, ref, side):
+    d = np.abs(np.diff(f))
+    win = np.lib.stride_tricks.sliding_window_view(d, 4).max(axis=1)
+    dmax = win[:-1] if side > 0 else win[1:]
+    return 2.0 ** -51 * (dmax + np.abs(ref))
+
+
+@pytest.mark.parametrize("eps,A", [(1e-40, 10.0), (1e-6, 10.0), (1e-60, 1e6), (1.0, 0.1)])
+@pytest.mark.parametrize("name", list(_lines()))
+def test_integer_evaluation_against_binary128(wide, orc, name, eps, A):
+    f = np.ascontiguousarray(_lines()[name])
+    for scale in (1.0, 2.0 ** -200, 2.0 ** 390):
+        fs = f * scale
+        for side in (1, -1):
+            got, refused = wide(fs, side, eps, A)
+            assert refused == 0 or scale != 1.0
+            ref = orc.reconstruct_quad(fs, side, eps=eps, A=A)
+            if refused == 0:
+                assert np.all(np.abs(got - ref) <= _bound(fs, ref, side)), (scale, side)
+
+
+def test_constant_data_are_exact_and_other_values_refused(wide):
+    for c in (0.0, -0.0, 0.1, -3.7e200):
+        got, refused = wide(np.full(40, c), 1)
+        assert refused == 0 and np.array_equal(got, np.full(35, c))
+    for bad in (np.nan, np.inf, 2.0 ** 402):
+        f = np.zeros(40)
+        f[20] = bad
+        assert wide(f, 1)[1] > 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", [-320, -301, -300, -299, 0, 398, 399, 400])
+def test_gpu_reconstruction_across_the_range_switch(orc, k):
+    """Differences on both sides of the exponents where the double evaluation takes over, block
+    and warp remainders, a NaN reaching exactly the stencils that hold it."""
+    import torch
+    from paper_2004_07954_gb300 import build, wenozn as W
+    build.build()
+    for n in (1, 31, 255, 256, 257, 600):
+        f = np.random.default_rng(n).normal(size=n + 6) * 2.0 ** k
+        t = torch.from_numpy(f).cuda()
+        out = torch.empty(n + 1, dtype=torch.float64, device="cuda")
+        for side in (1, -1):
+            W.wenozn_reconstruct(t, out, side)
+            ref = orc.reconstruct_quad(f, side)
+            # (the double evaluation's own bound in this suite is 1e-12 of the data's scale)
+            assert np.abs(out.cpu().numpy() - ref).max() <= 1e-12 * np.abs(f).max()
+    f[n // 2] = np.nan
+    W.wenozn_reconstruct(torch.from_numpy(f).cuda(), out, 1)
+    bad = np.isnan(out.cpu().numpy())
+    assert np.array_equal(np.flatnonzero(bad), np.arange(n // 2 - 4, n // 2 + 1))
