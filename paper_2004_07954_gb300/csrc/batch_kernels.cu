@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(THREADS, 2) batch_stage_kernel(BatchArgs a) {
             split_cell<NV>(Uc, alpha, 0.0, gm1, sp, i);
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < cl_used - 1; i += THREADS) cell_diffs<NV>(sp, i, 1);
+        for (int i = threadIdx.x; i < cl_used - 1; i += THREADS) cell_diffs_wide<NV>(sp, i, 1);
         __syncthreads();
         for (int jl = threadIdx.x; jl <= ncell; jl += THREADS) {     // interfaces c0 .. c0+ncell
             double Fh[NV];

@@ -10,22 +10,25 @@ namespace wz {
 
 // Shared-memory planes of one tile of NC cells: split fluxes h+ and h- (NV planes each),
 // and for the Euler systems sqrt(rho), u_n, H (and u_t in 2D), the differences
-// dh+-_c = h+-_c - h+-_{c+1} along the sweep (NV planes each) and, in the generic kernels,
-// the cell's |u_n| + c.
+// dh+-_c = h+-_c - h+-_{c+1} along the sweep (NV planes each; as doubles in the generic kernels,
+// as signed 64-bit mantissas with their exponents in the default ones) and, in the generic
+// kernels, the cell's |u_n| + c.
 template <int NV>
 struct CellPlanes {
     static constexpr int kPerCell = NV == 1 ? 2 : 2 * NV + (NV == 4 ? 4 : 3);
-    static constexpr int kPerCellDefault = kPerCell + (NV == 1 ? 0 : 2 * NV);   // + dh+, dh-
-    static constexpr int kPerCellGeneric = kPerCellDefault + (NV == 1 ? 0 : 1);   // + |u_n| + c
+    // + dh+, dh- and four exponent words (two 16-bit exponents each)
+    static constexpr int kPerCellDefault = kPerCell + (NV == 1 ? 0 : 2 * NV + 2);
+    static constexpr int kPerCellGeneric = kPerCell + (NV == 1 ? 0 : 2 * NV + 1);   // + dh+, dh-, |u_n| + c
     double* hp;
     double* hm;
     double* sr;
     double* un;
     double* H;
     double* ut;
-    double* dp;          // Euler: dh+ and dh-
+    double* dp;          // Euler: dh+ and dh- (mantissas: the same words as int64_t)
     double* dm;
     double* sp;          // generic kernels: the cell's |u_n| + c (local LF)
+    uint32_t* ex;        // default kernels: exponents of dh+ (0, 1), (2, 3) and dh- alike, a plane each
     int NC;
     __device__ __forceinline__ CellPlanes(double* base, int nc) : NC(nc) {
         hp = base;
@@ -36,7 +39,8 @@ struct CellPlanes {
         ut = H + nc;
         dp = base + kPerCell * nc;
         dm = dp + NV * nc;
-        sp = base + kPerCellDefault * nc;
+        sp = dm + NV * nc;
+        ex = reinterpret_cast<uint32_t*>(sp);
     }
 };
 
@@ -49,6 +53,22 @@ __device__ __forceinline__ void cell_diffs(const CellPlanes<NV>& s, int si, int 
     for (int k = 0; k < NV; ++k) {
         s.dp[k * s.NC + si] = s.hp[k * s.NC + si] - s.hp[k * s.NC + si + stride];
         s.dm[k * s.NC + si] = s.hm[k * s.NC + si] - s.hm[k * s.NC + si + stride];
+    }
+}
+
+// The same as mantissas and exponents for the integer projection.
+template <int NV>
+__device__ __forceinline__ void cell_diffs_wide(const CellPlanes<NV>& s, int si, int stride) {
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const double* h = side == 0 ? s.hp : s.hm;
+        int64_t* d = reinterpret_cast<int64_t*>(side == 0 ? s.dp : s.dm);
+        int e[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            d[k * s.NC + si] = wide_unpack(h[k * s.NC + si] - h[k * s.NC + si + stride], e[k]);
+        s.ex[2 * side * s.NC + si] = uint32_t(e[0] | (e[1] << 16));
+        s.ex[(2 * side + 1) * s.NC + si] = uint32_t(e[2] | (e[3] << 16));
     }
 }
 
@@ -166,46 +186,44 @@ __device__ __forceinline__ void split_cell_gen(const double* Uc, int split, doub
 }
 
 // Numerical flux F^ at the interface between the stencil's cells 2 and 3, the stencil being
-// the six cells base + k*stride, k = 0..5 (cells i-2 .. i+3 around x_{i+1/2}); for the
-// Euler systems the planes dh+ of cells 0..3 and dh- of cells 1..4 must be filled
-// (cell_diffs).  Fh is in the sweep direction's frame.
+// the six cells base + k*stride, k = 0..5 (cells i-2 .. i+3 around x_{i+1/2}), in the sweep
+// direction's frame: Roe average of cells 2 and 3, projection of the split fluxes onto its left
+// eigenvectors (rows, direction frame)
+//   l_{u-c} = ( (b2 + u/c)/2, -(b1 u + 1/c)/2, -b1 v/2, b1/2 )
+//   l_u     = ( 1 - b2, b1 u, b1 v, -b1 )
+//   l_shear = ( -v, 0, 1, 0 )                          (2D only)
+//   l_{u+c} = ( (b2 - u/c)/2, -(b1 u - 1/c)/2, -b1 v/2, b1/2 )
+// (b1 = (gamma - 1)/c^2, b2 = q^2 b1 / 2), reconstruction of both parts per field, and
+// back-projection F^ = R g^ with the right eigenvectors (columns)
+//   r_{u-c} = (1, u-c, [v,] H-uc), r_u = (1, u, [v,] q^2/2), r_shear = (0, 0, 1, v),
+//   r_{u+c} = (1, u+c, [v,] H+uc).
+// Each field's reconstructions need only the first differences of its stencil and the centre
+// value: plus side (g+ at cells 0..4) D_s = l.dh+ at cells s - 1, centre l.h+_2; minus side,
+// the mirrored stencil of g- at cells 5..1, D_s = -l.dh- at cells 5 - s, centre l.h-_3; both
+// centres at once as l.(h+_2 + h-_3).
 template <int NV>
-__device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base, int stride,
-                                               double gm1, const WideConst& wc, double eps4, double kappa,
-                                               double* Fh) {
-    const int NC = s.NC;
-    if (NV == 1) {
-        Fh[0] = zn_split_flux(s.hp[base], s.hp[base + stride], s.hp[base + 2 * stride],
-                              s.hp[base + 3 * stride], s.hp[base + 4 * stride],
-                              s.hm[base + stride], s.hm[base + 2 * stride], s.hm[base + 3 * stride],
-                              s.hm[base + 4 * stride], s.hm[base + 5 * stride], wc, eps4, kappa);
-        return;
+struct RoeState {
+    double u, v, H, c, hrc, hq2, hb1, hb2;       // hrc = 1/(2c), hq2 = q^2/2, hb1 = b1/2, hb2 = b2/2
+    __device__ __forceinline__ RoeState(const CellPlanes<NV>& s, int cl, int cr, double gm1) {
+        const double srl = s.sr[cl], srr = s.sr[cr];
+        const double rsum = rcp_nr(srl + srr);
+        const double wl = srl * rsum, wr = srr * rsum;
+        u = fma(wl, s.un[cl], wr * s.un[cr]);
+        v = NV == 4 ? fma(wl, s.ut[cl], wr * s.ut[cr]) : 0.0;
+        H = fma(wl, s.H[cl], wr * s.H[cr]);
+        const double q2 = NV == 4 ? fma(u, u, v * v) : u * u;
+        const double c2 = gm1 * fma(-0.5, q2, H);
+        const double rc = rsqrt(c2);
+        c = c2 * rc;
+        hrc = 0.5 * rc;
+        hq2 = 0.5 * q2;
+        hb1 = (0.5 * gm1) * (rc * rc);
+        hb2 = hq2 * hb1;
     }
-    // Roe average between the stencil's cells 2 and 3
-    const int cl = base + 2 * stride, cr = base + 3 * stride;
-    const double srl = s.sr[cl], srr = s.sr[cr];
-    const double rsum = rcp_nr(srl + srr);
-    const double wl = srl * rsum, wr = srr * rsum;
-    const double u = fma(wl, s.un[cl], wr * s.un[cr]);
-    const double v = NV == 4 ? fma(wl, s.ut[cl], wr * s.ut[cr]) : 0.0;
-    const double H = fma(wl, s.H[cl], wr * s.H[cr]);
-    const double q2 = NV == 4 ? fma(u, u, v * v) : u * u;
-    const double c2 = gm1 * fma(-0.5, q2, H);
-    const double rc = rsqrt(c2);
-    const double c = c2 * rc;
-    const double hrc = 0.5 * rc;
-    const double hq2 = 0.5 * q2;
-    const double hb1 = (0.5 * gm1) * (rc * rc);        // b1 / 2, b1 = (gamma - 1) / c^2
-    const double hb2 = hq2 * hb1;                      // b2 / 2, b2 = q^2 b1 / 2
-    // Projection onto the left eigenvectors of the Roe state (rows, direction frame)
-    //   l_{u-c} = ( (b2 + u/c)/2, -(b1 u + 1/c)/2, -b1 v/2, b1/2 )
-    //   l_u     = ( 1 - b2, b1 u, b1 v, -b1 )
-    //   l_shear = ( -v, 0, 1, 0 )                          (2D only)
-    //   l_{u+c} = ( (b2 - u/c)/2, -(b1 u - 1/c)/2, -b1 v/2, b1/2 )
-    // evaluated through their shared parts: with W = u h_1 + v h_2 - h_E,
-    // Z = b2 h_0 - b1 W and B = (u h_0 - h_1)/(2c),
+    // g = L h through the rows' shared parts: with W = u h_1 + v h_2 - h_E, Z = b2 h_0 - b1 W
+    // and B = (u h_0 - h_1)/(2c),
     //   l_u.h = h_0 - Z,  l_{u-+c}.h = Z/2 +- B,  l_shear.h = h_2 - v h_0.
-    auto project = [&](const double* h, double* g) {
+    __device__ __forceinline__ void project(const double* h, double* g) const {
         const double h0 = h[0], h1 = h[1], hE = h[NV - 1];
         const double W = NV == 4 ? fma(u, h1, fma(v, h[2], -hE)) : fma(u, h1, -hE);
         const double Zh = fma(hb2, h0, -(hb1 * W));          // Z / 2
@@ -214,51 +232,166 @@ __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base
         g[1] = fma(-2.0, Zh, h0);
         if (NV == 4) g[2] = fma(-v, h0, h[2]);
         g[NV - 1] = fma(-hrc, Bi, Zh);
-    };
-    auto project_at = [&](const double* planes, int i, double* g) {
-        double h[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) h[k] = planes[k * NC + i];
-        project(h, g);
-    };
-    // Each field's reconstructions need only the first differences of its stencil and the
-    // centre value: plus side (g+ at cells 0..4) D_s = l.dh+ at cells s - 1, centre l.h+_2;
-    // minus side, the mirrored stencil of g- at cells 5..1, D_s = -l.dh- at cells 5 - s,
-    // centre l.h-_3; both centres at once as l.(h+_2 + h-_3).
-    double Dp[4][NV], Dm[4][NV], C[NV];
-#pragma unroll
-    for (int st = 0; st < 4; ++st) {
-        project_at(s.dp, base + st * stride, Dp[st]);
-        project_at(s.dm, base + (st + 1) * stride, Dm[st]);
     }
+    __device__ __forceinline__ void back_project(const double* gh, double* Fh) const {
+        const double uc = u * c;
+        if (NV == 3) {
+            const double d20 = gh[2] - gh[0];
+            Fh[0] = gh[0] + gh[1] + gh[2];
+            Fh[1] = fma(u, Fh[0], c * d20);
+            Fh[2] = fma(H, gh[0] + gh[2], fma(uc, d20, hq2 * gh[1]));
+        } else {
+            const double d30 = gh[3] - gh[0];
+            Fh[0] = gh[0] + gh[1] + gh[3];
+            Fh[1] = fma(u, Fh[0], c * d30);
+            Fh[2] = fma(v, Fh[0], gh[2]);
+            Fh[3] = fma(H, gh[0] + gh[3], fma(uc, d30, fma(hq2, gh[1], v * gh[2])));
+        }
+    }
+};
+
+// The fields' f^ (both parts) in double arithmetic throughout, for stencils outside the range of
+// the integer projection.
+template <int NV>
+__device__ __noinline__ void field_fluxes_double(const CellPlanes<NV>& s, const RoeState<NV>& R, const double* C,
+                                                 int base, int stride, double eps4, double kappa, double* gh) {
+    double D[2][4][NV];
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side)
+#pragma unroll 1
+        for (int st = 0; st < 4; ++st) {
+            const double* h = side == 0 ? s.hp : s.hm;
+            const int i = base + (side == 0 ? st : 4 - st) * stride;
+            double dh[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) dh[k] = h[k * s.NC + i] - h[k * s.NC + i + stride];
+            R.project(dh, D[side][st]);
+        }
+#pragma unroll 1
+    for (int k = 0; k < NV; ++k) {
+        const double fm = zn_flux_d(-D[1][0][k], -D[1][1][k], -D[1][2][k], -D[1][3][k], C[k], eps4, kappa);
+        gh[k] = zn_flux_d(D[0][0][k], D[0][1][k], D[0][2][k], D[0][3][k], fm, eps4, kappa);
+    }
+}
+
+// The stencil differences projected in integer arithmetic.  All eight difference vectors (dh+ at
+// cells 0..3, dh- at cells 1..4) share one exponent per variable, so a projection is a sum of
+// products of integers whose coefficients were brought to a common scale once per
+// interface: the three fields of the density's dimension (u-c, u, u+c) share one, the shear
+// field has its own.  The scale is that of the sum's largest term in the stencil (an error of
+// 2^-55 of it, where the double projection rounds by 2^-54 in each of its steps).
+template <int NV>
+__device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base, int stride, double gm1,
+                                               const WideConst& wc, double eps4, double kappa, double* Fh) {
+    if (NV == 1) {
+        Fh[0] = zn_split_flux(s.hp[base], s.hp[base + stride], s.hp[base + 2 * stride],
+                              s.hp[base + 3 * stride], s.hp[base + 4 * stride],
+                              s.hm[base + stride], s.hm[base + 2 * stride], s.hm[base + 3 * stride],
+                              s.hm[base + 4 * stride], s.hm[base + 5 * stride], wc, eps4, kappa);
+        return;
+    }
+    const int NC = s.NC;
+    const RoeState<NV> R(s, base + 2 * stride, base + 3 * stride, gm1);
+    double gh[NV];
     {
         double hc[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) hc[k] = s.hp[k * NC + base + 2 * stride] + s.hm[k * NC + base + 3 * stride];
-        project(hc, C);
+        R.project(hc, gh);
     }
-    double gh[NV];
+
+    // the variables' exponents (16-bit pairs): the largest of the eight vectors'
+    uint32_t xa = 0, xb = 0;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const double fm = zn_flux_wide<true>(Dm[3][k], Dm[2][k], Dm[1][k], Dm[0][k], C[k], wc, eps4, kappa);
-        gh[k] = zn_flux_wide(Dp[0][k], Dp[1][k], Dp[2][k], Dp[3][k], fm, wc, eps4, kappa);
+    for (int st = 0; st < 4; ++st) {
+        const int i = base + st * stride;
+        xa = __vimax3_u16x2(xa, s.ex[i], s.ex[2 * NC + i + stride]);
+        xb = __vimax3_u16x2(xb, s.ex[NC + i], s.ex[3 * NC + i + stride]);
     }
-    // back-projection F^ = R g^ with the right eigenvectors (columns)
-    //   r_{u-c} = (1, u-c, [v,] H-uc), r_u = (1, u, [v,] q^2/2), r_shear = (0, 0, 1, v),
-    //   r_{u+c} = (1, u+c, [v,] H+uc)
-    const double uc = u * c;
-    if (NV == 3) {
-        const double d20 = gh[2] - gh[0];
-        Fh[0] = gh[0] + gh[1] + gh[2];
-        Fh[1] = fma(u, Fh[0], c * d20);
-        Fh[2] = fma(H, gh[0] + gh[2], fma(uc, d20, hq2 * gh[1]));
-    } else {
-        const double d30 = gh[3] - gh[0];
-        Fh[0] = gh[0] + gh[1] + gh[3];
-        Fh[1] = fma(u, Fh[0], c * d30);
-        Fh[2] = fma(v, Fh[0], gh[2]);
-        Fh[3] = fma(H, gh[0] + gh[3], fma(uc, d30, fma(hq2, gh[1], v * gh[2])));
+    const int X0 = int(xa & 0xffffu), X1 = int(xa >> 16), X2 = int(xb & 0xffffu), X3 = int(xb >> 16);
+    const int XE = NV == 4 ? X3 : X2;
+    // coefficients: Z/2 = z0 h_0 + z1 h_1 + [z2 h_2 +] zE h_E, B = p0 h_0 + p1 h_1, shear: h_2 + w0 h_0
+    int ez0, ez1, ez2 = 0, ezE, ep0, ep1, ew0 = 0;
+    int64_t z0 = wide_unpack(R.hb2, ez0), z1 = wide_unpack(-R.hb1 * R.u, ez1), zE = wide_unpack(R.hb1, ezE);
+    int64_t p0 = wide_unpack(R.hrc * R.u, ep0), p1 = wide_unpack(-R.hrc, ep1);
+    int64_t z2 = NV == 4 ? wide_unpack(-R.hb1 * R.v, ez2) : 0, w0 = NV == 4 ? wide_unpack(-R.v, ew0) : 0;
+    // a term's exponent, as of the double of its largest value
+    auto term = [](int e, int x) { return x == 0 ? 0 : e + x - 1022; };
+    const int tz0 = term(ez0, X0), tz1 = term(ez1, X1), tzE = term(ezE, XE), tp0 = term(ep0, X0), tp1 = term(ep1, X1);
+    const int tz2 = NV == 4 ? term(ez2, X2) : 0;
+    int G = max_i(max_i(max_i(tz0, tz1), max_i(tzE, tp0)), max_i(max_i(tp1, tz2), X0));
+    z0 = shr_s64(z0, G - tz0);
+    z1 = shr_s64(z1, G - tz1);
+    zE = shr_s64(zE, G - tzE);
+    p0 = shr_s64(p0, G - tp0);
+    p1 = shr_s64(p1, G - tp1);
+    if (NV == 4) z2 = shr_s64(z2, G - tz2);
+    const bool flat = (X0 | X1 | XE | (NV == 4 ? X2 : 0)) == 0;
+    G = flat ? wc.e_min : G + 4;
+    // the range of the integer evaluation: finite, not below the scale of eps (unless all zero)
+    bool ok = max_i(max_i(X0, X1), max_i(X2, X3)) < 2047;
+    ok = ok && (flat || (G >= wc.e_min && unsigned(G - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp)));
+    int Gw = 0;
+    if (NV == 4) {
+        const int tw = term(ew0, X0);
+        Gw = max_i(tw, X2);
+        w0 = shr_s64(w0, Gw - tw);
+        const bool flat2 = (X0 | X2) == 0;
+        Gw = flat2 ? wc.e_min : Gw + 4;
+        ok = ok && (flat2 || (Gw >= wc.e_min && unsigned(Gw - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp)));
     }
+    if (!ok) {
+        // (copies, so that the kept values need no address)
+        const RoeState<NV> Rc = R;
+        double C[NV], g2[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) C[k] = gh[k];
+        field_fluxes_double<NV>(s, Rc, C, base, stride, eps4, kappa, g2);
+        R.back_project(g2, Fh);
+        return;
+    }
+    const Limbs lz0(z0), lz1(z1), lz2(z2), lzE(zE), lp0(p0), lp1(p1), lw0(w0);
+
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        int64_t D[4][NV];
+        const int64_t* pl = reinterpret_cast<const int64_t*>(side == 0 ? s.dp : s.dm);
+        const uint32_t* ex = s.ex + 2 * side * NC;
+        const int step = side == 0 ? stride : -stride;
+        int i = side == 0 ? base : base + 4 * stride;
+#pragma unroll
+        for (int st = 0; st < 4; ++st, i += step) {
+            const uint32_t da = xa - ex[i], db = xb - ex[NC + i];
+            const int64_t h0 = shr_s64(pl[i], int(da & 0xffffu)), h1 = shr_s64(pl[NC + i], int(da >> 16));
+            const int64_t h2 = NV == 4 ? shr_s64(pl[2 * NC + i], int(db & 0xffffu)) : 0;
+            const int64_t hE = shr_s64(pl[(NV - 1) * NC + i], NV == 4 ? int(db >> 16) : int(db & 0xffffu));
+            const Limbs l0(h0), l1(h1), l2(h2), lE(hE);
+            int64_t zm = wide_mul(lz0.h, l0.h) + wide_mul(lz1.h, l1.h) + wide_mul(lzE.h, lE.h);
+            int64_t zc = wide_mul(lz0.h, l0.l) + wide_mul(lz0.l, l0.h) + wide_mul(lz1.h, l1.l) +
+                         wide_mul(lz1.l, l1.h) + wide_mul(lzE.h, lE.l) + wide_mul(lzE.l, lE.h);
+            if (NV == 4) {
+                zm += wide_mul(lz2.h, l2.h);
+                zc += wide_mul(lz2.h, l2.l) + wide_mul(lz2.l, l2.h);
+            }
+            const int64_t Z = zm + (zc >> 32);
+            const int64_t B = wide_mul(lp0.h, l0.h) + wide_mul(lp1.h, l1.h) +
+                              ((wide_mul(lp0.h, l0.l) + wide_mul(lp0.l, l0.h) + wide_mul(lp1.h, l1.l) +
+                                wide_mul(lp1.l, l1.h)) >> 32);
+            D[st][0] = Z + B;
+            D[st][NV - 1] = Z - B;
+            D[st][1] = shr_s64(h0, G - X0) - Z - Z;
+            if (NV == 4)
+                D[st][2] = shr_s64(h2, Gw - X2) + wide_mul(lw0.h, l0.h) +
+                           ((wide_mul(lw0.h, l0.l) + wide_mul(lw0.l, l0.h)) >> 32);
+        }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const double corr = wide_correction_int(D[0][k], D[1][k], D[2][k], D[3][k],
+                                                    NV == 4 && k == 2 ? Gw : G, wc);
+            gh[k] = side == 0 ? gh[k] + corr : gh[k] - corr;
+        }
+    }
+    R.back_project(gh, Fh);
 }
 
 // The interface flux of the generic kernels: weights and splitting chosen at run time.

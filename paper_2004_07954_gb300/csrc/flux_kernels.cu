@@ -20,17 +20,22 @@ namespace wz {
 
 namespace {
 
-// Tile shapes: TI interfaces along the sweep x TA lines across it, THREADS per block.
-// Long 1D lines use 507-interface tiles (512 cells with the halo: two full rounds of the cell
-// and difference passes); short ones (fewer tiles than twice the SM count) use 64-interface
-// tiles of 64 threads so that every SM gets work.
+// Tile shapes: TI interfaces along the sweep x TA lines across it, THREADS per block: one
+// interface a thread, and three blocks (24 warps) an SM in the default kernels (80 registers a
+// thread), because the FP64 phases of one block (cells, Roe state) have to run beside the
+// integer phases of others (4096^2, both sweeps: 10.45 ms; two interfaces a thread and two
+// blocks 11.37 ms, four blocks with 64 registers 10.35 ms but 104 against 90 us at 256^2).
+// Long 1D lines use 251-interface tiles (256 cells with the halo: one full round of the cell
+// and difference passes; a 2^20-cell step 0.95 ms against 1.08 ms with 507 and two blocks);
+// short ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
+// every SM gets work.
 template <int NV, int DIR, bool SMALL = false> struct Tile;
-template <> struct Tile<1, 0, false> { static constexpr int TI = 507, TA = 1, THREADS = 256; };
-template <> struct Tile<3, 0, false> { static constexpr int TI = 507, TA = 1, THREADS = 256; };
+template <> struct Tile<1, 0, false> { static constexpr int TI = 251, TA = 1, THREADS = 256; };
+template <> struct Tile<3, 0, false> { static constexpr int TI = 251, TA = 1, THREADS = 256; };
 template <> struct Tile<1, 0, true> { static constexpr int TI = 64, TA = 1, THREADS = 64; };
 template <> struct Tile<3, 0, true> { static constexpr int TI = 64, TA = 1, THREADS = 64; };
-template <> struct Tile<4, 0, false> { static constexpr int TI = 128, TA = 4, THREADS = 256; };
-template <> struct Tile<4, 1, false> { static constexpr int TI = 32, TA = 16, THREADS = 256; };
+template <> struct Tile<4, 0, false> { static constexpr int TI = 128, TA = 2, THREADS = 256; };
+template <> struct Tile<4, 1, false> { static constexpr int TI = 32, TA = 8, THREADS = 256; };
 
 // One tile of a sweep: tile ta along the sweep direction, tile tc across it.
 template <int NV, int DIR, bool SMALL, int GEN>
@@ -88,7 +93,9 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, int ta, int tc, dou
         for (int idx = threadIdx.x; idx < NC; idx += kThreads) {
             const int l = DIR == 0 ? idx / CL : idx % TA;
             const int lc = DIR == 0 ? idx % CL : idx / TA;
-            if (lc < cl_used - 1) cell_diffs<NV>(sp, sidx(l, lc), kStride);
+            if (lc >= cl_used - 1) continue;
+            if (GEN != 0) cell_diffs<NV>(sp, sidx(l, lc), kStride);
+            else cell_diffs_wide<NV>(sp, sidx(l, lc), kStride);
         }
         __syncthreads();
     }
@@ -124,7 +131,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, int ta, int tc, dou
 }
 
 template <int NV, int DIR, bool SMALL, int GEN>
-__global__ void __launch_bounds__(Tile<NV, DIR, SMALL>::THREADS, 2) flux_kernel(FluxArgs a) {
+__global__ void __launch_bounds__(Tile<NV, DIR, SMALL>::THREADS, GEN == 0 && !SMALL ? 3 : 2) flux_kernel(FluxArgs a) {
     extern __shared__ double smem[];
     pdl_wait();
     flux_tile<NV, DIR, SMALL, GEN>(a, DIR == 0 ? blockIdx.x : blockIdx.y, DIR == 0 ? blockIdx.y : blockIdx.x, smem);
@@ -134,8 +141,8 @@ __global__ void __launch_bounds__(Tile<NV, DIR, SMALL>::THREADS, 2) flux_kernel(
 // the x tiles (along the sweep fastest, as flux_kernel<4, 0>), the others the y tiles
 // (across the sweep fastest, as flux_kernel<4, 1>).
 template <int GEN>
-__global__ void __launch_bounds__(256, 2) flux_xy_kernel(FluxArgs ax, FluxArgs ay, int x_along, int nbx, int y_across) {
-    static_assert(Tile<4, 0>::THREADS == 256 && Tile<4, 1>::THREADS == 256, "one block size for both sweeps");
+__global__ void __launch_bounds__(256, GEN == 0 ? 3 : 2) flux_xy_kernel(FluxArgs ax, FluxArgs ay, int x_along, int nbx, int y_across) {
+    static_assert(Tile<4, 0>::THREADS == Tile<4, 1>::THREADS, "one block size for both sweeps");
     extern __shared__ double smem[];
     pdl_wait();
     const int b = int(blockIdx.x);
@@ -171,7 +178,7 @@ cudaError_t launch_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t s) {
     const int nbx = x_along * ((ax.ny + Tile<4, 0>::TA - 1) / Tile<4, 0>::TA);
     const int y_across = (ay.nx + Tile<4, 1>::TA - 1) / Tile<4, 1>::TA;
     const int nby = y_across * ((ay.ny + 1 + Tile<4, 1>::TI - 1) / Tile<4, 1>::TI);
-    return launch_pdl(flux_xy_kernel<GEN>, dim3(unsigned(nbx + nby)), dim3(256), smem, s, ax, ay, x_along, nbx,
+    return launch_pdl(flux_xy_kernel<GEN>, dim3(unsigned(nbx + nby)), dim3(Tile<4, 0>::THREADS), smem, s, ax, ay, x_along, nbx,
                       y_across);
 }
 

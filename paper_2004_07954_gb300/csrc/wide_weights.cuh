@@ -140,12 +140,12 @@ struct Limbs {
 WZ_HD int64_t wide_mul(int32_t a, int32_t b) { return int64_t(a) * b; }
 
 // b_k = beta_k + R of a sub-stencil: its second difference s and the factors p w of beta's
-// other part (beta = 4 s^2 + 3 p w) at the pair's scale, e its exponent.  B in [2^63, 2^64),
-// b = B 2^eb.
+// other part (beta = 4 s^2 + 3 p w) at the pair's scale, e its exponent: |2 s| <= 2^62,
+// |3 p|, |w| <= 3 2^60.  B in [2^63, 2^64), b = B 2^eb.
 WZ_HD uint64_t wide_indicator(int64_t s, int64_t p, int64_t w, int e, const WideConst& c, int& eb) {
     const Limbs S(s + s), P(p + p + p), Wl(w);
     const int64_t main = wide_mul(S.h, S.h) + wide_mul(P.h, Wl.h);
-    const int64_t cross = wide_mul(S.h + S.h, S.l) + wide_mul(P.h, Wl.l) + wide_mul(P.l, Wl.h);
+    const int64_t cross = wide_mul(S.h, S.l) + wide_mul(S.h, S.l) + wide_mul(P.h, Wl.l) + wide_mul(P.l, Wl.h);
     const uint64_t m = uint64_t(main + (cross >> 32)) + shr_u64(c.RM, 64 + 2 * e - c.eR);
     const int n = clz_u32(uint32_t(m >> 32));
     eb = 2 * e + 64 - n;
@@ -169,57 +169,24 @@ WZ_HD uint64_t wide_rcp(uint64_t d) {
     return r1 + ((uint64_t(uint32_t(r1 >> 32)) * e1) >> 31);
 }
 
-// f^ - c from the first differences; false where the caller has to take the double evaluation
-// (a difference outside the range above, infinite or not a number).
-WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const WideConst& c, double& corr) {
-    uint64_t u[4];
+// A double as a signed mantissa x, |x| in [2^59, 2^60), and its biased exponent e: the value is
+// x 2^(e - 1082).  Zeros and subnormals have e = 0 (a zero x = 0).
+WZ_HD int64_t wide_unpack(double v, int& e) {
 #ifdef __CUDA_ARCH__
-    u[0] = uint64_t(__double_as_longlong(D1));
-    u[1] = uint64_t(__double_as_longlong(D2));
-    u[2] = uint64_t(__double_as_longlong(D3));
-    u[3] = uint64_t(__double_as_longlong(D4));
+    const uint64_t u = uint64_t(__double_as_longlong(v));
 #else
-    std::memcpy(&u[0], &D1, 8);
-    std::memcpy(&u[1], &D2, 8);
-    std::memcpy(&u[2], &D3, 8);
-    std::memcpy(&u[3], &D4, 8);
+    uint64_t u;
+    std::memcpy(&u, &v, 8);
 #endif
-    // mantissas with their sign, |x| in [2^59, 2^60) (0 for zeros and subnormals' leading bit)
-    int64_t x[4];
-    int e[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t hi = uint32_t(u[i] >> 32), lo = uint32_t(u[i]);
-        e[i] = int((hi >> 20) & 0x7ffu);
-        const uint32_t mh = (hi & 0xfffffu) | (e[i] ? 0x100000u : 0u);
-        const uint64_t m = join(mh, lo) << 7;
-        const int64_t sg = int64_t(join(uint32_t(int32_t(hi) >> 31), uint32_t(int32_t(hi) >> 31)));
-        x[i] = (int64_t(m) ^ sg) - sg;
-    }
-    int e01 = max_i(e[0], e[1]), e12 = max_i(e[1], e[2]), e23 = max_i(e[2], e[3]);
-    const int E = max_i(e01, e23);
-    corr = 0.0;
-    if (unsigned(E - kWideMinExp) >= unsigned(kWideMaxExp - kWideMinExp)) return E == 0;
-    e01 = max_i(e01, c.e_min);
-    e12 = max_i(e12, c.e_min);
-    e23 = max_i(e23, c.e_min);
+    const uint32_t hi = uint32_t(u >> 32), sg = uint32_t(int32_t(hi) >> 31);
+    e = int((hi >> 20) & 0x7ffu);
+    const uint64_t m = join((hi & 0xfffffu) | (e ? 0x100000u : 0u), uint32_t(u)) << 7;
+    return int64_t((m ^ join(sg, sg)) - join(sg, sg));
+}
 
-    // the indicators
-    uint64_t b0, b1, b2;
-    int n0, n1, n2;                                           // exponents of b_k
-    {
-        const int64_t p = shr_s64(x[0], e01 - e[0]), q = shr_s64(x[1], e01 - e[1]);
-        b0 = wide_indicator(p - q, q, q + q - p, e01, c, n0);
-    }
-    {
-        const int64_t p = shr_s64(x[1], e12 - e[1]), q = shr_s64(x[2], e12 - e[2]);
-        b1 = wide_indicator(p - q, p, q, e12, c, n1);
-    }
-    {
-        const int64_t p = shr_s64(x[2], e23 - e[2]), q = shr_s64(x[3], e23 - e[3]);
-        b2 = wide_indicator(p - q, p, p + p - q, e23, c, n2);
-    }
-
+// f^ - c from the indicators b_k 2^(n_k) and the differences c_k 2^(E - 1082), |c_k| < 2^60.
+WZ_HD double wide_finish(uint64_t b0, uint64_t b1, uint64_t b2, int n0, int n1, int n2, int64_t c1, int64_t c2,
+                         int64_t c3, int64_t c4, int E, const WideConst& c) {
     // T = |b_0 - b_2| + R with the larger's exponent, h = min - R/2 with the smaller's
     const bool lt = n0 < n2 || (n0 == n2 && b0 < b2);
     const uint64_t mx = lt ? b2 : b0, mn = lt ? b0 : b2;
@@ -227,15 +194,11 @@ WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const Wid
     uint64_t T = mx - shr_u64(mn, nx - nn) + shr_u64(c.RM, nx - c.eR);
     const uint64_t h = mn - shr_u64(c.RM, nn - c.eR + 1);
 
-    // differences at the scale of the largest, |c_i| < 2^58
-    const int64_t c1 = shr_s64(x[0], E - e[0] + 2), c2 = shr_s64(x[1], E - e[1] + 2);
-    const int64_t c3 = shr_s64(x[2], E - e[2] + 2), c4 = shr_s64(x[3], E - e[3] + 2);
+    // z = K |d4| T from normalised factors (both may have lost their leading bits); Y = z^2
     const int64_t d23 = c2 - c3;
     const int64_t d4 = (c1 - c4) - (d23 + d23 + d23);
-
-    // z = K |d4| T from normalised factors (both may have lost their leading bits); Y = z^2
     uint64_t ad = uint64_t(d4 < 0 ? -d4 : d4);
-    int ez = E + nx + c.eK + 130;
+    int ez = E + nx + c.eK + 128;
     {
         const bool low = (ad >> 32) == 0;
         ad = low ? ad << 32 : ad;
@@ -277,21 +240,22 @@ WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const Wid
     const uint64_t a1 = (Xs + shr_u64(Y1, ec - f1)) * 6;
     const uint64_t a2 = (Xs + shr_u64(Y2, ec - f2)) * 3;
 
-    // numerator: sums of limb products, 96 bits kept
+    // numerator: sums of limb products, 96 bits kept (|A_h| < 2^30, |G_h| < 2^31)
     const Limbs A0{int64_t(a0)}, A1{int64_t(a1)}, A2{int64_t(a2)};
     const Limbs G0(c1 + c1 - 5 * c2), G1(c2 + c3 + c3), G2(c4 - 4 * c3);
     const int64_t main = wide_mul(A0.h, G0.h) - wide_mul(A1.h, G1.h) + wide_mul(A2.h, G2.h);
-    const int64_t cross = wide_mul(A0.h, G0.l) + wide_mul(A0.l, G0.h) - wide_mul(A1.h, G1.l) - wide_mul(A1.l, G1.h) +
-                          wide_mul(A2.h, G2.l) + wide_mul(A2.l, G2.h);
-    int64_t top = main + (cross >> 32);
-    uint32_t low = uint32_t(cross);
+    const int64_t cr1 = wide_mul(A0.h, G0.l) - wide_mul(A1.h, G1.l) + wide_mul(A2.h, G2.l);
+    const int64_t cr2 = wide_mul(A0.l, G0.h) - wide_mul(A1.l, G1.h) + wide_mul(A2.l, G2.h);
+    const uint64_t lows = uint64_t(uint32_t(cr1)) + uint32_t(cr2);
+    int64_t top = main + (cr1 >> 32) + (cr2 >> 32) + int64_t(lows >> 32);
+    uint32_t low = uint32_t(lows);
     const uint32_t sign = uint32_t(uint64_t(top) >> 32) & 0x80000000u;
     if (top < 0) {                                            // magnitude of the 96-bit value
         top = ~top;
         low = ~low;
     }
     uint32_t th = uint32_t(uint64_t(top) >> 32), tm = uint32_t(top);
-    int en = E + 6;
+    int en = E + 4;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const bool up = th == 0;
@@ -315,11 +279,86 @@ WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const Wid
     const uint32_t ex = uint32_t(en - nt + nd - nq - 1) << 20;
     const uint64_t bits = th == 0 ? 0 : r + join(ex | sign, 0);
 #ifdef __CUDA_ARCH__
-    corr = __longlong_as_double((long long)bits);
+    return __longlong_as_double((long long)bits);
 #else
+    double corr;
     std::memcpy(&corr, &bits, 8);
+    return corr;
 #endif
+}
+
+// f^ - c from the first differences; false where the caller has to take the double evaluation
+// (a difference outside the range above, infinite or not a number).
+WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const WideConst& c, double& corr) {
+    int e0, e1, e2, e3;
+    const int64_t x0 = wide_unpack(D1, e0), x1 = wide_unpack(D2, e1), x2 = wide_unpack(D3, e2),
+                  x3 = wide_unpack(D4, e3);
+    int e01 = max_i(e0, e1), e12 = max_i(e1, e2), e23 = max_i(e2, e3);
+    const int E = max_i(e01, e23);
+    corr = 0.0;
+    if (unsigned(E - kWideMinExp) >= unsigned(kWideMaxExp - kWideMinExp)) return E == 0;
+    e01 = max_i(e01, c.e_min);
+    e12 = max_i(e12, c.e_min);
+    e23 = max_i(e23, c.e_min);
+    uint64_t b0, b1, b2;
+    int n0, n1, n2;                                           // exponents of b_k
+    {
+        const int64_t p = shr_s64(x0, e01 - e0), q = shr_s64(x1, e01 - e1);
+        b0 = wide_indicator(p - q, q, q + q - p, e01, c, n0);
+    }
+    {
+        const int64_t p = shr_s64(x1, e12 - e1), q = shr_s64(x2, e12 - e2);
+        b1 = wide_indicator(p - q, p, q, e12, c, n1);
+    }
+    {
+        const int64_t p = shr_s64(x2, e23 - e2), q = shr_s64(x3, e23 - e3);
+        b2 = wide_indicator(p - q, p, p + p - q, e23, c, n2);
+    }
+    corr = wide_finish(b0, b1, b2, n0, n1, n2, shr_s64(x0, E - e0), shr_s64(x1, E - e1), shr_s64(x2, E - e2),
+                       shr_s64(x3, E - e3), E, c);
     return true;
+}
+
+WZ_HD int64_t shl_s64(int64_t x, int n) {            // n >= 0, zero from 64 on
+#ifdef __CUDA_ARCH__
+    int64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+    return r;
+#else
+    return n > 63 ? 0 : int64_t(uint64_t(x) << n);
+#endif
+}
+
+// The exponent of the integer D in units 2^(G - 1082), |D| < 2^60, brought to [2^59, 2^60] (the
+// upper end for a negative power of two); 0 for D = 0.
+WZ_HD int wide_exponent(int64_t D, int G) {
+    const uint32_t s = uint32_t(uint64_t(D >> 63)), h = uint32_t(uint64_t(D) >> 32) ^ s, l = uint32_t(D) ^ s;
+    const bool low = h == 0;
+    const int n = clz_u32((low ? l : h) | 1u) + (low ? 28 : -4);
+    return D == 0 ? 0 : G - max_i(n, 0);
+}
+
+// f^ - c from integer differences D_k 2^(G - 1082), |D_k| < 2^60, G >= e_min unless all are zero.
+WZ_HD double wide_correction_int(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G, const WideConst& c) {
+    const int e0 = wide_exponent(D1, G), e1 = wide_exponent(D2, G), e2 = wide_exponent(D3, G),
+              e3 = wide_exponent(D4, G);
+    const int e01 = max_i(max_i(e0, e1), c.e_min), e12 = max_i(max_i(e1, e2), c.e_min),
+              e23 = max_i(max_i(e2, e3), c.e_min);
+    uint64_t b0, b1, b2;
+    int n0, n1, n2;
+    {
+        const int64_t p = shl_s64(D1, G - e01), q = shl_s64(D2, G - e01);
+        b0 = wide_indicator(p - q, q, q + q - p, e01, c, n0);
+    }
+    {
+        const int64_t p = shl_s64(D2, G - e12), q = shl_s64(D3, G - e12);
+        b1 = wide_indicator(p - q, p, q, e12, c, n1);
+    }
+    {
+        const int64_t p = shl_s64(D3, G - e23), q = shl_s64(D4, G - e23);
+        b2 = wide_indicator(p - q, p, p + p - q, e23, c, n2);
+    }
+    return wide_finish(b0, b1, b2, n0, n1, n2, D1, D2, D3, D4, G, c);
 }
 
 }  // namespace wz

@@ -120,3 +120,49 @@ def test_gpu_reconstruction_across_the_range_switch(orc, k):
     W.wenozn_reconstruct(torch.from_numpy(f).cuda(), out, 1)
     bad = np.isnan(out.cpu().numpy())
     assert np.array_equal(np.flatnonzero(bad), np.arange(n // 2 - 4, n // 2 + 1))
+
+
+def _state_2d(kind, nx, ny):
+    """2D Euler states that put the integer projection at its limits."""
+    from paper_2004_07954_gb300 import inputs
+    g = np.random.default_rng(5)
+    one = np.ones((ny, nx))
+    rho, u, v, p = 1.0 + 0.2 * g.random((ny, nx)), 0.3 * g.random((ny, nx)), 0.2 * g.random((ny, nx)), 1.0 + 0.1 * g.random((ny, nx))
+    if kind == "rest":                       # every difference zero, momenta zero
+        rho, u, v, p = one, 0 * one, 0 * one, one
+    elif kind == "signed zeros":
+        rho, u, v, p = one, -0.0 * one, 0 * one, one
+    elif kind == "tiny shear":               # transverse differences below the scale of eps
+        v = 1e-30 * g.normal(size=(ny, nx))
+    elif kind == "blast":                    # neighbouring cells 10^5 apart in pressure, along a front
+        p = p * np.where(np.arange(nx) < nx // 2, 1000.0, 0.01)
+    elif kind == "low Mach":
+        u, v = 1e-6 * u, 1e-6 * v
+    elif kind == "units":                    # c = 340, E = 2.5e5: variables of unlike magnitude
+        rho, u, v, p = 1.2 * rho, 300.0 * u, 200.0 * v, 1.0e5 * p
+    elif kind == "supersonic":
+        u = u - 8.0
+    elif kind == "one jump":
+        rho, u, v, p = np.where(np.arange(nx) < nx // 2, 1.0, 0.125) * one, 0 * one, 0 * one, np.where(np.arange(nx) < nx // 2, 1.0, 0.1) * one
+    return np.ascontiguousarray(inputs.cons_from_prim(rho, u, p, v))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["rest", "signed zeros", "tiny shear", "blast", "low Mach", "units", "supersonic", "one jump"])
+def test_gpu_integer_projection(orc, kind):
+    """The RHS at the suite's bound (1e-12 of its largest value, per variable), tile remainders."""
+    import torch
+    from paper_2004_07954_gb300 import build, wenozn as W
+    build.build()
+    for nx, ny in ((131, 9), (5, 35), (64, 33)):
+        U = _state_2d(kind, nx, ny)
+        p = W.wenozn_problem_init(2, nx, ny, 1.0 / nx, 1.0 / ny)
+        got = W.Solver(p).rhs(torch.from_numpy(U).cuda()).cpu().numpy()
+        want = orc.rhs(orc.problem(2, nx, ny, dx=1.0 / nx, dy=1.0 / ny), U)
+        if kind in ("rest", "signed zeros"):
+            assert np.abs(got).max() == 0.0
+            continue
+        for k in range(4):
+            # rounding of the fluxes whose differences the RHS is: 1e-12 of the largest flux / dx
+            scale = max(np.abs(want[k]).max(), 1e-3 * np.abs(want).max())
+            assert np.abs(got[k] - want[k]).max() <= 1e-12 * scale, k
