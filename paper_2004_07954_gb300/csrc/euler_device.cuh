@@ -203,7 +203,7 @@ __device__ __forceinline__ void split_cell_gen(const double* Uc, int split, doub
 // centres at once as l.(h+_2 + h-_3).
 template <int NV>
 struct RoeState {
-    double u, v, H, c, hrc, hq2, hb1, hb2;       // hrc = 1/(2c), hq2 = q^2/2, hb1 = b1/2, hb2 = b2/2
+    double u, v, H, c, hrc, hq2, hb1, hb2;   // hrc = 1/(2c), hq2 = q^2/2, hb1 = b1/2, hb2 = b2/2
     __device__ __forceinline__ RoeState(const CellPlanes<NV>& s, int cl, int cr, double gm1) {
         const double srl = s.sr[cl], srr = s.sr[cr];
         const double rsum = rcp_nr(srl + srr);
@@ -274,12 +274,77 @@ __device__ __noinline__ void field_fluxes_double(const CellPlanes<NV>& s, const 
     }
 }
 
-// The stencil differences projected in integer arithmetic.  All eight difference vectors (dh+ at
-// cells 0..3, dh- at cells 1..4) share one exponent per variable, so a projection is a sum of
-// products of integers whose coefficients were brought to a common scale once per
-// interface: the three fields of the density's dimension (u-c, u, u+c) share one, the shear
-// field has its own.  The scale is that of the sum's largest term in the stencil (an error of
-// 2^-55 of it, where the double projection rounds by 2^-54 in each of its steps).
+// The stencil differences projected in integer arithmetic: Z/2, B and v h_0 of each difference
+// vector are sums of products of the vector's mantissas and the coefficients', brought to the
+// exponent of the sum's largest term at that point (so every point keeps its own relative
+// accuracy; an error of 2^-55 of that term, where the double projection rounds by 2^-54 in each
+// of its steps).
+template <int NV>
+struct WideProjection {
+    // Z/2 = z0 h_0 + z1 h_1 + [z2 h_2 +] zE h_E, B = p0 h_0 + p1 h_1, shear: h_2 + w0 h_0; the
+    // coefficients of h_0 (and of h_1) in Z/2 and B share an exponent
+    Limbs z0, z1, z2, zE, p0, p1, w0;
+    int e0, e1, e2, eE, ew;
+    __device__ __forceinline__ explicit WideProjection(const RoeState<NV>& R)
+        : z0(0), z1(0), z2(0), zE(0), p0(0), p1(0), w0(0), e2(0), ew(0) {
+        int a, b;
+        const int64_t c0 = wide_unpack(R.hb2, a), b0 = wide_unpack(R.hrc * R.u, b);
+        e0 = max_i(a, b);
+        z0 = Limbs(shr_s64(c0, e0 - a));
+        p0 = Limbs(shr_s64(b0, e0 - b));
+        const int64_t c1 = wide_unpack(-R.hb1 * R.u, a), b1 = wide_unpack(-R.hrc, b);
+        e1 = max_i(a, b);
+        z1 = Limbs(shr_s64(c1, e1 - a));
+        p1 = Limbs(shr_s64(b1, e1 - b));
+        zE = Limbs(wide_unpack(R.hb1, eE));
+        if (NV == 4) {
+            z2 = Limbs(wide_unpack(-R.hb1 * R.v, e2));
+            w0 = Limbs(wide_unpack(-R.v, ew));
+        }
+    }
+    // D[k] 2^(G[k] - 1082), |D[k]| < 2^60, of the vector at index i of the mantissa planes pl and
+    // exponent planes ex; xm: running maximum of the exponents
+    __device__ __forceinline__ void apply(const int64_t* pl, const uint32_t* ex, int NC, int i, int64_t* D, int* G,
+                                          uint32_t& xm) const {
+        const uint32_t xa = ex[i], xb = ex[NC + i];
+        xm = __vimax3_u16x2(xm, xa, xb);
+        const int x0 = int(xa & 0xffffu), x1 = int(xa >> 16), x2 = int(xb & 0xffffu);
+        const int xE = NV == 4 ? int(xb >> 16) : x2;
+        const int64_t h0 = pl[i], h1 = pl[NC + i], h2 = NV == 4 ? pl[2 * NC + i] : 0, hE = pl[(NV - 1) * NC + i];
+        // a term's exponent, as of the double of its largest value (+ 1022)
+        const int t0 = e0 + x0, t1 = e1 + x1, tE = eE + xE, t2 = NV == 4 ? e2 + x2 : 0;
+        const int t = max_i(max_i(t0, t1), max_i(t2, tE));
+        const Limbs l0(shr_s64(h0, t - t0)), l1(shr_s64(h1, t - t1)), lE(shr_s64(hE, t - tE));
+        int64_t zm = wide_mul(z0.h, l0.h) + wide_mul(z1.h, l1.h) + wide_mul(zE.h, lE.h);
+        int64_t zc = wide_mul(z0.h, l0.l) + wide_mul(z0.l, l0.h) + wide_mul(z1.h, l1.l) + wide_mul(z1.l, l1.h) +
+                     wide_mul(zE.h, lE.l) + wide_mul(zE.l, lE.h);
+        if (NV == 4) {
+            const Limbs l2(shr_s64(h2, t - t2));
+            zm += wide_mul(z2.h, l2.h);
+            zc += wide_mul(z2.h, l2.l) + wide_mul(z2.l, l2.h);
+        }
+        const int64_t Z = zm + (zc >> 32);                               // units 2^(g - 1082)
+        const int64_t B = wide_mul(p0.h, l0.h) + wide_mul(p1.h, l1.h) +
+                          ((wide_mul(p0.h, l0.l) + wide_mul(p0.l, l0.h) + wide_mul(p1.h, l1.l) +
+                            wide_mul(p1.l, l1.h)) >> 32);
+        const int g = t - 1018;
+        D[0] = Z + B;
+        D[NV - 1] = Z - B;
+        G[0] = G[NV - 1] = g;
+        // h_0 - 2 Z/2 at its own scale
+        const int gu = max_i(g + 2, x0 + 1);
+        D[1] = shr_s64(h0, gu - x0) - (shr_s64(Z, gu - g) << 1);
+        G[1] = gu;
+        if (NV == 4) {
+            const int gp = ew + x0 - 1018, gw = max_i(gp + 1, x2 + 1);  // w0 h_0 / 2^64 in units 2^(gp - 1082)
+            const Limbs m0(h0);
+            const int64_t P = wide_mul(w0.h, m0.h) + ((wide_mul(w0.h, m0.l) + wide_mul(w0.l, m0.h)) >> 32);
+            D[2] = shr_s64(h2, gw - x2) + shr_s64(P, gw - gp);
+            G[2] = gw;
+        }
+    }
+};
+
 template <int NV>
 __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base, int stride, double gm1,
                                                const WideConst& wc, double eps4, double kappa, double* Fh) {
@@ -292,104 +357,44 @@ __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base
     }
     const int NC = s.NC;
     const RoeState<NV> R(s, base + 2 * stride, base + 3 * stride, gm1);
-    double gh[NV];
+    double gh[NV], C[NV];
     {
         double hc[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) hc[k] = s.hp[k * NC + base + 2 * stride] + s.hm[k * NC + base + 3 * stride];
-        R.project(hc, gh);
+        R.project(hc, C);
     }
-
-    // the variables' exponents (16-bit pairs): the largest of the eight vectors'
-    uint32_t xa = 0, xb = 0;
 #pragma unroll
-    for (int st = 0; st < 4; ++st) {
-        const int i = base + st * stride;
-        xa = __vimax3_u16x2(xa, s.ex[i], s.ex[2 * NC + i + stride]);
-        xb = __vimax3_u16x2(xb, s.ex[NC + i], s.ex[3 * NC + i + stride]);
-    }
-    const int X0 = int(xa & 0xffffu), X1 = int(xa >> 16), X2 = int(xb & 0xffffu), X3 = int(xb >> 16);
-    const int XE = NV == 4 ? X3 : X2;
-    // coefficients: Z/2 = z0 h_0 + z1 h_1 + [z2 h_2 +] zE h_E, B = p0 h_0 + p1 h_1, shear: h_2 + w0 h_0
-    int ez0, ez1, ez2 = 0, ezE, ep0, ep1, ew0 = 0;
-    int64_t z0 = wide_unpack(R.hb2, ez0), z1 = wide_unpack(-R.hb1 * R.u, ez1), zE = wide_unpack(R.hb1, ezE);
-    int64_t p0 = wide_unpack(R.hrc * R.u, ep0), p1 = wide_unpack(-R.hrc, ep1);
-    int64_t z2 = NV == 4 ? wide_unpack(-R.hb1 * R.v, ez2) : 0, w0 = NV == 4 ? wide_unpack(-R.v, ew0) : 0;
-    // a term's exponent, as of the double of its largest value
-    auto term = [](int e, int x) { return x == 0 ? 0 : e + x - 1022; };
-    const int tz0 = term(ez0, X0), tz1 = term(ez1, X1), tzE = term(ezE, XE), tp0 = term(ep0, X0), tp1 = term(ep1, X1);
-    const int tz2 = NV == 4 ? term(ez2, X2) : 0;
-    int G = max_i(max_i(max_i(tz0, tz1), max_i(tzE, tp0)), max_i(max_i(tp1, tz2), X0));
-    z0 = shr_s64(z0, G - tz0);
-    z1 = shr_s64(z1, G - tz1);
-    zE = shr_s64(zE, G - tzE);
-    p0 = shr_s64(p0, G - tp0);
-    p1 = shr_s64(p1, G - tp1);
-    if (NV == 4) z2 = shr_s64(z2, G - tz2);
-    const bool flat = (X0 | X1 | XE | (NV == 4 ? X2 : 0)) == 0;
-    G = flat ? wc.e_min : G + 4;
-    // the range of the integer evaluation: finite, not below the scale of eps (unless all zero)
-    bool ok = max_i(max_i(X0, X1), max_i(X2, X3)) < 2047;
-    ok = ok && (flat || (G >= wc.e_min && unsigned(G - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp)));
-    int Gw = 0;
-    if (NV == 4) {
-        const int tw = term(ew0, X0);
-        Gw = max_i(tw, X2);
-        w0 = shr_s64(w0, Gw - tw);
-        const bool flat2 = (X0 | X2) == 0;
-        Gw = flat2 ? wc.e_min : Gw + 4;
-        ok = ok && (flat2 || (Gw >= wc.e_min && unsigned(Gw - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp)));
-    }
-    if (!ok) {
-        // (copies, so that the kept values need no address)
-        const RoeState<NV> Rc = R;
-        double C[NV], g2[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) C[k] = gh[k];
-        field_fluxes_double<NV>(s, Rc, C, base, stride, eps4, kappa, g2);
-        R.back_project(g2, Fh);
-        return;
-    }
-    const Limbs lz0(z0), lz1(z1), lz2(z2), lzE(zE), lp0(p0), lp1(p1), lw0(w0);
-
+    for (int k = 0; k < NV; ++k) gh[k] = C[k];
+    const WideProjection<NV> W(R);
+    uint32_t xm = 0;
+    bool ok = true;
 #pragma unroll 1
     for (int side = 0; side < 2; ++side) {
         int64_t D[4][NV];
+        int G[4][NV];
         const int64_t* pl = reinterpret_cast<const int64_t*>(side == 0 ? s.dp : s.dm);
-        const uint32_t* ex = s.ex + 2 * side * NC;
         const int step = side == 0 ? stride : -stride;
-        int i = side == 0 ? base : base + 4 * stride;
 #pragma unroll
-        for (int st = 0; st < 4; ++st, i += step) {
-            const uint32_t da = xa - ex[i], db = xb - ex[NC + i];
-            const int64_t h0 = shr_s64(pl[i], int(da & 0xffffu)), h1 = shr_s64(pl[NC + i], int(da >> 16));
-            const int64_t h2 = NV == 4 ? shr_s64(pl[2 * NC + i], int(db & 0xffffu)) : 0;
-            const int64_t hE = shr_s64(pl[(NV - 1) * NC + i], NV == 4 ? int(db >> 16) : int(db & 0xffffu));
-            const Limbs l0(h0), l1(h1), l2(h2), lE(hE);
-            int64_t zm = wide_mul(lz0.h, l0.h) + wide_mul(lz1.h, l1.h) + wide_mul(lzE.h, lE.h);
-            int64_t zc = wide_mul(lz0.h, l0.l) + wide_mul(lz0.l, l0.h) + wide_mul(lz1.h, l1.l) +
-                         wide_mul(lz1.l, l1.h) + wide_mul(lzE.h, lE.l) + wide_mul(lzE.l, lE.h);
-            if (NV == 4) {
-                zm += wide_mul(lz2.h, l2.h);
-                zc += wide_mul(lz2.h, l2.l) + wide_mul(lz2.l, l2.h);
-            }
-            const int64_t Z = zm + (zc >> 32);
-            const int64_t B = wide_mul(lp0.h, l0.h) + wide_mul(lp1.h, l1.h) +
-                              ((wide_mul(lp0.h, l0.l) + wide_mul(lp0.l, l0.h) + wide_mul(lp1.h, l1.l) +
-                                wide_mul(lp1.l, l1.h)) >> 32);
-            D[st][0] = Z + B;
-            D[st][NV - 1] = Z - B;
-            D[st][1] = shr_s64(h0, G - X0) - Z - Z;
-            if (NV == 4)
-                D[st][2] = shr_s64(h2, Gw - X2) + wide_mul(lw0.h, l0.h) +
-                           ((wide_mul(lw0.h, l0.l) + wide_mul(lw0.l, l0.h)) >> 32);
-        }
+        for (int st = 0; st < 4; ++st)
+            W.apply(pl, s.ex + 2 * side * NC, NC, (side == 0 ? base : base + 4 * stride) + st * step, D[st], G[st], xm);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const double corr = wide_correction_int(D[0][k], D[1][k], D[2][k], D[3][k],
-                                                    NV == 4 && k == 2 ? Gw : G, wc);
+            double corr;
+            ok = wide_correction(D[0][k], D[1][k], D[2][k], D[3][k], G[0][k], G[1][k], G[2][k], G[3][k], wc, corr) && ok;
             gh[k] = side == 0 ? gh[k] + corr : gh[k] - corr;
         }
+    }
+    if (!ok || (xm & 0xffffu) == 2047u || (xm >> 16) == 2047u) {
+        // out of the integer evaluation's range, infinite or not a number (copies, so that the
+        // kept values need no address)
+        const RoeState<NV> Rc = R;
+        double Cc[NV], gd[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) Cc[k] = C[k];
+        field_fluxes_double<NV>(s, Rc, Cc, base, stride, eps4, kappa, gd);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) gh[k] = gd[k];
     }
     R.back_project(gh, Fh);
 }

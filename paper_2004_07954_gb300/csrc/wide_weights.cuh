@@ -27,10 +27,10 @@
 // and f^ - c = (a_0 g_0 + 6 a_1 g_1 + 3 a_2 g_2) / (6 (a_0 + 6 a_1 + 3 a_2)) with
 //   g_0 = 2 D1 - 5 D2,  g_1 = -(D2 + 2 D3),  g_2 = D4 - 4 D3.
 //
-// Scales.  D_i enters with the scale of its sub-stencil's pair in beta_k (relative accuracy of
-// a flat sub-stencil beside a jump) and with the scale of the largest difference in d4 and
-// g_k, where an error of 2^-58 of that difference is below the result's own rounding.  A pair
-// scale is never below that of sqrt(eps), so b_k >= R > 0 always has its leading bits.
+// Scales.  Each D_i comes with an exponent of its own.  A sub-stencil's pair takes the scale of
+// its larger difference, each weight a_k and each product a_k g_k an exponent of its own too,
+// so a flat sub-stencil beside a jump keeps its full relative accuracy (the result there is
+// its small difference, whatever the jump).  d4 takes the largest difference's scale.
 #pragma once
 
 #include <cmath>
@@ -184,9 +184,58 @@ WZ_HD int64_t wide_unpack(double v, int& e) {
     return int64_t((m ^ join(sg, sg)) - join(sg, sg));
 }
 
-// f^ - c from the indicators b_k 2^(n_k) and the differences c_k 2^(E - 1082), |c_k| < 2^60.
-WZ_HD double wide_finish(uint64_t b0, uint64_t b1, uint64_t b2, int n0, int n1, int n2, int64_t c1, int64_t c2,
-                         int64_t c3, int64_t c4, int E, const WideConst& c) {
+WZ_HD int64_t shl_s64(int64_t x, int n) {            // 0 <= n < 64
+#ifdef __CUDA_ARCH__
+    int64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+    return r;
+#else
+    return int64_t(uint64_t(x) << n);
+#endif
+}
+
+// D 2^(G - 1082), |D| <= 2^60, as x 2^(e - 1082) with |x| in [2^59, 2^60]; e = 0 for D = 0.
+WZ_HD int64_t wide_normalise(int64_t D, int G, int& e) {
+    const uint32_t s = uint32_t(uint64_t(D >> 63)), h = uint32_t(uint64_t(D) >> 32) ^ s, l = uint32_t(D) ^ s;
+    const bool low = h == 0;
+    const int n = max_i(clz_u32((low ? l : h) | 1u) + (low ? 28 : -4), 0);
+    e = D == 0 ? 0 : G - n;
+    return shl_s64(D, n);
+}
+
+// f^ - c from the differences x_i 2^(e_i - 1082), |x_i| in [2^59, 2^60] (or x_i = 0, e_i = 0).
+WZ_HD double wide_correction(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e0, int e1, int e2, int e3,
+                             const WideConst& c) {
+    // the sub-stencils' pairs at their own scales
+    const int g01 = max_i(e0, e1), g12 = max_i(e1, e2), g23 = max_i(e2, e3);
+    const int E = max_i(g01, g23);
+    const int64_t p0 = shr_s64(x0, g01 - e0), q0 = shr_s64(x1, g01 - e1);
+    const int64_t p1 = shr_s64(x1, g12 - e1), q1 = shr_s64(x2, g12 - e2);
+    const int64_t p2 = shr_s64(x2, g23 - e2), q2 = shr_s64(x3, g23 - e3);
+
+    // the indicators; a pair below the scale of eps enters at that scale (b_k is then R to
+    // within rounding, and never loses its leading bits)
+    uint64_t b0, b1, b2;
+    int n0, n1, n2;                                           // exponents of b_k
+    {
+        int64_t u0 = p0, v0 = q0, u1 = p1, v1 = q1, u2 = p2, v2 = q2;
+        int h01 = g01, h12 = g12, h23 = g23;
+        if (g01 < c.e_min || g12 < c.e_min || g23 < c.e_min) {
+            h01 = max_i(g01, c.e_min);
+            h12 = max_i(g12, c.e_min);
+            h23 = max_i(g23, c.e_min);
+            u0 = shr_s64(u0, h01 - g01);
+            v0 = shr_s64(v0, h01 - g01);
+            u1 = shr_s64(u1, h12 - g12);
+            v1 = shr_s64(v1, h12 - g12);
+            u2 = shr_s64(u2, h23 - g23);
+            v2 = shr_s64(v2, h23 - g23);
+        }
+        b0 = wide_indicator(u0 - v0, v0, v0 + v0 - u0, h01, c, n0);
+        b1 = wide_indicator(u1 - v1, u1, v1, h12, c, n1);
+        b2 = wide_indicator(u2 - v2, u2, u2 + u2 - v2, h23, c, n2);
+    }
+
     // T = |b_0 - b_2| + R with the larger's exponent, h = min - R/2 with the smaller's
     const bool lt = n0 < n2 || (n0 == n2 && b0 < b2);
     const uint64_t mx = lt ? b2 : b0, mn = lt ? b0 : b2;
@@ -195,6 +244,7 @@ WZ_HD double wide_finish(uint64_t b0, uint64_t b1, uint64_t b2, int n0, int n1, 
     const uint64_t h = mn - shr_u64(c.RM, nn - c.eR + 1);
 
     // z = K |d4| T from normalised factors (both may have lost their leading bits); Y = z^2
+    const int64_t c1 = shr_s64(x0, E - e0), c2 = shr_s64(x1, E - e1), c3 = shr_s64(x2, E - e2), c4 = shr_s64(x3, E - e3);
     const int64_t d23 = c2 - c3;
     const int64_t d4 = (c1 - c4) - (d23 + d23 + d23);
     uint64_t ad = uint64_t(d4 < 0 ? -d4 : d4);
@@ -226,58 +276,49 @@ WZ_HD double wide_finish(uint64_t b0, uint64_t b1, uint64_t b2, int n0, int n1, 
     const uint64_t b01 = mul_hi(b0, b1), b12 = mul_hi(b1, b2), b02 = mul_hi(b0, b2);
     const uint64_t X = mul_hi(sqr_hi(h), mul_hi(b01, b2));
     const uint64_t Y0 = mul_hi(Y, b12), Y1 = mul_hi(Y, b02), Y2 = mul_hi(Y, b01);
-    // exponents relative to that of b_0 b_1 b_2: X = X 2^eX, Y_k = Y_k 2^(eY - n_k)
+    // exponents relative to that of b_0 b_1 b_2: X = X 2^eX, Y_k = Y_k 2^(eY - n_k); a_k = X + Y_k
+    // below 2^59 with the exponent of its larger term's leading bit (at most six zeros counted)
     const int eX = 2 * nn + 256, eY = 2 * ez + 192;
     const int f0 = eY - n0, f1 = eY - n1, f2 = eY - n2;
-    // the common exponent from the terms' own leading bits (at most six zeros are counted)
-    int ec = eX - leading_zeros6(X);
-    ec = max_i(ec, f0 - leading_zeros6(Y0));
-    ec = max_i(ec, f1 - leading_zeros6(Y1));
-    ec = max_i(ec, f2 - leading_zeros6(Y2)) + 6;
-    const uint64_t Xs = shr_u64(X, ec - eX);
-    // a_k below 2^59 (a common exponent), with the optimal weights 1 : 6 : 3
-    const uint64_t a0 = Xs + shr_u64(Y0, ec - f0);
-    const uint64_t a1 = (Xs + shr_u64(Y1, ec - f1)) * 6;
-    const uint64_t a2 = (Xs + shr_u64(Y2, ec - f2)) * 3;
+    const int tX = eX - leading_zeros6(X);
+    const int m0 = max_i(tX, f0 - leading_zeros6(Y0)) + 6;
+    const int m1 = max_i(tX, f1 - leading_zeros6(Y1)) + 6;
+    const int m2 = max_i(tX, f2 - leading_zeros6(Y2)) + 6;
+    // with the optimal weights 1 : 6 : 3
+    const uint64_t a0 = shr_u64(X, m0 - eX) + shr_u64(Y0, m0 - f0);
+    const uint64_t a1 = (shr_u64(X, m1 - eX) + shr_u64(Y1, m1 - f1)) * 6;
+    const uint64_t a2 = (shr_u64(X, m2 - eX) + shr_u64(Y2, m2 - f2)) * 3;
 
-    // numerator: sums of limb products, 96 bits kept (|A_h| < 2^30, |G_h| < 2^31)
-    const Limbs A0{int64_t(a0)}, A1{int64_t(a1)}, A2{int64_t(a2)};
-    const Limbs G0(c1 + c1 - 5 * c2), G1(c2 + c3 + c3), G2(c4 - 4 * c3);
-    const int64_t main = wide_mul(A0.h, G0.h) - wide_mul(A1.h, G1.h) + wide_mul(A2.h, G2.h);
-    const int64_t cr1 = wide_mul(A0.h, G0.l) - wide_mul(A1.h, G1.l) + wide_mul(A2.h, G2.l);
-    const int64_t cr2 = wide_mul(A0.l, G0.h) - wide_mul(A1.l, G1.h) + wide_mul(A2.l, G2.h);
-    const uint64_t lows = uint64_t(uint32_t(cr1)) + uint32_t(cr2);
-    int64_t top = main + (cr1 >> 32) + (cr2 >> 32) + int64_t(lows >> 32);
-    uint32_t low = uint32_t(lows);
-    const uint32_t sign = uint32_t(uint64_t(top) >> 32) & 0x80000000u;
-    if (top < 0) {                                            // magnitude of the 96-bit value
-        top = ~top;
-        low = ~low;
-    }
-    uint32_t th = uint32_t(uint64_t(top) >> 32), tm = uint32_t(top);
-    int en = E + 4;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const bool up = th == 0;
-        th = up ? tm : th;
-        tm = up ? low : tm;
-        low = up ? 0u : low;
-        en = up ? en - 32 : en;
-    }
-    const int nt = clz_u32(th | 1u);
-    const uint64_t N = join(funnel_l(tm, th, nt), funnel_l(low, tm, nt));
-
-    // denominator, reciprocal, quotient
-    uint64_t d = (a0 + a1 + a2) * 3;
+    // numerator: products a_k g_k / 2^62, |.| < 2^61.3, each with its own exponent, summed at the
+    // largest (g_k: |p|, |q| <= 2^60; limbs |A_h| < 2^30, |G_h| < 2^31)
+    auto product = [](uint64_t a, int64_t g) {
+        const Limbs A{int64_t(a)}, G(g);
+        const int64_t cross = wide_mul(A.h, G.l) + wide_mul(A.l, G.h);
+        const int64_t top = wide_mul(A.h, G.h) + (cross >> 32);
+        return int64_t(join(funnel_l(uint32_t(top), uint32_t(uint64_t(top) >> 32), 2),
+                            funnel_l(uint32_t(cross), uint32_t(top), 2)));
+    };
+    const int k0 = m0 + g01, k1 = m1 + g12, k2 = m2 + g23, km = max_i(max_i(k0, k1), k2);
+    const int64_t S = shr_s64(product(a0, p0 + p0 - 5 * q0), km - k0) - shr_s64(product(a1, p1 + q1 + q1), km - k1) +
+                      shr_s64(product(a2, q2 - 4 * p2), km - k2);
+    // denominator
+    const int dm = max_i(max_i(m0, m1), m2);
+    uint64_t d = (shr_u64(a0, dm - m0) + shr_u64(a1, dm - m1) + shr_u64(a2, dm - m2)) * 3;
     const int nd = clz_u32(uint32_t(d >> 32));
     d <<= nd;
-    uint64_t q = mul_hi(N, wide_rcp(d));
+    // |S|, normalised, times the reciprocal
+    const uint32_t sign = uint32_t(uint64_t(S) >> 32) & 0x80000000u;
+    uint64_t N = uint64_t(S < 0 ? -S : S);
+    const bool up = (N >> 32) == 0;
+    N = up ? N << 32 : N;
+    const int nt = clz_u32(uint32_t(N >> 32) | 1u);
+    uint64_t q = mul_hi(N << nt, wide_rcp(d));
     const int nq = clz_u32(uint32_t(q >> 32) | 1u);
     q <<= nq;
     // round to 53 bits; a carry out of the mantissa raises the exponent by itself
     const uint64_t r = ((q >> 10) + 1) >> 1;
-    const uint32_t ex = uint32_t(en - nt + nd - nq - 1) << 20;
-    const uint64_t bits = th == 0 ? 0 : r + join(ex | sign, 0);
+    const uint32_t ex = uint32_t(km - dm + 1 - nt - (up ? 32 : 0) + nd - nq) << 20;
+    const uint64_t bits = N == 0 ? 0 : r + join(ex | sign, 0);
 #ifdef __CUDA_ARCH__
     return __longlong_as_double((long long)bits);
 #else
@@ -287,78 +328,35 @@ WZ_HD double wide_finish(uint64_t b0, uint64_t b1, uint64_t b2, int n0, int n1, 
 #endif
 }
 
-// f^ - c from the first differences; false where the caller has to take the double evaluation
-// (a difference outside the range above, infinite or not a number).
+WZ_HD bool wide_in_range(int E, bool& zero) {      // of the largest exponent (0: all are zero)
+    zero = E == 0;
+    return unsigned(E - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp);
+}
+
+// The same from D_i 2^(G_i - 1082), |D_i| <= 2^60.  False where the caller has to take the double
+// evaluation (the largest difference outside the range above).
+WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4,
+                           const WideConst& c, double& corr) {
+    int e0, e1, e2, e3;
+    const int64_t x0 = wide_normalise(D1, G1, e0), x1 = wide_normalise(D2, G2, e1), x2 = wide_normalise(D3, G3, e2),
+                  x3 = wide_normalise(D4, G4, e3);
+    bool zero;
+    corr = 0.0;
+    if (!wide_in_range(max_i(max_i(e0, e1), max_i(e2, e3)), zero)) return zero;
+    corr = wide_correction(x0, x1, x2, x3, e0, e1, e2, e3, c);
+    return true;
+}
+
+// The same from the first differences as doubles (infinities and NaN return false).
 WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const WideConst& c, double& corr) {
     int e0, e1, e2, e3;
     const int64_t x0 = wide_unpack(D1, e0), x1 = wide_unpack(D2, e1), x2 = wide_unpack(D3, e2),
                   x3 = wide_unpack(D4, e3);
-    int e01 = max_i(e0, e1), e12 = max_i(e1, e2), e23 = max_i(e2, e3);
-    const int E = max_i(e01, e23);
+    bool zero;
     corr = 0.0;
-    if (unsigned(E - kWideMinExp) >= unsigned(kWideMaxExp - kWideMinExp)) return E == 0;
-    e01 = max_i(e01, c.e_min);
-    e12 = max_i(e12, c.e_min);
-    e23 = max_i(e23, c.e_min);
-    uint64_t b0, b1, b2;
-    int n0, n1, n2;                                           // exponents of b_k
-    {
-        const int64_t p = shr_s64(x0, e01 - e0), q = shr_s64(x1, e01 - e1);
-        b0 = wide_indicator(p - q, q, q + q - p, e01, c, n0);
-    }
-    {
-        const int64_t p = shr_s64(x1, e12 - e1), q = shr_s64(x2, e12 - e2);
-        b1 = wide_indicator(p - q, p, q, e12, c, n1);
-    }
-    {
-        const int64_t p = shr_s64(x2, e23 - e2), q = shr_s64(x3, e23 - e3);
-        b2 = wide_indicator(p - q, p, p + p - q, e23, c, n2);
-    }
-    corr = wide_finish(b0, b1, b2, n0, n1, n2, shr_s64(x0, E - e0), shr_s64(x1, E - e1), shr_s64(x2, E - e2),
-                       shr_s64(x3, E - e3), E, c);
+    if (!wide_in_range(max_i(max_i(e0, e1), max_i(e2, e3)), zero)) return zero;
+    corr = wide_correction(x0, x1, x2, x3, e0, e1, e2, e3, c);
     return true;
-}
-
-WZ_HD int64_t shl_s64(int64_t x, int n) {            // n >= 0, zero from 64 on
-#ifdef __CUDA_ARCH__
-    int64_t r;
-    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
-    return r;
-#else
-    return n > 63 ? 0 : int64_t(uint64_t(x) << n);
-#endif
-}
-
-// The exponent of the integer D in units 2^(G - 1082), |D| < 2^60, brought to [2^59, 2^60] (the
-// upper end for a negative power of two); 0 for D = 0.
-WZ_HD int wide_exponent(int64_t D, int G) {
-    const uint32_t s = uint32_t(uint64_t(D >> 63)), h = uint32_t(uint64_t(D) >> 32) ^ s, l = uint32_t(D) ^ s;
-    const bool low = h == 0;
-    const int n = clz_u32((low ? l : h) | 1u) + (low ? 28 : -4);
-    return D == 0 ? 0 : G - max_i(n, 0);
-}
-
-// f^ - c from integer differences D_k 2^(G - 1082), |D_k| < 2^60, G >= e_min unless all are zero.
-WZ_HD double wide_correction_int(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G, const WideConst& c) {
-    const int e0 = wide_exponent(D1, G), e1 = wide_exponent(D2, G), e2 = wide_exponent(D3, G),
-              e3 = wide_exponent(D4, G);
-    const int e01 = max_i(max_i(e0, e1), c.e_min), e12 = max_i(max_i(e1, e2), c.e_min),
-              e23 = max_i(max_i(e2, e3), c.e_min);
-    uint64_t b0, b1, b2;
-    int n0, n1, n2;
-    {
-        const int64_t p = shl_s64(D1, G - e01), q = shl_s64(D2, G - e01);
-        b0 = wide_indicator(p - q, q, q + q - p, e01, c, n0);
-    }
-    {
-        const int64_t p = shl_s64(D2, G - e12), q = shl_s64(D3, G - e12);
-        b1 = wide_indicator(p - q, p, q, e12, c, n1);
-    }
-    {
-        const int64_t p = shl_s64(D3, G - e23), q = shl_s64(D4, G - e23);
-        b2 = wide_indicator(p - q, p, p + p - q, e23, c, n2);
-    }
-    return wide_finish(b0, b1, b2, n0, n1, n2, D1, D2, D3, D4, G, c);
 }
 
 }  // namespace wz
