@@ -244,7 +244,7 @@ template <bool NEG = false>
 __device__ __forceinline__ double zn_flux_wide(double D1, double D2, double D3, double D4, double base,
                                                const WideConst& wc, double eps4, double kappa) {
     double corr;
-    if (!wide_correction(D1, D2, D3, D4, wc, corr)) corr = zn_correction_double(D1, D2, D3, D4, eps4, kappa);
+    if (!wide_correction(D1, D2, D3, D4, exponent_of(base), wc, corr)) corr = zn_correction_double(D1, D2, D3, D4, eps4, kappa);
     return NEG ? base - corr : base + corr;
 }
 

@@ -4,10 +4,11 @@
 // integer and FMA pipes one every 2: a 64 x 64-bit product of which only the top half is kept
 // is three 32 x 32 multiply-adds, an addition two instructions.  A reconstruction is 46 FP64
 // instructions (2,944 cycles of a sub-partition's FP64 unit) or about 325 ALU and 270
-// multiply-add ones, on pipes that otherwise idle.  Measured with the FP64 weights before and
-// these after: wenozn_reconstruct 1.24 -> 0.40 ms per side of 2^24 points (the ALU pipe 66 %
-// busy), the 2D Euler step 99.8 -> 40.7 ms at 4096^2 and 6.5 -> 2.8 ms at 1024^2, the 1D step
-// 2.63 -> 1.14 ms at 2^20 cells.
+// multiply-add ones, on pipes that otherwise idle; where the weights hardly differ from the
+// optimal ones (wide_linear) about 150 in all.  Measured with the FP64 weights before and these
+// after (with the integer projection of euler_device.cuh in the solver): wenozn_reconstruct
+// 1.24 -> 0.24 ms per side of 2^24 points, the 2D Euler step 99.9 -> 25.6 ms at 4096^2 and 6.5 ->
+// 1.85 ms at 1024^2, the 1D step 2.63 -> 0.66 ms at 2^20 cells.
 //
 // Precision.  Every quantity carries a 64-bit mantissa (block floating point: integers with a
 // common exponent), every truncation stays below that of a 53-bit one, so the result is
@@ -38,7 +39,7 @@
 #include <cstring>
 
 #ifdef __CUDACC__
-#define WZ_HD __host__ __device__ __forceinline__
+#define WZ_HD __device__ __forceinline__
 #else
 #define WZ_HD inline
 #endif
@@ -50,6 +51,7 @@ struct WideConst {
     uint64_t RM, KM;      // mantissas in [2^63, 2^64) of R = 3 eps and K = sqrt(3 / (4 A))
     int eR, eK;           // R = RM 2^(eR - 2164), K = KM 2^eK
     int e_min;            // smallest pair exponent: that of sqrt(eps)
+    float Rf, Kf;         // R = Rf 2^(eR - 2101), Rf in [1, 2); K
 };
 
 inline WideConst wide_const(double eps, double A) {
@@ -62,6 +64,8 @@ inline WideConst wide_const(double eps, double A) {
     w.KM = uint64_t(std::ldexp(k, 53)) << 11;
     w.eK = e - 64;
     w.e_min = (w.eR - 57) >> 1;
+    w.Rf = float(2.0 * r);
+    w.Kf = float(std::sqrt(0.75 / A));
     return w;
 }
 
@@ -204,8 +208,8 @@ WZ_HD int64_t wide_normalise(int64_t D, int G, int& e) {
 }
 
 // f^ - c from the differences x_i 2^(e_i - 1082), |x_i| in [2^59, 2^60] (or x_i = 0, e_i = 0).
-WZ_HD double wide_correction(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e0, int e1, int e2, int e3,
-                             const WideConst& c) {
+WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e0, int e1, int e2, int e3,
+                           const WideConst& c) {
     // the sub-stencils' pairs at their own scales
     const int g01 = max_i(e0, e1), g12 = max_i(e1, e2), g23 = max_i(e2, e3);
     const int E = max_i(g01, g23);
@@ -328,34 +332,225 @@ WZ_HD double wide_correction(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int
 #endif
 }
 
-WZ_HD bool wide_in_range(int E, bool& zero) {      // of the largest exponent (0: all are zero)
-    zero = E == 0;
-    return unsigned(E - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp);
+WZ_HD float bits_float(uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float f;
+    std::memcpy(&f, &b, 4);
+    return f;
+#endif
 }
 
-// The same from D_i 2^(G_i - 1082), |D_i| <= 2^60.  False where the caller has to take the double
-// evaluation (the largest difference outside the range above).
-WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4,
-                           const WideConst& c, double& corr) {
+WZ_HD uint32_t float_bits(float f) {
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(f);
+#else
+    uint32_t b;
+    std::memcpy(&b, &f, 4);
+    return b;
+#endif
+}
+
+WZ_HD int exponent_of(double v) {                    // biased
+#ifdef __CUDA_ARCH__
+    return (__double2hiint(v) >> 20) & 0x7ff;
+#else
+    uint64_t u;
+    std::memcpy(&u, &v, 8);
+    return int(u >> 52) & 0x7ff;
+#endif
+}
+
+WZ_HD float float_rcp(float x) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+WZ_HD float wide_float(int64_t x) {                  // x 2^-57 to 24 bits
+    const Limbs l(x);
+    return fmaf(float(l.h), 0x1p-25f, float(l.l) * 0x1p-57f);
+}
+
+WZ_HD uint64_t double_bits(double v) {
+#ifdef __CUDA_ARCH__
+    return uint64_t(__double_as_longlong(v));
+#else
+    uint64_t u;
+    std::memcpy(&u, &v, 8);
+    return u;
+#endif
+}
+
+WZ_HD double bits_double(uint64_t u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double v;
+    std::memcpy(&v, &u, 8);
+    return v;
+#endif
+}
+
+// x / 2 (exact) on the exponent field; by multiplication only where that underflows
+WZ_HD double wide_half(double x) {
+    const uint64_t u = double_bits(x);
+    const uint32_t e = uint32_t(u >> 52) & 0x7ffu;
+    if (e - 2u < 2045u) return bits_double(u - (uint64_t(1) << 52));
+    return (u << 1) == 0 ? x : 0.5 * x;
+}
+
+// 1 / x of a positive normal x below 2^1021, rounded to 53 bits from an error below 2^-60
+WZ_HD double wide_reciprocal(double x) {
+    const uint64_t u = double_bits(x);
+    const uint64_t r = wide_rcp((u << 11) | (uint64_t(1) << 63));
+    return bits_double((((r >> 10) + 1) >> 1) + (uint64_t(2044 - int(u >> 52)) << 52));
+}
+
+// 1 / sqrt(x) of a positive normal x: the float approximation Y0 of y = 1/sqrt(t), t in [1/4, 1)
+// the mantissa with an even exponent, and one step of y = y0 (1 + h/2 + 3/8 h^2 + ...),
+// h = 1 - t y0^2 < 2^-19 in units of 2^-62, so the truncated terms are below 2^-59 and the result
+// is within 2^-59 before its rounding to 53 bits.  Where x is not positive and normal: ok = false.
+WZ_HD double wide_rsqrt(double x, bool& ok) {
+    const uint64_t u = double_bits(x);
+    const int e = int(u >> 52);                                // the sign included
+    ok = unsigned(e - 1) < 2046u;
+    const uint64_t m = ((u << 11) | (uint64_t(1) << 63)) >> ((e & 1) ? 1 : 0);   // t = m / 2^64
+#ifdef __CUDA_ARCH__
+    float f;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rz(uint32_t(m >> 32))));
+    const uint32_t y0 = __float2uint_rz(f * 140737421246464.0f);         // 2^47 (1 - 2^-21)
+#else
+    const uint32_t y0 = uint32_t((1.0f / std::sqrt(float(uint32_t(m >> 32)))) * 140737421246464.0f);
+#endif
+    const uint64_t hh = (uint64_t(1) << 62) - mul_hi(m, uint64_t(y0) * y0);
+    const uint64_t h = hh > 2 ? hh - 2 : 0;
+    const uint32_t hs = uint32_t(h >> 12);
+    const uint64_t q = h + ((uint64_t(uint32_t((uint64_t(hs) * hs) >> 32)) * 3) >> 8);
+    const uint64_t y = (uint64_t(y0) << 32) + ((uint64_t(y0) * uint32_t(q)) >> 31) + ((uint64_t(y0) * uint32_t(q >> 32)) << 1);
+    // x = t 2^(e - 1022) with e odd after the shift's adjustment: y 2^((1022 - e') / 2)
+    const int ee = e + (e & 1);                                // even exponent field of t
+    return bits_double((((y >> 10) + 1) >> 1) + (uint64_t(1022 - ((ee - 1022) >> 1)) << 52));
+}
+
+// f^ - c where the weights hardly differ from the optimal ones; false where that is not shown.
+// With r_k = (K d4 T)^2 / (h^2 b_k) the weights are c_k (1 + r_k), so f^ - c is the optimal
+// linear combination of the differences, formed exactly in integers, plus
+//   sum c_k r_k (g_k - lin) / (1 + sum c_k r_k),
+// a combination of the second differences delta_0 = D1 - 2 D2 + D3 and delta_1 = D2 - 2 D3 + D4.
+// This part is evaluated in float from integers (each converted with 24 bits of its own: T is
+// formed from the delta's, without the cancellation in b_0 - b_2), and accepted only where the
+// bound on its error, from the bound ET on T's, is below 2^-56 of the differences and the value
+// they are added to: a quarter of a last place of the result.  Smooth data resolved by some 30
+// cells a wave are accepted (r falls like the twelfth power of the spacing), as are constant
+// data and differences at the rounding level of the value itself.  2^(eb - 1023) bounds that
+// value from below (eb <= 0: nothing is known of it).
+// About 150 instructions instead of 600 for a warp whose lanes are all accepted.
+WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
+                       const WideConst& c, double& corr) {
+    const int G = max_i(max_i(G1, G2), max_i(G3, G4));
+    const int64_t c1 = shr_s64(D1, G - G1 + 3), c2 = shr_s64(D2, G - G2 + 3);      // |c_i| <= 2^57
+    const int64_t c3 = shr_s64(D3, G - G3 + 3), c4 = shr_s64(D4, G - G4 + 3);
+    const int64_t s0 = c1 - c2, s1 = c2 - c3, s2 = c3 - c4, d0 = s0 - s1, d1 = s1 - s2;
+    const float f2 = wide_float(c2), f3 = wide_float(c3), S1 = wide_float(s1), E0 = wide_float(d0),
+                E1 = wide_float(d1), Q = wide_float(d0 - d1);
+    const float S0 = S1 + E0, S2 = S1 - E1;
+    const int er = c.eR - 57 - 2 * G;                         // R in the floats' units
+    const float R = c.Rf * bits_float(uint32_t((er < -126 ? -126 : (er > 60 ? 60 : er)) + 127) << 23);
+    const float be0 = fmaf(4.0f * S0, S0, 3.0f * f2 * (f2 - S0)), be2 = fmaf(4.0f * S2, S2, 3.0f * f3 * (f3 + S2));
+    const float be1 = fmaf(4.0f * S1, S1, 3.0f * f2 * f3);
+    const float b0 = be0 + R, b1 = be1 + R, b2 = be2 + R;
+    const float A = fabsf(E0) + fabsf(E1), M = fabsf(f2) + fabsf(S1) + A;
+    const float T = fabsf(fmaf(4.0f * (E0 + E1), S0 + S2, 3.0f * fmaf(f3, E1, -(f2 * E0)))) + R;
+    const float ET = 0x1p-18f * A * M;
+    const float u = c.Kf * Q * float_rcp(fminf(be0, be2) + 0.5f * R);
+    const float w = (u * T) * (u * T);
+    const float i0 = float_rcp(b0), i1 = float_rcp(b1), i2 = float_rcp(b2);
+    const float im = fmaxf(fmaxf(i0, i1), i2), rm = w * im;
+    const float err = fmaf(fabsf(u) * ET * im, fabsf(u) * fmaf(2.0f, T, ET), 0x1p-14f * rm);
+    const int ef = eb - G + 126;                              // 2^(eb - 1023) in the floats' units
+    const float fb = bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
+    if (!(A * err <= 0x1p-53f * (fabsf(f2) + fabsf(f3) + fb)) ||
+        unsigned(G - kWideMinExp) >= unsigned(kWideMaxExp - kWideMinExp))
+        return false;
+    // 60 (f^ - c) = lin + sum 10 c_k r_k (10 g_k - lin) / (10 + sum 10 c_k r_k)
+    const float r0 = w * i0, r1 = 6.0f * w * i1, r2 = 3.0f * w * i2;
+    const float num = fmaf(r0, fmaf(18.0f, E0, -3.0f * E1),
+                           fmaf(r1, fmaf(-2.0f, E0, -3.0f * E1), r2 * fmaf(-2.0f, E0, 7.0f * E1)));
+    const uint32_t v = float_bits(num * float_rcp(10.0f + (r0 + r1 + r2)));
+    const int ve = int((v >> 23) & 0xffu);
+    const int64_t vm = int64_t(shr_u64(join(((v & 0x7fffffu) | (ve ? 0x800000u : 0u)) << 6, 0), 131 - ve > 0 ? 131 - ve : 0));
+    const int64_t S = 2 * c1 - 11 * c2 - 24 * c3 + 3 * c4 + (int32_t(v) < 0 ? -vm : vm);
+    // S 2^(G - 1079) / 60 as a double
+    const uint32_t sign = uint32_t(uint64_t(S) >> 32) & 0x80000000u;
+    uint64_t N = uint64_t(S < 0 ? -S : S);
+    const bool up = (N >> 32) == 0;
+    N = up ? N << 32 : N;
+    const int nt = clz_u32(uint32_t(N >> 32) | 1u);
+    uint64_t q = mul_hi(N << nt, 9838263505978427528ull);     // 2^69 / 60
+    const int nq = clz_u32(uint32_t(q >> 32) | 1u);
+    q <<= nq;
+    const uint64_t r = ((q >> 10) + 1) >> 1;
+    const uint32_t ex = uint32_t(G + 1 - nt - (up ? 32 : 0) - nq) << 20;
+    const uint64_t bits = N == 0 ? 0 : r + join(ex | sign, 0);
+#ifdef __CUDA_ARCH__
+    corr = __longlong_as_double((long long)bits);
+#else
+    std::memcpy(&corr, &bits, 8);
+#endif
+    return true;
+}
+
+// The weighted evaluation as a call of its own: the warps of smooth data pass it by, and one copy
+// of its code serves every field (inlined four times it does not fit the instruction cache).
+#ifdef __CUDACC__
+static __device__ __noinline__
+#else
+inline
+#endif
+double wide_weighted_call(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, WideConst c) {
     int e0, e1, e2, e3;
     const int64_t x0 = wide_normalise(D1, G1, e0), x1 = wide_normalise(D2, G2, e1), x2 = wide_normalise(D3, G3, e2),
                   x3 = wide_normalise(D4, G4, e3);
-    bool zero;
+    return wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c);
+}
+
+// Whether the largest difference lies in the range of the integer evaluation (E its exponent).
+WZ_HD bool wide_in_range(int E) { return unsigned(E - kWideMinExp) < unsigned(kWideMaxExp - kWideMinExp); }
+
+// f^ - c from D_i 2^(G_i - 1082), |D_i| <= 2^60, to be added to a value of exponent eb.  False
+// where the caller has to take the double evaluation (the largest difference outside the range
+// above).
+WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
+                           const WideConst& c, double& corr) {
+    if (wide_linear(D1, D2, D3, D4, G1, G2, G3, G4, eb, c, corr)) return true;
     corr = 0.0;
-    if (!wide_in_range(max_i(max_i(e0, e1), max_i(e2, e3)), zero)) return zero;
-    corr = wide_correction(x0, x1, x2, x3, e0, e1, e2, e3, c);
+    int e0, e1, e2, e3;
+    wide_normalise(D1, G1, e0);
+    wide_normalise(D2, G2, e1);
+    wide_normalise(D3, G3, e2);
+    wide_normalise(D4, G4, e3);
+    const int E = max_i(max_i(e0, e1), max_i(e2, e3));
+    if (!wide_in_range(E)) return E == 0;
+    corr = wide_weighted_call(D1, D2, D3, D4, G1, G2, G3, G4, c);
     return true;
 }
 
 // The same from the first differences as doubles (infinities and NaN return false).
-WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, const WideConst& c, double& corr) {
+WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, int eb, const WideConst& c, double& corr) {
     int e0, e1, e2, e3;
     const int64_t x0 = wide_unpack(D1, e0), x1 = wide_unpack(D2, e1), x2 = wide_unpack(D3, e2),
                   x3 = wide_unpack(D4, e3);
-    bool zero;
+    const int E = max_i(max_i(e0, e1), max_i(e2, e3));
     corr = 0.0;
-    if (!wide_in_range(max_i(max_i(e0, e1), max_i(e2, e3)), zero)) return zero;
-    corr = wide_correction(x0, x1, x2, x3, e0, e1, e2, e3, c);
+    if (!wide_in_range(E)) return E == 0;
+    if (!wide_linear(x0, x1, x2, x3, e0, e1, e2, e3, eb, c, corr))
+        corr = wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c);
     return true;
 }
 

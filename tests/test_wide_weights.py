@@ -22,7 +22,8 @@ extern "C" long wide_line(const double* f, long n, int side, double eps, double 
         const double* s = f + j;
         double v[5], corr;
         for (int k = 0; k < 5; ++k) v[k] = side > 0 ? s[k] : s[5 - k];
-        if (!wz::wide_correction(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], c, corr)) ++refused, corr = 0.0;
+        if (!wz::wide_correction(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], wz::exponent_of(v[2]), c, corr))
+            ++refused, corr = 0.0;
         out[j] = v[2] + corr;
     }
     return refused;
