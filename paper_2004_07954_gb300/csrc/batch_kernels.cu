@@ -99,11 +99,11 @@ __global__ void __launch_bounds__(THREADS, 2) batch_stage_kernel(BatchArgs a) {
             split_cell<NV>(Uc, alpha, 0.0, gm1, sp, i);
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < cl_used - 1; i += THREADS) cell_diffs_wide<NV>(sp, i, 1);
+        for (int i = threadIdx.x; i < cl_used - 1; i += THREADS) cell_diffs<NV>(sp, i, 1);
         __syncthreads();
         for (int jl = threadIdx.x; jl <= ncell; jl += THREADS) {     // interfaces c0 .. c0+ncell
             double Fh[NV];
-            interface_flux<NV>(sp, jl, 1, gm1, a.wide, a.eps4, a.kappa, Fh);
+            interface_flux<NV, 0>(sp, jl, 1, gm1, a.wide, a.eps4, a.kappa, 0, 0, nullptr, Fh);
 #pragma unroll
             for (int k = 0; k < NV; ++k) sF[k * TI + jl] = Fh[k];
         }

@@ -10,25 +10,24 @@ namespace wz {
 
 // Shared-memory planes of one tile of NC cells: split fluxes h+ and h- (NV planes each),
 // and for the Euler systems sqrt(rho), u_n, H (and u_t in 2D), the differences
-// dh+-_c = h+-_c - h+-_{c+1} along the sweep (NV planes each; as doubles in the generic kernels,
-// as signed 64-bit mantissas with their exponents in the default ones) and, in the generic
-// kernels, the cell's |u_n| + c.
+// dh+-_c = h+-_c - h+-_{c+1} along the sweep (NV planes each, as signed 64-bit mantissas with
+// their exponents) and, in the generic kernels, the cell's |u_n| + c.
 template <int NV>
 struct CellPlanes {
     static constexpr int kPerCell = NV == 1 ? 2 : 2 * NV + (NV == 4 ? 4 : 3);
     // + dh+, dh- and four exponent words (two 16-bit exponents each)
     static constexpr int kPerCellDefault = kPerCell + (NV == 1 ? 0 : 2 * NV + 2);
-    static constexpr int kPerCellGeneric = kPerCell + (NV == 1 ? 0 : 2 * NV + 1);   // + dh+, dh-, |u_n| + c
+    static constexpr int kPerCellGeneric = kPerCellDefault + (NV == 1 ? 0 : 1);   // + |u_n| + c
     double* hp;
     double* hm;
     double* sr;
     double* un;
     double* H;
     double* ut;
-    double* dp;          // Euler: dh+ and dh- (mantissas: the same words as int64_t)
-    double* dm;
+    int64_t* dp;         // Euler: mantissas of dh+ and dh-
+    int64_t* dm;
+    uint32_t* ex;        // exponents of dh+ (0, 1), (2, 3) and dh- alike, a plane each
     double* sp;          // generic kernels: the cell's |u_n| + c (local LF)
-    uint32_t* ex;        // default kernels: exponents of dh+ (0, 1), (2, 3) and dh- alike, a plane each
     int NC;
     __device__ __forceinline__ CellPlanes(double* base, int nc) : NC(nc) {
         hp = base;
@@ -37,10 +36,10 @@ struct CellPlanes {
         un = sr + nc;
         H = un + nc;
         ut = H + nc;
-        dp = base + kPerCell * nc;
+        dp = reinterpret_cast<int64_t*>(base + kPerCell * nc);
         dm = dp + NV * nc;
-        sp = dm + NV * nc;
-        ex = reinterpret_cast<uint32_t*>(sp);
+        ex = reinterpret_cast<uint32_t*>(dm + NV * nc);
+        sp = base + kPerCellDefault * nc;
     }
 };
 
@@ -50,19 +49,9 @@ struct CellPlanes {
 template <int NV>
 __device__ __forceinline__ void cell_diffs(const CellPlanes<NV>& s, int si, int stride) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        s.dp[k * s.NC + si] = s.hp[k * s.NC + si] - s.hp[k * s.NC + si + stride];
-        s.dm[k * s.NC + si] = s.hm[k * s.NC + si] - s.hm[k * s.NC + si + stride];
-    }
-}
-
-// The same as mantissas and exponents for the integer projection.
-template <int NV>
-__device__ __forceinline__ void cell_diffs_wide(const CellPlanes<NV>& s, int si, int stride) {
-#pragma unroll
     for (int side = 0; side < 2; ++side) {
         const double* h = side == 0 ? s.hp : s.hm;
-        int64_t* d = reinterpret_cast<int64_t*>(side == 0 ? s.dp : s.dm);
+        int64_t* d = side == 0 ? s.dp : s.dm;
         int e[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int k = 0; k < NV; ++k)
@@ -78,6 +67,13 @@ __device__ __forceinline__ double inv_sqrt(double x) {
     bool ok;
     const double r = wide_rsqrt(x, ok);
     return ok ? r : rsqrt(x);
+}
+
+// sqrt(x) through it (one more rounding)
+__device__ __forceinline__ double square_root(double x) {
+    bool ok;
+    const double r = wide_rsqrt(x, ok);
+    return ok ? x * r : sqrt(x);
 }
 
 // One cell: Uc = (rho, m_n[, m_t], E) in the sweep direction's frame (or the scalar u with
@@ -143,49 +139,57 @@ __device__ __forceinline__ void split_cell_gen(const double* Uc, int split, doub
     }
     const double rho = Uc[0], mn = Uc[1], E = Uc[NV - 1];
     const double mt = NV == 4 ? Uc[2] : 0.0;
-    const double rs = rsqrt(rho);
+    const double rs = inv_sqrt(rho);
     const double rr = rs * rs;
     const double un = mn * rr;
     const double ut = mt * rr;
-    const double kin = NV == 4 ? 0.5 * fma(mn, un, mt * ut) : 0.5 * (mn * un);
+    const double kin = wide_half(NV == 4 ? fma(mn, un, mt * ut) : mn * un);
     const double p = gm1 * (E - kin);
     const double Ep = E + p;
     if (split == 3) {
-        const double c = sqrt(gamma * p * rr);
+        const double c = square_root(gamma * p * rr);
         const double l1 = un - c, l3 = un + c;
-        const double lp[3] = {0.5 * (l1 + fabs(l1)), 0.5 * (un + fabs(un)), 0.5 * (l3 + fabs(l3))};
-        const double lm[3] = {0.5 * (l1 - fabs(l1)), 0.5 * (un - fabs(un)), 0.5 * (l3 - fabs(l3))};
-        const double k0 = rho / (2.0 * gamma);
+        // (l + |l|)/2 and (l - |l|)/2: l or zero by its sign
+        const double l[3] = {l1, un, l3};
+        double lp[3], lm[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const bool neg = __double2hiint(l[i]) < 0;
+            lp[i] = neg ? 0.0 : l[i];
+            lm[i] = neg ? l[i] : 0.0;
+        }
+        const double k0 = rho * (1.0 / (2.0 * gamma));
         const double q2 = NV == 4 ? fma(un, un, ut * ut) : un * un;
         const double vv = NV == 4 ? ut * ut : 0.0;
-        const double e1 = 0.5 * fma(l1, l1, vv), e3 = 0.5 * fma(l3, l3, vv);     // ((u -+ c)^2 + v^2)/2
-        const double w13 = (3.0 - gamma) * c * c / (2.0 * gm1);
+        const double e1 = wide_half(fma(l1, l1, vv)), e3 = wide_half(fma(l3, l3, vv));     // ((u -+ c)^2 + v^2)/2
+        const double w13 = ((3.0 - gamma) / (2.0 * gm1)) * (c * c);
         const double g2 = 2.0 * gm1;
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
-            const double* l = side == 0 ? lp : lm;
+            const double* ls = side == 0 ? lp : lm;
             double* h = side == 0 ? s.hp : s.hm;
-            const double m0 = fma(g2, l[1], l[0] + l[2]);
+            const double s13 = ls[0] + ls[2];
+            const double m0 = fma(g2, ls[1], s13);
             h[si] = k0 * m0;
-            h[s.NC + si] = k0 * fma(g2 * l[1], un, fma(l[0], l1, l[2] * l3));
+            h[s.NC + si] = k0 * fma(g2 * ls[1], un, fma(ls[0], l1, ls[2] * l3));
             if (NV == 4) h[2 * s.NC + si] = k0 * (m0 * ut);
-            h[(NV - 1) * s.NC + si] = k0 * fma(gm1 * l[1], q2, fma(l[0], e1, fma(l[2], e3, (l[0] + l[2]) * w13)));
+            h[(NV - 1) * s.NC + si] = k0 * fma(gm1 * ls[1], q2, fma(ls[0], e1, fma(ls[2], e3, s13 * w13)));
         }
     } else {
-        const double hun = 0.5 * un;
+        const double hun = wide_half(un);
         double hF[NV];
-        hF[0] = 0.5 * mn;
-        hF[1] = fma(mn, hun, 0.5 * p);
+        hF[0] = wide_half(mn);
+        hF[1] = fma(mn, hun, wide_half(p));
         if (NV == 4) hF[2] = mt * hun;
         hF[NV - 1] = hun * Ep;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             s.hp[k * s.NC + si] = hF[k];
-            s.hm[k * s.NC + si] = 0.5 * Uc[k];
+            s.hm[k * s.NC + si] = wide_half(Uc[k]);
         }
         // local LF: the cell's |u_n| + c (the interface takes the largest of its six cells;
         // the per-field splitting reads global speeds instead)
-        if (split == 2) s.sp[si] = fabs(un) + sqrt(gamma * p * rr);
+        if (split == 2) s.sp[si] = fabs(un) + square_root(gamma * p * rr);
     }
     s.sr[si] = rho * rs;
     s.un[si] = un;
@@ -256,27 +260,37 @@ struct RoeState {
     }
 };
 
-// The fields' f^ - c (sum of both parts) in double arithmetic throughout, for stencils outside the range of
-// the integer projection.
-template <int NV>
+// The fields' f^ - c (sum of both parts) in double arithmetic throughout, for stencils outside the
+// range of the integer projection.  GEN 2: the planes hold F/2 and U/2, split per field with
+// the speeds ak.
+template <int NV, int GEN>
 __device__ __noinline__ void field_fluxes_double(const CellPlanes<NV>& s, const RoeState<NV>& R, int base,
-                                                 int stride, double eps4, double kappa, double* gh) {
+                                                 int stride, double eps4, double kappa, int weights,
+                                                 const double* ak, double* gh) {
     double D[2][4][NV];
 #pragma unroll 1
     for (int side = 0; side < 2; ++side)
 #pragma unroll 1
         for (int st = 0; st < 4; ++st) {
-            const double* h = side == 0 ? s.hp : s.hm;
             const int i = base + (side == 0 ? st : 4 - st) * stride;
-            double dh[NV];
+            double g[2][NV];
+#pragma unroll 1
+            for (int q = 0; q < 2; ++q) {
+                const double* h = q == 0 ? s.hp : s.hm;
+                double dh[NV];
 #pragma unroll
-            for (int k = 0; k < NV; ++k) dh[k] = h[k * s.NC + i] - h[k * s.NC + i + stride];
-            R.project(dh, D[side][st]);
+                for (int k = 0; k < NV; ++k) dh[k] = h[k * s.NC + i] - h[k * s.NC + i + stride];
+                R.project(dh, g[q]);
+            }
+#pragma unroll 1
+            for (int k = 0; k < NV; ++k)
+                D[side][st][k] = GEN == 2 ? (side == 0 ? fma(ak[k], g[1][k], g[0][k]) : fma(ak[k], g[1][k], -g[0][k]))
+                                          : (side == 0 ? g[0][k] : -g[1][k]);
         }
 #pragma unroll 1
     for (int k = 0; k < NV; ++k) {
-        const double fm = zn_flux_d(-D[1][0][k], -D[1][1][k], -D[1][2][k], -D[1][3][k], 0.0, eps4, kappa);
-        gh[k] = zn_flux_d(D[0][0][k], D[0][1][k], D[0][2][k], D[0][3][k], fm, eps4, kappa);
+        const double fm = zn_flux_w_d(D[1][0][k], D[1][1][k], D[1][2][k], D[1][3][k], 0.0, eps4, kappa, weights);
+        gh[k] = zn_flux_w_d(D[0][0][k], D[0][1][k], D[0][2][k], D[0][3][k], fm, eps4, kappa, weights);
     }
 }
 
@@ -351,42 +365,91 @@ struct WideProjection {
     }
 };
 
-template <int NV>
+// The interface flux.  GEN 0: WENO-ZN on the split fluxes of global Lax-Friedrichs; 1: any weight
+// function on the split fluxes the planes hold (global LF, Steger-Warming); 2: the planes
+// hold F/2 and U/2 and each field is split with its own speed after the projection,
+// g+-_c = l.F_c/2 +- a_k l.U_c/2, a_k = alpha_f[kind of field k] (split 1; kinds 0 u-c, 1 u, 2
+// u+c) or the largest |u_n| + c of the six cells (split 2).  The planes dh+- must be filled.
+template <int NV, int GEN>
 __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base, int stride, double gm1,
-                                               const WideConst& wc, double eps4, double kappa, double* Fh) {
+                                               const WideConst& wc, double eps4, double kappa, int weights, int split,
+                                               const double* alpha_f, double* Fh) {
+    constexpr int W = GEN == 0 ? 0 : -1;
     if (NV == 1) {
-        Fh[0] = zn_split_flux(s.hp[base], s.hp[base + stride], s.hp[base + 2 * stride],
-                              s.hp[base + 3 * stride], s.hp[base + 4 * stride],
-                              s.hm[base + stride], s.hm[base + 2 * stride], s.hm[base + 3 * stride],
-                              s.hm[base + 4 * stride], s.hm[base + 5 * stride], wc, eps4, kappa);
+        Fh[0] = zn_split_flux<W>(s.hp[base], s.hp[base + stride], s.hp[base + 2 * stride],
+                                 s.hp[base + 3 * stride], s.hp[base + 4 * stride],
+                                 s.hm[base + stride], s.hm[base + 2 * stride], s.hm[base + 3 * stride],
+                                 s.hm[base + 4 * stride], s.hm[base + 5 * stride], wc, eps4, kappa,
+                                 GEN == 0 ? 0 : weights);
         return;
     }
     const int NC = s.NC, cl = base + 2 * stride;
     const RoeState<NV> R(s, cl, cl + stride, gm1);
+    double ak[NV];
+    int64_t xk[NV];
+    int ek[NV];
+    int ebl = 0;
+    if (GEN == 2) {
+        if (split == 2) {
+            // (non-negative doubles order like their bit patterns)
+            long long m = __double_as_longlong(s.sp[base]);
+#pragma unroll
+            for (int st = 1; st < 6; ++st) m = max(m, __double_as_longlong(s.sp[base + st * stride]));
+#pragma unroll
+            for (int k = 0; k < NV; ++k) ak[k] = __longlong_as_double(m);
+        } else {
+            ak[0] = alpha_f[0];
+            ak[1] = alpha_f[1];
+            if (NV == 4) ak[2] = alpha_f[1];
+            ak[NV - 1] = alpha_f[2];
+        }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) xk[k] = wide_unpack(ak[k], ek[k]);
+        ebl = exponent_of(s.hm[cl]) + ek[0] - 1024;            // |a U/2|, U the density
+    }
     // scales of the fields' values (the centre's terms), below which an error does not count:
-    // h+_0 > c rho / 2 for the fields of the density's dimension
-    const int eb0 = exponent_of(s.hp[cl]);
+    // for the fields of the density's dimension h+-_0 (h+_0 > c rho / 2 for Lax-Friedrichs)
+    const int eb0 = GEN == 0 ? exponent_of(s.hp[cl]) : max_i(max_i(exponent_of(s.hp[cl]), ebl),
+                                                             GEN == 1 ? exponent_of(s.hm[cl + stride]) : 0);
     const int ebw = NV == 4 ? max_i(exponent_of(s.hp[2 * NC + cl]), exponent_of(R.v) + eb0 - 1024) : 0;
     double gh[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) gh[k] = 0.0;
-    const WideProjection<NV> W(R);
+    const WideProjection<NV> P(R);
     uint32_t xm = 0;
     bool ok = true;
 #pragma unroll 1
     for (int side = 0; side < 2; ++side) {
         int64_t D[4][NV];
         int G[4][NV];
-        const int64_t* pl = reinterpret_cast<const int64_t*>(side == 0 ? s.dp : s.dm);
         const int step = side == 0 ? stride : -stride;
+        const int first = side == 0 ? base : base + 4 * stride;
 #pragma unroll
-        for (int st = 0; st < 4; ++st)
-            W.apply(pl, s.ex + 2 * side * NC, NC, (side == 0 ? base : base + 4 * stride) + st * step, D[st], G[st], xm);
+        for (int st = 0; st < 4; ++st) {
+            if (GEN != 2) {
+                P.apply(side == 0 ? s.dp : s.dm, s.ex + 2 * side * NC, NC, first + st * step, D[st], G[st], xm);
+            } else {
+                // plus side l.dF/2 + a_k l.dU/2, minus side its negative l.dF/2 - a_k l.dU/2
+                int64_t u[NV];
+                int gu[NV];
+                P.apply(s.dp, s.ex, NC, first + st * step, D[st], G[st], xm);
+                P.apply(s.dm, s.ex + 2 * NC, NC, first + st * step, u, gu, xm);
+#pragma unroll
+                for (int k = 0; k < NV; ++k) {
+                    const Limbs A(xk[k]), B(u[k]);
+                    const int64_t v = wide_mul(A.h, B.h) + ((wide_mul(A.h, B.l) + wide_mul(A.l, B.h)) >> 32);
+                    const int gv = gu[k] + ek[k] - 1018, g = max_i(gv, G[st][k]) + 1;
+                    const int64_t w = shr_s64(v, g - gv);
+                    D[st][k] = shr_s64(D[st][k], g - G[st][k]) + (side == 0 ? w : -w);
+                    G[st][k] = g;
+                }
+            }
+        }
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             double corr;
-            ok = wide_correction(D[0][k], D[1][k], D[2][k], D[3][k], G[0][k], G[1][k], G[2][k], G[3][k],
-                                 NV == 4 && k == 2 ? ebw : eb0 - 2, wc, corr) && ok;
+            ok = wide_correction<W>(D[0][k], D[1][k], D[2][k], D[3][k], G[0][k], G[1][k], G[2][k], G[3][k],
+                                    NV == 4 && k == 2 ? ebw : eb0 - 2, wc, weights, corr) && ok;
             gh[k] = side == 0 ? corr : gh[k] - corr;
         }
     }
@@ -394,150 +457,36 @@ __device__ __forceinline__ void interface_flux(const CellPlanes<NV>& s, int base
         // out of the integer evaluation's range, infinite or not a number (copies, so that the
         // kept values need no address)
         const RoeState<NV> Rc = R;
-        double gd[NV];
-        field_fluxes_double<NV>(s, Rc, base, stride, eps4, kappa, gd);
+        double gd[NV], ac[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) ac[k] = GEN == 2 ? ak[k] : 0.0;
+        field_fluxes_double<NV, GEN>(s, Rc, base, stride, eps4, kappa, GEN == 0 ? 0 : weights, ac, gd);
 #pragma unroll
         for (int k = 0; k < NV; ++k) gh[k] = gd[k];
     }
     double hc[NV];
+    if (GEN != 2) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) hc[k] = s.hp[k * NC + cl] + s.hm[k * NC + cl + stride];
-    R.back_project(gh, hc, Fh);
-}
-
-// The interface flux of the generic kernels: weights and splitting chosen at run time.
-// Splits 0 and 3 (DIFF) project the cell split fluxes h+- (their differences and centres);
-// splits 1 and 2 project F/2 and U/2 of the six cells (their differences and centres) and
-// split each field k with its speed alpha_k: g+- = l_k.(F/2) +- alpha_k l_k.(U/2),
-// alpha_k = alpha_f[kind of field k] (split 1; kinds 0 u-c, 1 u, 2 u+c) or the largest
-// |u_n| + c of the six cells (split 2).  The planes dh+- must be filled (cell_diffs).
-template <int NV, bool DIFF>
-__device__ __forceinline__ void interface_flux_gen(const CellPlanes<NV>& s, int base, int stride, double gm1,
-                                                   double eps4, double kappa, int weights, int split,
-                                                   const double* alpha_f, double* Fh) {
-    const int NC = s.NC;
-    if (NV == 1) {
-        const double p0 = s.hp[base], p1 = s.hp[base + stride], p2 = s.hp[base + 2 * stride];
-        const double p3 = s.hp[base + 3 * stride], p4 = s.hp[base + 4 * stride];
-        const double m0 = s.hm[base + stride], m1 = s.hm[base + 2 * stride], m2 = s.hm[base + 3 * stride];
-        const double m3 = s.hm[base + 4 * stride], m4 = s.hm[base + 5 * stride];
-        Fh[0] = zn_flux_w(p0, p1, p2, p3, p4, eps4, kappa, weights) +
-                zn_flux_w(m4, m3, m2, m1, m0, eps4, kappa, weights);
-        return;
-    }
-    const int cl = base + 2 * stride, cr = base + 3 * stride;
-    const double srl = s.sr[cl], srr = s.sr[cr];
-    const double rsum = rcp_nr(srl + srr);
-    const double wl = srl * rsum, wr = srr * rsum;
-    const double u = fma(wl, s.un[cl], wr * s.un[cr]);
-    const double v = NV == 4 ? fma(wl, s.ut[cl], wr * s.ut[cr]) : 0.0;
-    const double H = fma(wl, s.H[cl], wr * s.H[cr]);
-    const double q2 = NV == 4 ? fma(u, u, v * v) : u * u;
-    const double c2 = gm1 * fma(-0.5, q2, H);
-    const double rc = rsqrt(c2);
-    const double c = c2 * rc;
-    const double hrc = 0.5 * rc;
-    const double hq2 = 0.5 * q2;
-    const double hb1 = (0.5 * gm1) * (rc * rc);        // b1 / 2, b1 = (gamma - 1) / c^2
-    const double hb2 = hq2 * hb1;                      // b2 / 2, b2 = q^2 b1 / 2
-    // left eigenvectors through their shared parts, as in interface_flux
-    auto project = [&](const double* h, double* g) {
-        const double h0 = h[0], h1 = h[1], hE = h[NV - 1];
-        const double W = NV == 4 ? fma(u, h1, fma(v, h[2], -hE)) : fma(u, h1, -hE);
-        const double Zh = fma(hb2, h0, -(hb1 * W));          // Z / 2
-        const double Bi = fma(u, h0, -h1);                   // 2 c B
-        g[0] = fma(hrc, Bi, Zh);
-        g[1] = fma(-2.0, Zh, h0);
-        if (NV == 4) g[2] = fma(-v, h0, h[2]);
-        g[NV - 1] = fma(-hrc, Bi, Zh);
-    };
-    auto project_at = [&](const double* planes, int i, double* g) {
-        double h[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) h[k] = planes[k * NC + i];
-        project(h, g);
-    };
-    double gh[NV];
-    if (DIFF) {
-        // splits 0 and 3, split fluxes per cell: the stencil differences and both centre
-        // values projected as in interface_flux (the planes dh+- filled by cell_diffs)
-        double Dp[4][NV], Dm[4][NV], C[NV];
-#pragma unroll
-        for (int st = 0; st < 4; ++st) {
-            project_at(s.dp, base + st * stride, Dp[st]);
-            project_at(s.dm, base + (st + 1) * stride, Dm[st]);
-        }
-        double hc[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) hc[k] = s.hp[k * NC + base + 2 * stride] + s.hm[k * NC + base + 3 * stride];
-        project(hc, C);
+        for (int k = 0; k < NV; ++k) hc[k] = s.hp[k * NC + cl] + s.hm[k * NC + cl + stride];
+    } else {
+        // the centres (F_2 + F_3)/2 + R diag(a_k) L (U_2 - U_3)/2
+        double du[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const double fm = zn_flux_w_d(-Dm[3][k], -Dm[2][k], -Dm[1][k], -Dm[0][k], C[k], eps4, kappa, weights);
-            gh[k] = zn_flux_w_d(Dp[0][k], Dp[1][k], Dp[2][k], Dp[3][k], fm, eps4, kappa, weights);
+            hc[k] = s.hp[k * NC + cl] + s.hp[k * NC + cl + stride];
+            du[k] = s.hm[k * NC + cl] - s.hm[k * NC + cl + stride];
         }
-    } else {
-        // splits 1 and 2: hp = F/2 and hm = U/2 per cell, each field split with its speed after
-        // the projection, g+-_c = l.F_c/2 +- a_k l.U_c/2; differences g+-_c - g+-_{c+1} =
-        // l.dF_c/2 +- a_k l.dU_c/2 (dh+- of cells 0..4), both centres at once as
-        // l.(F_2 + F_3)/2 + a_k l.(U_2 - U_3)/2
-        double ak[NV];
         if (split == 2) {
-            double a = s.sp[base];
 #pragma unroll
-            for (int st = 1; st < 6; ++st) a = fmax(a, s.sp[base + st * stride]);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) ak[k] = a;
+            for (int k = 0; k < NV; ++k) hc[k] = fma(ak[k], du[k], hc[k]);
         } else {
-            ak[0] = alpha_f[0];
-            ak[1] = alpha_f[1];
-            if (NV == 4) ak[2] = alpha_f[1];
-            ak[NV - 1] = alpha_f[2];
-        }
-        // plus side D_s = g+_{s-1} - g+_s (cells 0..3 of dh), minus side the mirrored
-        // D_s = -(g-_{5-s} - g-_{6-s}) (cells 4..1), combined as each point is projected
-        double Dp[4][NV], Dm[4][NV], cF[NV], cU[NV];
+            double gu[NV];
+            R.project(du, gu);
 #pragma unroll
-        for (int st = 0; st < 5; ++st) {
-            double gF[NV], gU[NV];
-            project_at(s.dp, base + st * stride, gF);
-            project_at(s.dm, base + st * stride, gU);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                if (st <= 3) Dp[st][k] = fma(ak[k], gU[k], gF[k]);
-                if (st >= 1) Dm[st - 1][k] = fma(ak[k], gU[k], -gF[k]);
-            }
-        }
-        {
-            double hf[NV], hu[NV];
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                hf[k] = s.hp[k * NC + base + 2 * stride] + s.hp[k * NC + base + 3 * stride];
-                hu[k] = s.hm[k * NC + base + 2 * stride] - s.hm[k * NC + base + 3 * stride];
-            }
-            project(hf, cF);
-            project(hu, cU);
-        }
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            const double C = fma(ak[k], cU[k], cF[k]);
-            const double fm = zn_flux_w_d(Dm[3][k], Dm[2][k], Dm[1][k], Dm[0][k], C, eps4, kappa, weights);
-            gh[k] = zn_flux_w_d(Dp[0][k], Dp[1][k], Dp[2][k], Dp[3][k], fm, eps4, kappa, weights);
+            for (int k = 0; k < NV; ++k) gh[k] = fma(ak[k], gu[k], gh[k]);
         }
     }
-    const double uc = u * c;
-    if (NV == 3) {
-        const double d20 = gh[2] - gh[0];
-        Fh[0] = gh[0] + gh[1] + gh[2];
-        Fh[1] = fma(u, Fh[0], c * d20);
-        Fh[2] = fma(H, gh[0] + gh[2], fma(uc, d20, hq2 * gh[1]));
-    } else {
-        const double d30 = gh[3] - gh[0];
-        Fh[0] = gh[0] + gh[1] + gh[3];
-        Fh[1] = fma(u, Fh[0], c * d30);
-        Fh[2] = fma(v, Fh[0], gh[2]);
-        Fh[3] = fma(H, gh[0] + gh[3], fma(uc, d30, fma(hq2, gh[1], v * gh[2])));
-    }
+    R.back_project(gh, hc, Fh);
 }
 
 }  // namespace wz

@@ -33,7 +33,9 @@ namespace {
 // Long 1D lines use 251-interface tiles (256 cells with the halo: one full round of the cell
 // and difference passes; a 2^20-cell step 0.70 ms, with three blocks 0.73, with two 0.83 ms);
 // short ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
-// every SM gets work.
+// every SM gets work.  GEN = 2 projects F and U (twice the difference vectors a thread) and runs
+// best with two blocks and 128 registers (a 640 x 777 local-LF step 1.76 ms; three blocks 1.81,
+// four 1.85 ms).
 template <int NV, bool SMALL = false> struct Tile { static constexpr int TI = 251, TA = 1, THREADS = 256, BLOCKS = 4; };
 template <int NV> struct Tile<NV, true> { static constexpr int TI = 64, TA = 1, THREADS = 64, BLOCKS = 2; };
 template <> struct Tile<4, false> { static constexpr int TI = 32, TA = 8, THREADS = 256, BLOCKS = 4; };
@@ -92,8 +94,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
         // the split-flux differences of neighbouring cells along the sweep
         for (int idx = threadIdx.x; idx < NC; idx += kThreads) {
             if (idx / TA >= cl_used - 1) break;
-            if (GEN != 0) cell_diffs<NV>(sp, idx, kStride);
-            else cell_diffs_wide<NV>(sp, idx, kStride);
+            cell_diffs<NV>(sp, idx, kStride);
         }
         __syncthreads();
     }
@@ -104,10 +105,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
         const int j = j0 + idx / TA, line = l0 + idx % TA;
         if (j >= nint || line >= nlines) continue;
         double Fh[NV];
-        if (GEN != 0)
-            interface_flux_gen<NV, GEN == 1>(sp, idx, kStride, gm1, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
-        else
-            interface_flux<NV>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, Fh);
+        interface_flux<NV, GEN>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
         // store, undoing the direction frame
         const int64_t base = x ? int64_t(line) * (a.nx + 1) + j : int64_t(j) * a.nx + line;
         const int64_t plane = x ? int64_t(a.ny) * (a.nx + 1) : int64_t(a.ny + 1) * a.nx;
@@ -121,7 +119,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
 }
 
 template <int NV, int DIR, bool SMALL, int GEN>
-__global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, GEN == 0 ? Tile<NV, SMALL>::BLOCKS : 2)
+__global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, SMALL || GEN == 2 ? 2 : Tile<NV, SMALL>::BLOCKS)
     flux_kernel(FluxArgs a) {
     extern __shared__ double smem[];
     pdl_wait();
@@ -133,7 +131,7 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, GEN == 0 ? Tile<NV, 
 // the x tiles (along the sweep fastest, as flux_kernel<4, 0>), the others the y tiles
 // (across the sweep fastest, as flux_kernel<4, 1>).
 template <int GEN>
-__global__ void __launch_bounds__(Tile<4>::THREADS, GEN == 0 ? Tile<4>::BLOCKS : 2)
+__global__ void __launch_bounds__(Tile<4>::THREADS, GEN == 2 ? 2 : Tile<4>::BLOCKS)
     flux_xy_kernel(FluxArgs ax, double* Fy, int bc_y, int x_along, int nbx, int y_across) {
     extern __shared__ double smem[];
     pdl_wait();

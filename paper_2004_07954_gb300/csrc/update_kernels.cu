@@ -265,18 +265,19 @@ __global__ void __launch_bounds__(kThreads) reconstruct_zn_kernel(const double* 
     const int64_t j = j0 + tid;
     if (j > n) return;
     const int i = tid;
-    if (side > 0) fhat[j] = zn_flux_wide(sD[i], sD[i + 1], sD[i + 2], sD[i + 3], sf[i + 2], wc, eps4, kappa);
-    else fhat[j] = zn_flux_wide<true>(sD[i + 4], sD[i + 3], sD[i + 2], sD[i + 1], sf[i + 3], wc, eps4, kappa);
+    if (side > 0) fhat[j] = zn_flux_wide<0>(sD[i], sD[i + 1], sD[i + 2], sD[i + 3], sf[i + 2], wc, eps4, kappa);
+    else fhat[j] = zn_flux_wide<0, true>(sD[i + 4], sD[i + 3], sD[i + 2], sD[i + 1], sf[i + 3], wc, eps4, kappa);
 }
 
 __global__ void __launch_bounds__(kThreads) reconstruct_kernel(const double* f, int64_t n, double* fhat,
-                                                                int side, double eps4, double kappa,
+                                                                int side, WideConst wc, double eps4, double kappa,
                                                                 int weights) {
     const int64_t j = blockIdx.x * int64_t(kThreads) + threadIdx.x;
     if (j > n) return;
-    const double* s = f + j;
-    fhat[j] = side > 0 ? zn_flux_w(s[0], s[1], s[2], s[3], s[4], eps4, kappa, weights)
-                       : zn_flux_w(s[5], s[4], s[3], s[2], s[1], eps4, kappa, weights);
+    double v[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] = f[j + (side > 0 ? k : 5 - k)];
+    fhat[j] = zn_flux_wide<-1>(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], v[2], wc, eps4, kappa, weights);
 }
 
 // x-ghosts of the interior rows (phase 0) or y-ghosts of every padded column (phase 1).
@@ -391,7 +392,8 @@ cudaError_t launch_reconstruct(const double* f_padded, int64_t n, double* fhat, 
         reconstruct_zn_kernel<<<grid, kThreads, 0, s>>>(f_padded, n, fhat, side, wide_const(eps, A), 4.0 * eps,
                                                          zn_kappa(A));
     else
-        reconstruct_kernel<<<grid, kThreads, 0, s>>>(f_padded, n, fhat, side, 4.0 * eps, zn_kappa(A), weights);
+        reconstruct_kernel<<<grid, kThreads, 0, s>>>(f_padded, n, fhat, side, wide_const(eps, A), 4.0 * eps,
+                                                      zn_kappa(A), weights);
     return cudaGetLastError();
 }
 

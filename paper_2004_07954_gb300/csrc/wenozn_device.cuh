@@ -232,32 +232,6 @@ __host__ __device__ __forceinline__ double zn_flux_d(double D1, double D2, doubl
     return fma(num, rcp_nr(den), base);
 }
 
-// f^ - c in double arithmetic, for the stencils the integer evaluation does not take.
-[[maybe_unused]] static __device__ __noinline__ double zn_correction_double(double D1, double D2, double D3, double D4, double eps4,
-                                                    double kappa) {
-    return zn_flux_d(D1, D2, D3, D4, 0.0, eps4, kappa);
-}
-
-// base + (f^ - c) of the differences D1..D4, or base - (f^ - c) (NEG: the value for the
-// negated differences, in which f^ - c is odd), in integer arithmetic (wide_weights.cuh).
-template <bool NEG = false>
-__device__ __forceinline__ double zn_flux_wide(double D1, double D2, double D3, double D4, double base,
-                                               const WideConst& wc, double eps4, double kappa) {
-    double corr;
-    if (!wide_correction(D1, D2, D3, D4, exponent_of(base), wc, corr)) corr = zn_correction_double(D1, D2, D3, D4, eps4, kappa);
-    return NEG ? base - corr : base + corr;
-}
-
-// f^+ + f^- at one interface: plus side from (p0..p4) = h+_{i-2..i+2}, minus side from the
-// mirrored stencil (m4, m3, m2, m1, m0) where (m0..m4) = h-_{i-1..i+3} (Sec. 2, the
-// "symmetric rule about x_{i+1/2}").
-__device__ __forceinline__ double zn_split_flux(double p0, double p1, double p2, double p3, double p4,
-                                                double m0, double m1, double m2, double m3, double m4,
-                                                const WideConst& wc, double eps4, double kappa) {
-    return zn_flux_wide(p0 - p1, p1 - p2, p2 - p3, p3 - p4, p2, wc, eps4, kappa) +
-           zn_flux_wide(m4 - m3, m3 - m2, m2 - m1, m1 - m0, m2, wc, eps4, kappa);
-}
-
 // zn_flux_d with the weight function chosen at run time
 __host__ __device__ __forceinline__ double zn_flux_w_d(double D1, double D2, double D3, double D4, double base,
                                                        double eps4, double kappa, int weights) {
@@ -268,9 +242,33 @@ __host__ __device__ __forceinline__ double zn_flux_w_d(double D1, double D2, dou
     return fma(num, rcp_nr(den), base);
 }
 
-__host__ __device__ __forceinline__ double zn_flux_w(double a, double b, double c, double d, double e,
-                                                     double eps4, double kappa, int weights) {
-    return zn_flux_w_d(a - b, b - c, c - d, d - e, c, eps4, kappa, weights);
+// f^ - c in double arithmetic, for the stencils the integer evaluation does not take.
+[[maybe_unused]] static __device__ __noinline__ double zn_correction_double(double D1, double D2, double D3, double D4,
+                                                                            double eps4, double kappa, int weights) {
+    return zn_flux_w_d(D1, D2, D3, D4, 0.0, eps4, kappa, weights);
+}
+
+// base + (f^ - c) of the differences D1..D4, or base - (f^ - c) (NEG: the value for the
+// negated differences, in which f^ - c is odd), in integer arithmetic (wide_weights.cuh).  W:
+// the weight function, -1 for the run-time value.
+template <int W, bool NEG = false>
+__device__ __forceinline__ double zn_flux_wide(double D1, double D2, double D3, double D4, double base,
+                                               const WideConst& wc, double eps4, double kappa, int weights = W) {
+    double corr;
+    if (!wide_correction<W>(D1, D2, D3, D4, exponent_of(base), wc, weights, corr))
+        corr = zn_correction_double(D1, D2, D3, D4, eps4, kappa, weights);
+    return NEG ? base - corr : base + corr;
+}
+
+// f^+ + f^- at one interface: plus side from (p0..p4) = h+_{i-2..i+2}, minus side from the
+// mirrored stencil (m4, m3, m2, m1, m0) where (m0..m4) = h-_{i-1..i+3} (Sec. 2, the
+// "symmetric rule about x_{i+1/2}").
+template <int W>
+__device__ __forceinline__ double zn_split_flux(double p0, double p1, double p2, double p3, double p4,
+                                                double m0, double m1, double m2, double m3, double m4,
+                                                const WideConst& wc, double eps4, double kappa, int weights = W) {
+    return zn_flux_wide<W>(p0 - p1, p1 - p2, p2 - p3, p3 - p4, p2, wc, eps4, kappa, weights) +
+           zn_flux_wide<W>(m4 - m3, m3 - m2, m2 - m1, m1 - m0, m2, wc, eps4, kappa, weights);
 }
 
 // ------------------------------------------------------------------------------------

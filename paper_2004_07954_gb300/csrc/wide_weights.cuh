@@ -208,8 +208,10 @@ WZ_HD int64_t wide_normalise(int64_t D, int G, int& e) {
 }
 
 // f^ - c from the differences x_i 2^(e_i - 1082), |x_i| in [2^59, 2^60] (or x_i = 0, e_i = 0).
+// weights: 0 WENO-ZN, as above; 1 WENO-Z (q = 1), a_k = b_0 b_1 b_2 + |b_0 - b_2| b_i b_j; 3
+// Jiang-Shu, a_k = (b_i b_j)^2 (the linear weights, 2, are wide_linear's).
 WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e0, int e1, int e2, int e3,
-                           const WideConst& c) {
+                           const WideConst& c, int weights) {
     // the sub-stencils' pairs at their own scales
     const int g01 = max_i(e0, e1), g12 = max_i(e1, e2), g23 = max_i(e2, e3);
     const int E = max_i(g01, g23);
@@ -240,50 +242,69 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
         b2 = wide_indicator(u2 - v2, u2, u2 + u2 - v2, h23, c, n2);
     }
 
-    // T = |b_0 - b_2| + R with the larger's exponent, h = min - R/2 with the smaller's
-    const bool lt = n0 < n2 || (n0 == n2 && b0 < b2);
-    const uint64_t mx = lt ? b2 : b0, mn = lt ? b0 : b2;
-    const int nx = lt ? n2 : n0, nn = lt ? n0 : n2;
-    uint64_t T = mx - shr_u64(mn, nx - nn) + shr_u64(c.RM, nx - c.eR);
-    const uint64_t h = mn - shr_u64(c.RM, nn - c.eR + 1);
-
-    // z = K |d4| T from normalised factors (both may have lost their leading bits); Y = z^2
-    const int64_t c1 = shr_s64(x0, E - e0), c2 = shr_s64(x1, E - e1), c3 = shr_s64(x2, E - e2), c4 = shr_s64(x3, E - e3);
-    const int64_t d23 = c2 - c3;
-    const int64_t d4 = (c1 - c4) - (d23 + d23 + d23);
-    uint64_t ad = uint64_t(d4 < 0 ? -d4 : d4);
-    int ez = E + nx + c.eK + 128;
-    {
-        const bool low = (ad >> 32) == 0;
-        ad = low ? ad << 32 : ad;
-        const int n = clz_u32(uint32_t(ad >> 32) | 1u);
-        ad <<= n;
-        ez -= n + (low ? 32 : 0);
-    }
-    {
+    // a_k = X 2^eX + Y_k 2^(f_k), exponents relative to that of b_0 b_1 b_2
+    const uint64_t b01 = mul_hi(b0, b1), b12 = mul_hi(b1, b2), b02 = mul_hi(b0, b2);
+    uint64_t X = 0, Y0, Y1, Y2;
+    int eX = -(1 << 20), f0, f1, f2;
+    if (weights == 3) {
+        Y0 = sqr_hi(b12);
+        Y1 = sqr_hi(b02);
+        Y2 = sqr_hi(b01);
+        const int eS = n0 + n1 + n2 + 192;
+        f0 = eS - 2 * n0;
+        f1 = eS - 2 * n1;
+        f2 = eS - 2 * n2;
+    } else {
+        // T = |b_0 - b_2| (+ R) with the larger's exponent, normalised
+        const bool lt = n0 < n2 || (n0 == n2 && b0 < b2);
+        const uint64_t mx = lt ? b2 : b0, mn = lt ? b0 : b2;
+        const int nx = lt ? n2 : n0, nn = lt ? n0 : n2;
+        uint64_t T = mx - shr_u64(mn, nx - nn) + (weights == 0 ? shr_u64(c.RM, nx - c.eR) : 0);
+        int eT = nx;
         if ((T >> 32) == 0) {
             T <<= 32;
-            ez -= 32;
+            eT -= 32;
         }
-        const int n = clz_u32(uint32_t(T >> 32) | 1u);
-        T <<= n;
-        ez -= n;
+        const int nT = clz_u32(uint32_t(T >> 32) | 1u);
+        T <<= nT;
+        eT -= nT;
+        uint64_t Y;
+        int eY;
+        if (weights == 1) {
+            X = mul_hi(b01, b2);
+            eX = 128;
+            Y = T;
+            eY = T == 0 ? -(1 << 20) : eT + 128;
+        } else {
+            // z = K |d4| T from normalised factors (both may have lost their leading bits);
+            // X = h^2 b_0 b_1 b_2 with h = min - R/2, Y = z^2
+            const int64_t c1 = shr_s64(x0, E - e0), c2 = shr_s64(x1, E - e1), c3 = shr_s64(x2, E - e2),
+                          c4 = shr_s64(x3, E - e3);
+            const int64_t d23 = c2 - c3;
+            const int64_t d4 = (c1 - c4) - (d23 + d23 + d23);
+            uint64_t ad = uint64_t(d4 < 0 ? -d4 : d4);
+            const bool low = (ad >> 32) == 0;
+            ad = low ? ad << 32 : ad;
+            const int na = clz_u32(uint32_t(ad >> 32) | 1u);
+            ad <<= na;
+            uint64_t z = mul_hi(mul_hi(ad, T), c.KM);
+            const int nz = clz_u32(uint32_t(z >> 32) | 1u);
+            z <<= nz;
+            const int ez = E + eT + c.eK + 128 - na - (low ? 32 : 0) - nz;
+            const uint64_t h = mn - shr_u64(c.RM, nn - c.eR + 1);
+            X = mul_hi(sqr_hi(h), mul_hi(b01, b2));
+            eX = 2 * nn + 256;
+            Y = sqr_hi(z);
+            eY = z == 0 ? -(1 << 20) : 2 * ez + 192;
+        }
+        Y0 = mul_hi(Y, b12);
+        Y1 = mul_hi(Y, b02);
+        Y2 = mul_hi(Y, b01);
+        f0 = eY - n0;
+        f1 = eY - n1;
+        f2 = eY - n2;
     }
-    uint64_t z = mul_hi(mul_hi(ad, T), c.KM);
-    {
-        const int n = clz_u32(uint32_t(z >> 32) | 1u);
-        z <<= n;
-        ez -= n;
-    }
-    ez = z == 0 ? -(1 << 20) : ez;
-    const uint64_t Y = sqr_hi(z);
-    const uint64_t b01 = mul_hi(b0, b1), b12 = mul_hi(b1, b2), b02 = mul_hi(b0, b2);
-    const uint64_t X = mul_hi(sqr_hi(h), mul_hi(b01, b2));
-    const uint64_t Y0 = mul_hi(Y, b12), Y1 = mul_hi(Y, b02), Y2 = mul_hi(Y, b01);
-    // exponents relative to that of b_0 b_1 b_2: X = X 2^eX, Y_k = Y_k 2^(eY - n_k); a_k = X + Y_k
-    // below 2^59 with the exponent of its larger term's leading bit (at most six zeros counted)
-    const int eX = 2 * nn + 256, eY = 2 * ez + 192;
-    const int f0 = eY - n0, f1 = eY - n1, f2 = eY - n2;
+    // a_k below 2^59 with the exponent of its larger term's leading bit (at most six zeros counted)
     const int tX = eX - leading_zeros6(X);
     const int m0 = max_i(tX, f0 - leading_zeros6(Y0)) + 6;
     const int m1 = max_i(tX, f1 - leading_zeros6(Y1)) + 6;
@@ -321,8 +342,9 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
     q <<= nq;
     // round to 53 bits; a carry out of the mantissa raises the exponent by itself
     const uint64_t r = ((q >> 10) + 1) >> 1;
-    const uint32_t ex = uint32_t(km - dm + 1 - nt - (up ? 32 : 0) + nd - nq) << 20;
-    const uint64_t bits = N == 0 ? 0 : r + join(ex | sign, 0);
+    // (an exponent below the normal range: every product of weight vanished against a flat pair's)
+    const int ex = km - dm + 1 - nt - (up ? 32 : 0) + nd - nq;
+    const uint64_t bits = N == 0 || ex < 0 ? 0 : r + join((uint32_t(ex) << 20) | sign, 0);
 #ifdef __CUDA_ARCH__
     return __longlong_as_double((long long)bits);
 #else
@@ -372,9 +394,9 @@ WZ_HD float float_rcp(float x) {
 #endif
 }
 
-WZ_HD float wide_float(int64_t x) {                  // x 2^-57 to 24 bits
+WZ_HD float wide_float(int64_t x) {                  // x 2^-56 to 24 bits
     const Limbs l(x);
-    return fmaf(float(l.h), 0x1p-25f, float(l.l) * 0x1p-57f);
+    return fmaf(float(l.h), 0x1p-24f, float(l.l) * 0x1p-56f);
 }
 
 WZ_HD uint64_t double_bits(double v) {
@@ -439,7 +461,8 @@ WZ_HD double wide_rsqrt(double x, bool& ok) {
 }
 
 // f^ - c where the weights hardly differ from the optimal ones; false where that is not shown.
-// With r_k = (K d4 T)^2 / (h^2 b_k) the weights are c_k (1 + r_k), so f^ - c is the optimal
+// With r_k = (K d4 T)^2 / (h^2 b_k) the weights are c_k (1 + r_k) (the other weight functions alike
+// with their own r_k), so f^ - c is the optimal
 // linear combination of the differences, formed exactly in integers, plus
 //   sum c_k r_k (g_k - lin) / (1 + sum c_k r_k),
 // a combination of the second differences delta_0 = D1 - 2 D2 + D3 and delta_1 = D2 - 2 D3 + D4.
@@ -452,10 +475,10 @@ WZ_HD double wide_rsqrt(double x, bool& ok) {
 // value from below (eb <= 0: nothing is known of it).
 // About 150 instructions instead of 600 for a warp whose lanes are all accepted.
 WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
-                       const WideConst& c, double& corr) {
+                       const WideConst& c, int weights, double& corr) {
     const int G = max_i(max_i(G1, G2), max_i(G3, G4));
-    const int64_t c1 = shr_s64(D1, G - G1 + 3), c2 = shr_s64(D2, G - G2 + 3);      // |c_i| <= 2^57
-    const int64_t c3 = shr_s64(D3, G - G3 + 3), c4 = shr_s64(D4, G - G4 + 3);
+    const int64_t c1 = shr_s64(D1, G - G1 + 4), c2 = shr_s64(D2, G - G2 + 4);      // |c_i| <= 2^56
+    const int64_t c3 = shr_s64(D3, G - G3 + 4), c4 = shr_s64(D4, G - G4 + 4);
     const int64_t s0 = c1 - c2, s1 = c2 - c3, s2 = c3 - c4, d0 = s0 - s1, d1 = s1 - s2;
     const float f2 = wide_float(c2), f3 = wide_float(c3), S1 = wide_float(s1), E0 = wide_float(d0),
                 E1 = wide_float(d1), Q = wide_float(d0 - d1);
@@ -468,25 +491,47 @@ WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, i
     const float A = fabsf(E0) + fabsf(E1), M = fabsf(f2) + fabsf(S1) + A;
     const float T = fabsf(fmaf(4.0f * (E0 + E1), S0 + S2, 3.0f * fmaf(f3, E1, -(f2 * E0)))) + R;
     const float ET = 0x1p-18f * A * M;
-    const float u = c.Kf * Q * float_rcp(fminf(be0, be2) + 0.5f * R);
-    const float w = (u * T) * (u * T);
     const float i0 = float_rcp(b0), i1 = float_rcp(b1), i2 = float_rcp(b2);
-    const float im = fmaxf(fmaxf(i0, i1), i2), rm = w * im;
-    const float err = fmaf(fabsf(u) * ET * im, fabsf(u) * fmaf(2.0f, T, ET), 0x1p-14f * rm);
+    const float im = fmaxf(fmaxf(i0, i1), i2);
+    float r0, r1, r2, err;
+    if (weights == 0) {
+        const float u = c.Kf * Q * float_rcp(fminf(be0, be2) + 0.5f * R);
+        const float w = (u * T) * (u * T);
+        r0 = w * i0;
+        r1 = w * i1;
+        r2 = w * i2;
+        err = fmaf(fabsf(u) * ET * im, fabsf(u) * fmaf(2.0f, T, ET), 0x1p-14f * (w * im));
+    } else if (weights == 1) {
+        // WENO-Z: r_k = |b_0 - b_2| / b_k
+        r0 = (T - R) * i0;
+        r1 = (T - R) * i1;
+        r2 = (T - R) * i2;
+        err = fmaf(ET, im, 0x1p-14f * (T * im));
+    } else if (weights == 3) {
+        // Jiang-Shu: r_k = (b_1 - b_k)(b_1 + b_k) / b_k^2, the differences of the b's from the delta's
+        r0 = E0 * fmaf(3.0f, f2, -4.0f * (S0 + S1)) * (b1 + b0) * i0 * i0;
+        r1 = 0.0f;
+        r2 = E1 * fmaf(3.0f, f3, 4.0f * (S1 + S2)) * (b1 + b2) * i2 * i2;
+        err = ET * (b0 + b1 + b2) * im * im + 0x1p-14f * (fabsf(r0) + fabsf(r2));
+    } else {
+        r0 = r1 = r2 = err = 0.0f;
+    }
     const int ef = eb - G + 126;                              // 2^(eb - 1023) in the floats' units
     const float fb = bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
     if (!(A * err <= 0x1p-53f * (fabsf(f2) + fabsf(f3) + fb)) ||
         unsigned(G - kWideMinExp) >= unsigned(kWideMaxExp - kWideMinExp))
         return false;
     // 60 (f^ - c) = lin + sum 10 c_k r_k (10 g_k - lin) / (10 + sum 10 c_k r_k)
-    const float r0 = w * i0, r1 = 6.0f * w * i1, r2 = 3.0f * w * i2;
+    r1 *= 6.0f;
+    r2 *= 3.0f;
     const float num = fmaf(r0, fmaf(18.0f, E0, -3.0f * E1),
                            fmaf(r1, fmaf(-2.0f, E0, -3.0f * E1), r2 * fmaf(-2.0f, E0, 7.0f * E1)));
     const uint32_t v = float_bits(num * float_rcp(10.0f + (r0 + r1 + r2)));
     const int ve = int((v >> 23) & 0xffu);
-    const int64_t vm = int64_t(shr_u64(join(((v & 0x7fffffu) | (ve ? 0x800000u : 0u)) << 6, 0), 131 - ve > 0 ? 131 - ve : 0));
+    // (below 2^7: the float is an average of 18 delta_0 - 3 delta_1 and the like, |delta| <= 4)
+    const int64_t vm = int64_t(shr_u64(join(((v & 0x7fffffu) | (ve ? 0x800000u : 0u)) << 7, 0), 133 - ve));
     const int64_t S = 2 * c1 - 11 * c2 - 24 * c3 + 3 * c4 + (int32_t(v) < 0 ? -vm : vm);
-    // S 2^(G - 1079) / 60 as a double
+    // S 2^(G - 1078) / 60 as a double, |S| <= 70 2^56
     const uint32_t sign = uint32_t(uint64_t(S) >> 32) & 0x80000000u;
     uint64_t N = uint64_t(S < 0 ? -S : S);
     const bool up = (N >> 32) == 0;
@@ -496,7 +541,7 @@ WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, i
     const int nq = clz_u32(uint32_t(q >> 32) | 1u);
     q <<= nq;
     const uint64_t r = ((q >> 10) + 1) >> 1;
-    const uint32_t ex = uint32_t(G + 1 - nt - (up ? 32 : 0) - nq) << 20;
+    const uint32_t ex = uint32_t(G + 2 - nt - (up ? 32 : 0) - nq) << 20;
     const uint64_t bits = N == 0 ? 0 : r + join(ex | sign, 0);
 #ifdef __CUDA_ARCH__
     corr = __longlong_as_double((long long)bits);
@@ -508,16 +553,19 @@ WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, i
 
 // The weighted evaluation as a call of its own: the warps of smooth data pass it by, and one copy
 // of its code serves every field (inlined four times it does not fit the instruction cache).
+// W: the weight function, -1 for the run-time value.
+template <int W>
 #ifdef __CUDACC__
 static __device__ __noinline__
 #else
 inline
 #endif
-double wide_weighted_call(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, WideConst c) {
+double wide_weighted_call(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, WideConst c,
+                          int weights) {
     int e0, e1, e2, e3;
     const int64_t x0 = wide_normalise(D1, G1, e0), x1 = wide_normalise(D2, G2, e1), x2 = wide_normalise(D3, G3, e2),
                   x3 = wide_normalise(D4, G4, e3);
-    return wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c);
+    return wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c, W < 0 ? weights : W);
 }
 
 // Whether the largest difference lies in the range of the integer evaluation (E its exponent).
@@ -525,10 +573,11 @@ WZ_HD bool wide_in_range(int E) { return unsigned(E - kWideMinExp) < unsigned(kW
 
 // f^ - c from D_i 2^(G_i - 1082), |D_i| <= 2^60, to be added to a value of exponent eb.  False
 // where the caller has to take the double evaluation (the largest difference outside the range
-// above).
+// above).  W: the weight function, -1 for the run-time value.
+template <int W>
 WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
-                           const WideConst& c, double& corr) {
-    if (wide_linear(D1, D2, D3, D4, G1, G2, G3, G4, eb, c, corr)) return true;
+                           const WideConst& c, int weights, double& corr) {
+    if (wide_linear(D1, D2, D3, D4, G1, G2, G3, G4, eb, c, W < 0 ? weights : W, corr)) return true;
     corr = 0.0;
     int e0, e1, e2, e3;
     wide_normalise(D1, G1, e0);
@@ -536,21 +585,24 @@ WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G
     wide_normalise(D3, G3, e2);
     wide_normalise(D4, G4, e3);
     const int E = max_i(max_i(e0, e1), max_i(e2, e3));
-    if (!wide_in_range(E)) return E == 0;
-    corr = wide_weighted_call(D1, D2, D3, D4, G1, G2, G3, G4, c);
+    if (!wide_in_range(E) || (W < 0 && weights == 2)) return E == 0;
+    corr = wide_weighted_call<W>(D1, D2, D3, D4, G1, G2, G3, G4, c, weights);
     return true;
 }
 
 // The same from the first differences as doubles (infinities and NaN return false).
-WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, int eb, const WideConst& c, double& corr) {
+template <int W>
+WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, int eb, const WideConst& c, int weights,
+                           double& corr) {
     int e0, e1, e2, e3;
     const int64_t x0 = wide_unpack(D1, e0), x1 = wide_unpack(D2, e1), x2 = wide_unpack(D3, e2),
                   x3 = wide_unpack(D4, e3);
     const int E = max_i(max_i(e0, e1), max_i(e2, e3));
     corr = 0.0;
     if (!wide_in_range(E)) return E == 0;
-    if (!wide_linear(x0, x1, x2, x3, e0, e1, e2, e3, eb, c, corr))
-        corr = wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c);
+    if (wide_linear(x0, x1, x2, x3, e0, e1, e2, e3, eb, c, W < 0 ? weights : W, corr)) return true;
+    if (W < 0 && weights == 2) return false;
+    corr = wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c, W < 0 ? weights : W);
     return true;
 }
 

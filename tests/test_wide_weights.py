@@ -15,14 +15,15 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2004_07954_gb300", "csrc")
 SHIM = """
 #include "wide_weights.cuh"
-extern "C" long wide_line(const double* f, long n, int side, double eps, double A, double* out) {
+extern "C" long wide_line(const double* f, long n, int side, double eps, double A, int weights,
+                          double* out) {
     const wz::WideConst c = wz::wide_const(eps, A);
     long refused = 0;
     for (long j = 0; j <= n; ++j) {
         const double* s = f + j;
         double v[5], corr;
         for (int k = 0; k < 5; ++k) v[k] = side > 0 ? s[k] : s[5 - k];
-        if (!wz::wide_correction(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], wz::exponent_of(v[2]), c, corr))
+        if (!wz::wide_correction<-1>(v[0] - v[1], v[1] - v[2], v[2] - v[3], v[3] - v[4], wz::exponent_of(v[2]), c, weights, corr))
             ++refused, corr = 0.0;
         out[j] = v[2] + corr;
     }
@@ -41,12 +42,12 @@ def wide(tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(so)
     P = ctypes.c_void_p
-    L.wide_line.argtypes = [P, ctypes.c_long, ctypes.c_int, ctypes.c_double, ctypes.c_double, P]
+    L.wide_line.argtypes = [P, ctypes.c_long, ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.c_int, P]
     L.wide_line.restype = ctypes.c_long
 
-    def line(f, side, eps=1e-40, A=10.0):
+    def line(f, side, eps=1e-40, A=10.0, weights=0):
         out = np.empty(f.size - 5)
-        refused = L.wide_line(f.ctypes.data, f.size - 6, side, eps, A, out.ctypes.data)
+        refused = L.wide_line(f.ctypes.data, f.size - 6, side, eps, A, weights, out.ctypes.data)
         return out, refused
 
     return line
@@ -88,6 +89,18 @@ def test_integer_evaluation_against_binary128(wide, orc, name, eps, A):
             ref = orc.reconstruct_quad(fs, side, eps=eps, A=A)
             if refused == 0:
                 assert np.all(np.abs(got - ref) <= _bound(fs, ref, side)), (scale, side)
+
+
+@pytest.mark.parametrize("weights,eps", [(1, 1e-40), (1, 1e-6), (2, 1e-40), (3, 1e-6), (3, 1e-40)])
+@pytest.mark.parametrize("name", list(_lines()))
+def test_integer_evaluation_of_the_other_weights(wide, orc, name, weights, eps):
+    """WENO-Z, linear and Jiang-Shu weights, the same bound."""
+    f = np.ascontiguousarray(_lines()[name])
+    for side in (1, -1):
+        got, refused = wide(f, side, eps, 10.0, weights)
+        ref = orc.reconstruct_quad(f, side, eps=eps, kind=weights)
+        assert refused == 0
+        assert np.all(np.abs(got - ref) <= _bound(f, ref, side)), side
 
 
 def test_constant_data_are_exact_and_other_values_refused(wide):
