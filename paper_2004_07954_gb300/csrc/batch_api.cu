@@ -97,18 +97,36 @@ int resolve_shape(const wenozn_batch_params* bp, int64_t cells) {
 
 struct TileSizes { int v[kNumBatchShapes]; };
 
-// Tile prefix counts of every shape: tile_off[s][b] = sum_{b' < b} ceil(n_b' / (tile_s - 1)).
-__global__ void batch_tiles_kernel(const int64_t* off, int B, int32_t* tile_off, TileSizes tiles) {
-    const int s = threadIdx.x;
-    if (s >= kNumBatchShapes) return;
-    const int per = tiles.v[s] - 1;
-    int32_t acc = 0;
+// Tile prefix counts of every shape: tile_off[s][b] = sum_{b' < b} ceil(n_b' / (tile_s - 1)),
+// one block per shape, 256 instances at a time (warp scans, then the warps' totals).
+__global__ void __launch_bounds__(256) batch_tiles_kernel(const int64_t* off, int B, int32_t* tile_off,
+                                                          TileSizes tiles) {
+    __shared__ int32_t s_warp[8];
+    const int s = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t per = uint32_t(tiles.v[s] - 1);
     int32_t* row = tile_off + size_t(s) * (B + 1);
-    row[0] = 0;
-    for (int b = 0; b < B; ++b) {
-        const int64_t n = off[b + 1] - off[b];
-        acc += int32_t((n + per - 1) / per);
-        row[b + 1] = acc;
+    int32_t base = 0;
+    if (threadIdx.x == 0) row[0] = 0;
+    for (int b0 = 0; b0 < B; b0 += 256) {
+        const int b = b0 + int(threadIdx.x);
+        // (an instance holds fewer than 2^31 cells)
+        int32_t v = b < B ? int32_t((uint32_t(off[b + 1] - off[b]) + per - 1) / per) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
+        }
+        if (lane == 31) s_warp[w] = v;
+        __syncthreads();
+        int32_t before = 0, total = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            before += q < w ? s_warp[q] : 0;
+            total += s_warp[q];
+        }
+        if (b < B) row[b + 1] = base + before + v;
+        base += total;
+        __syncthreads();
     }
 }
 
@@ -229,7 +247,7 @@ wenozn_status wenozn_batch_init(const wenozn_batch_params* bp, const int64_t* of
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p.dx, dx, size_t(bp->nbatch) * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-        batch_tiles_kernel<<<1, 32, 0, s>>>(p.off, bp->nbatch, p.tile_off, tiles);
+        batch_tiles_kernel<<<kNumBatchShapes, 256, 0, s>>>(p.off, bp->nbatch, p.tile_off, tiles);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {

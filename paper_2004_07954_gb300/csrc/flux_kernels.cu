@@ -21,29 +21,35 @@ namespace wz {
 namespace {
 
 // Tile shapes: TI interfaces along the sweep x TA lines across it, THREADS per block: one
-// interface a thread, and four blocks (32 warps, 64 registers a thread) an SM in the default
-// kernels, because the FP64 phases of one block (cells, Roe state) have to run beside the
-// integer phases of others.  Both sweeps of a 2D tile lie alike in shared memory (cell lc of
-// line l at lc TA + l), so one copy of the interface code serves both, and a warp covers a
-// patch of 4 x 8 interfaces, which few fronts touch (a warp with one stencil at a front runs
-// the weighted evaluation for all of its lanes).  Both sweeps at 256^2 / 1024^2 / 4096^2: 80 us /
-// 0.54 / 7.4 ms; three blocks 91 us / 0.54 / 7.6 ms, two 97 us / 0.71 / 9.2 ms, 64 x 4 tiles (four
-// blocks) 88 us / 0.58 / 7.55 ms, 128-thread blocks (eight) 84 us / 0.58 / 7.8 ms, a copy of the
+// interface a thread, and several small blocks an SM, because the FP64 phases of one block
+// (cells, Roe state) have to run beside the integer phases of others.  Both sweeps of a 2D
+// tile lie alike in shared memory (cell lc of line l at lc TA + l), so one copy of the
+// interface code serves both, and a warp covers a patch of 4 x 8 interfaces, which few fronts
+// touch (a warp with one stencil at a front runs the weighted evaluation for all of its lanes).
+// Both sweeps at 256^2 / 1024^2 / 4096^2, without the linear pass: 80 us / 0.54 / 7.5 ms with four
+// blocks (32 warps, 64 registers); three blocks 86 us / 0.53 / 7.5 ms, two 97 us / 0.71 / 9.2 ms,
+// 64 x 4 tiles 88 us / 0.58 / 7.55 ms, 128-thread blocks (eight) 84 us / 0.58 / 7.8 ms, a copy of the
 // code per sweep (128 x 2 and 32 x 8 tiles) 98 us / 0.63 / 7.85 ms.
+// The linear pass (LIN, interface_linear first, the rest compacted): 97 us / 0.47 / 5.75 ms with
+// three blocks, 97 us / 0.55 / 5.8 ms with four.  It pays where most interfaces pass, so lines of
+// kLinearMin cells and more take it; a single wave of blocks (short 1D lines) waits for its
+// slowest block, which pays for both passes, and does without (a rollout at 8192 cells 7.7 ms
+// without, 8.2 ms with).
 // Long 1D lines use 251-interface tiles (256 cells with the halo: one full round of the cell
-// and difference passes; a 2^20-cell step 0.70 ms, with three blocks 0.73, with two 0.83 ms);
-// short ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
+// and difference passes; a 2^20-cell step 0.52 ms, without the linear pass 0.70 ms); short
+// ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
 // every SM gets work.  GEN = 2 projects F and U (twice the difference vectors a thread) and runs
 // best with two blocks and 128 registers (a 640 x 777 local-LF step 1.76 ms; three blocks 1.81,
 // four 1.85 ms).
-template <int NV, bool SMALL = false> struct Tile { static constexpr int TI = 251, TA = 1, THREADS = 256, BLOCKS = 4; };
-template <int NV> struct Tile<NV, true> { static constexpr int TI = 64, TA = 1, THREADS = 64, BLOCKS = 2; };
-template <> struct Tile<4, false> { static constexpr int TI = 32, TA = 8, THREADS = 256, BLOCKS = 4; };
+constexpr int kLinearMin = 1024;
+template <int NV, bool SMALL = false> struct Tile { static constexpr int TI = 251, TA = 1, THREADS = 256; };
+template <int NV> struct Tile<NV, true> { static constexpr int TI = 64, TA = 1, THREADS = 64; };
+template <> struct Tile<4, false> { static constexpr int TI = 32, TA = 8, THREADS = 256; };
 
 // One tile of a sweep along dir: tile ta along the sweep direction, tile tc across it.  (The
 // direction is a run-time value where one kernel holds both, so that they share one copy of
 // the interface code, which fills most of the instruction cache.)
-template <int NV, bool SMALL, int GEN>
+template <int NV, bool SMALL, int GEN, bool LIN>
 __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int bc, const int dir, int ta, int tc,
                                           double* smem) {
     using T = Tile<NV, SMALL>;
@@ -101,12 +107,9 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
 
     // ---- interfaces ----------------------------------------------------------------
     const int nint = n + 1;
-    for (int idx = threadIdx.x; idx < TI * TA; idx += kThreads) {
+    auto store = [&](int idx, const double* Fh) {
+        // undoing the direction frame
         const int j = j0 + idx / TA, line = l0 + idx % TA;
-        if (j >= nint || line >= nlines) continue;
-        double Fh[NV];
-        interface_flux<NV, GEN>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
-        // store, undoing the direction frame
         const int64_t base = x ? int64_t(line) * (a.nx + 1) + j : int64_t(j) * a.nx + line;
         const int64_t plane = x ? int64_t(a.ny) * (a.nx + 1) : int64_t(a.ny + 1) * a.nx;
         Fout[base] = Fh[0];
@@ -115,30 +118,64 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
             if (NV == 4) Fout[(x ? 2 : 1) * plane + base] = Fh[2];
             Fout[(NV - 1) * plane + base] = Fh[NV - 1];
         }
+    };
+    // LIN: the interfaces with near-optimal weights first; the others are listed and share full
+    // warps afterwards
+    __shared__ int s_count;
+    __shared__ unsigned short s_list[LIN ? TI * TA : 1];
+    int count = TI * TA;
+    const bool linear = LIN && n >= kLinearMin;
+    if (LIN && linear) {
+        if (threadIdx.x == 0) s_count = 0;
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < TI * TA; idx += kThreads) {
+            const int j = j0 + idx / TA, line = l0 + idx % TA;
+            if (j >= nint || line >= nlines) continue;
+            double Fh[NV];
+            if (interface_linear<NV>(sp, idx, kStride, gm1, a.wide, Fh)) store(idx, Fh);
+            else s_list[atomicAdd(&s_count, 1)] = (unsigned short)idx;
+        }
+        __syncthreads();
+        count = s_count;
+    }
+    for (int q = threadIdx.x; q < count; q += kThreads) {
+        const int idx = LIN && linear ? s_list[q] : q;
+        const int j = j0 + idx / TA, line = l0 + idx % TA;
+        if (j >= nint || line >= nlines) continue;
+        double Fh[NV];
+        interface_flux<NV, GEN, LIN>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
+        store(idx, Fh);
     }
 }
 
-template <int NV, int DIR, bool SMALL, int GEN>
-__global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, SMALL || GEN == 2 ? 2 : Tile<NV, SMALL>::BLOCKS)
-    flux_kernel(FluxArgs a) {
+// Whether a problem takes the LIN kernels: WENO-ZN weights on split fluxes, and a line long
+// enough for smooth data to be resolved well.
+bool takes_linear(const FluxArgs& a, int n) { return a.weights == 0 && (a.split == 0 || a.split == 3) && n >= kLinearMin; }
+
+// Blocks an SM: see the tile shapes
+template <int NV, bool SMALL, int GEN, bool LIN>
+constexpr int min_blocks() { return SMALL || GEN == 2 ? 2 : (NV == 4 && LIN ? 3 : 4); }
+
+template <int NV, int DIR, bool SMALL, int GEN, bool LIN>
+__global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMALL, GEN, LIN>())) flux_kernel(FluxArgs a) {
     extern __shared__ double smem[];
     pdl_wait();
-    flux_tile<NV, SMALL, GEN>(a, a.Fout, a.bc, DIR, DIR == 0 ? blockIdx.x : blockIdx.y,
-                              DIR == 0 ? blockIdx.y : blockIdx.x, smem);
+    flux_tile<NV, SMALL, GEN, LIN>(a, a.Fout, a.bc, DIR, DIR == 0 ? blockIdx.x : blockIdx.y,
+                                   DIR == 0 ? blockIdx.y : blockIdx.x, smem);
 }
 
 // Both sweeps of a 2D stage in one grid, so that they share one tail: blocks [0, nbx) take
 // the x tiles (along the sweep fastest, as flux_kernel<4, 0>), the others the y tiles
 // (across the sweep fastest, as flux_kernel<4, 1>).
-template <int GEN>
-__global__ void __launch_bounds__(Tile<4>::THREADS, GEN == 2 ? 2 : Tile<4>::BLOCKS)
+template <int GEN, bool LIN>
+__global__ void __launch_bounds__(Tile<4>::THREADS, (min_blocks<4, false, GEN, LIN>()))
     flux_xy_kernel(FluxArgs ax, double* Fy, int bc_y, int x_along, int nbx, int y_across) {
     extern __shared__ double smem[];
     pdl_wait();
     const int b = int(blockIdx.x), q = b - nbx;
     const bool x = b < nbx;
-    flux_tile<4, false, GEN>(ax, x ? ax.Fout : Fy, x ? ax.bc : bc_y, x ? 0 : 1, x ? b % x_along : q / y_across,
-                             x ? b / x_along : q % y_across, smem);
+    flux_tile<4, false, GEN, LIN>(ax, x ? ax.Fout : Fy, x ? ax.bc : bc_y, x ? 0 : 1, x ? b % x_along : q / y_across,
+                                  x ? b / x_along : q % y_across, smem);
 }
 
 template <int NV, bool SMALL, int GEN>
@@ -147,7 +184,7 @@ constexpr size_t tile_smem() {
            (GEN != 0 ? CellPlanes<NV>::kPerCellGeneric : CellPlanes<NV>::kPerCellDefault) * sizeof(double);
 }
 
-template <int GEN>
+template <int GEN, bool LIN>
 cudaError_t launch_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t s) {
     constexpr size_t smem = tile_smem<4, false, GEN>();
     static std::atomic<unsigned long long> configured{0};
@@ -156,7 +193,7 @@ cudaError_t launch_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(flux_xy_kernel<GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        e = cudaFuncSetAttribute(flux_xy_kernel<GEN, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
@@ -164,11 +201,11 @@ cudaError_t launch_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t s) {
     const int nbx = x_along * ((ax.ny + Tile<4>::TA - 1) / Tile<4>::TA);
     const int y_across = (ay.nx + Tile<4>::TA - 1) / Tile<4>::TA;
     const int nby = y_across * ((ay.ny + 1 + Tile<4>::TI - 1) / Tile<4>::TI);
-    return launch_pdl(flux_xy_kernel<GEN>, dim3(unsigned(nbx + nby)), dim3(Tile<4>::THREADS), smem, s, ax, ay.Fout,
+    return launch_pdl(flux_xy_kernel<GEN, LIN>, dim3(unsigned(nbx + nby)), dim3(Tile<4>::THREADS), smem, s, ax, ay.Fout,
                       ay.bc, x_along, nbx, y_across);
 }
 
-template <int NV, int DIR, bool SMALL, int GEN>
+template <int NV, int DIR, bool SMALL, int GEN, bool LIN>
 cudaError_t launch_one(const FluxArgs& a, cudaStream_t s) {
     constexpr int TI = Tile<NV, SMALL>::TI, TA = Tile<NV, SMALL>::TA;
     constexpr size_t smem = tile_smem<NV, SMALL, GEN>();
@@ -179,7 +216,7 @@ cudaError_t launch_one(const FluxArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(flux_kernel<NV, DIR, SMALL, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(flux_kernel<NV, DIR, SMALL, GEN, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(smem));
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
@@ -189,7 +226,7 @@ cudaError_t launch_one(const FluxArgs& a, cudaStream_t s) {
     const unsigned along = unsigned((n + 1 + TI - 1) / TI);
     const unsigned across = unsigned((nlines + TA - 1) / TA);
     dim3 grid = DIR == 0 ? dim3(along, across) : dim3(across, along);
-    return launch_pdl(flux_kernel<NV, DIR, SMALL, GEN>, grid, dim3(Tile<NV, SMALL>::THREADS), smem, s, a);
+    return launch_pdl(flux_kernel<NV, DIR, SMALL, GEN, LIN>, grid, dim3(Tile<NV, SMALL>::THREADS), smem, s, a);
 }
 
 int sm_count_cached() {
@@ -208,18 +245,26 @@ cudaError_t launch_flux_t(int system, int dir, const FluxArgs& a, cudaStream_t s
         // 1D: short lines take the small tiles so that every SM has work
         const int64_t big_tiles = (int64_t(a.nx) + Tile<3>::TI) / Tile<3>::TI * a.ny;
         const bool small = big_tiles < 2 * sm_count_cached();
-        if (system == 0) return small ? launch_one<1, 0, true, GEN>(a, s) : launch_one<1, 0, false, GEN>(a, s);
-        return small ? launch_one<3, 0, true, GEN>(a, s) : launch_one<3, 0, false, GEN>(a, s);
+        if (system == 0)
+            return small ? launch_one<1, 0, true, GEN, false>(a, s) : launch_one<1, 0, false, GEN, false>(a, s);
+        if (small) return launch_one<3, 0, true, GEN, false>(a, s);
+        if constexpr (GEN != 2)
+            if (takes_linear(a, a.nx)) return launch_one<3, 0, false, GEN, true>(a, s);
+        return launch_one<3, 0, false, GEN, false>(a, s);
     }
-    return dir == 0 ? launch_one<4, 0, false, GEN>(a, s) : launch_one<4, 1, false, GEN>(a, s);
+    if constexpr (GEN != 2)
+        if (takes_linear(a, dir == 0 ? a.nx : a.ny))
+            return dir == 0 ? launch_one<4, 0, false, GEN, true>(a, s) : launch_one<4, 1, false, GEN, true>(a, s);
+    return dir == 0 ? launch_one<4, 0, false, GEN, false>(a, s) : launch_one<4, 1, false, GEN, false>(a, s);
 }
 
 }  // namespace
 
 cudaError_t launch_flux_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t s) {
-    if (ax.weights == 0 && ax.split == 0) return launch_xy<0>(ax, ay, s);
-    const bool diff = ax.split == 0 || ax.split == 3;
-    return diff ? launch_xy<1>(ax, ay, s) : launch_xy<2>(ax, ay, s);
+    const bool lin = takes_linear(ax, ax.nx > ax.ny ? ax.nx : ax.ny);
+    if (ax.weights == 0 && ax.split == 0) return lin ? launch_xy<0, true>(ax, ay, s) : launch_xy<0, false>(ax, ay, s);
+    if (ax.split == 0 || ax.split == 3) return lin ? launch_xy<1, true>(ax, ay, s) : launch_xy<1, false>(ax, ay, s);
+    return launch_xy<2, false>(ax, ay, s);
 }
 
 cudaError_t launch_flux(int system, int dir, const FluxArgs& a, cudaStream_t s) {

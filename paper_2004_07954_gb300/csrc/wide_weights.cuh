@@ -460,6 +460,29 @@ WZ_HD double wide_rsqrt(double x, bool& ok) {
     return bits_double((((y >> 10) + 1) >> 1) + (uint64_t(1022 - ((ee - 1022) >> 1)) << 52));
 }
 
+// S 2^(G - 1078) / 60 as a double, |S| < 2^63
+WZ_HD double wide_sixtieth(int64_t S, int G) {
+    const uint32_t sign = uint32_t(uint64_t(S) >> 32) & 0x80000000u;
+    uint64_t N = uint64_t(S < 0 ? -S : S);
+    const bool up = (N >> 32) == 0;
+    N = up ? N << 32 : N;
+    const int nt = clz_u32(uint32_t(N >> 32) | 1u);
+    uint64_t q = mul_hi(N << nt, 9838263505978427528ull);     // 2^69 / 60
+    const int nq = clz_u32(uint32_t(q >> 32) | 1u);
+    q <<= nq;
+    const uint64_t r = ((q >> 10) + 1) >> 1;
+    const uint32_t ex = uint32_t(G + 2 - nt - (up ? 32 : 0) - nq) << 20;
+    return bits_double(N == 0 ? 0 : r + join(ex | sign, 0));
+}
+
+// A double to float by truncation of its bits; not a number outside [2^-126, 2^127) but for 0.
+WZ_HD float wide_truncate(double v) {
+    const uint64_t u = double_bits(v);
+    const uint32_t hi = uint32_t(u >> 32), a = (hi & 0x7fffffffu) - (897u << 20);
+    const uint32_t f = funnel_l(uint32_t(u), a + (1u << 20), 3) | (hi & 0x80000000u);
+    return bits_float(a < (253u << 20) ? f : ((u << 1) == 0 ? 0u : 0x7fffffffu));
+}
+
 // f^ - c where the weights hardly differ from the optimal ones; false where that is not shown.
 // With r_k = (K d4 T)^2 / (h^2 b_k) the weights are c_k (1 + r_k) (the other weight functions alike
 // with their own r_k), so f^ - c is the optimal
@@ -531,23 +554,7 @@ WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, i
     // (below 2^7: the float is an average of 18 delta_0 - 3 delta_1 and the like, |delta| <= 4)
     const int64_t vm = int64_t(shr_u64(join(((v & 0x7fffffu) | (ve ? 0x800000u : 0u)) << 7, 0), 133 - ve));
     const int64_t S = 2 * c1 - 11 * c2 - 24 * c3 + 3 * c4 + (int32_t(v) < 0 ? -vm : vm);
-    // S 2^(G - 1078) / 60 as a double, |S| <= 70 2^56
-    const uint32_t sign = uint32_t(uint64_t(S) >> 32) & 0x80000000u;
-    uint64_t N = uint64_t(S < 0 ? -S : S);
-    const bool up = (N >> 32) == 0;
-    N = up ? N << 32 : N;
-    const int nt = clz_u32(uint32_t(N >> 32) | 1u);
-    uint64_t q = mul_hi(N << nt, 9838263505978427528ull);     // 2^69 / 60
-    const int nq = clz_u32(uint32_t(q >> 32) | 1u);
-    q <<= nq;
-    const uint64_t r = ((q >> 10) + 1) >> 1;
-    const uint32_t ex = uint32_t(G + 2 - nt - (up ? 32 : 0) - nq) << 20;
-    const uint64_t bits = N == 0 ? 0 : r + join(ex | sign, 0);
-#ifdef __CUDA_ARCH__
-    corr = __longlong_as_double((long long)bits);
-#else
-    std::memcpy(&corr, &bits, 8);
-#endif
+    corr = wide_sixtieth(S, G);
     return true;
 }
 

@@ -180,3 +180,67 @@ def test_gpu_integer_projection(orc, kind):
             # rounding of the fluxes whose differences the RHS is: 1e-12 of the largest flux / dx
             scale = max(np.abs(want[k]).max(), 1e-3 * np.abs(want).max())
             assert np.abs(got[k] - want[k]).max() <= 1e-12 * scale, k
+
+
+def _smooth_line(kind, n, dx):
+    """Periodic 1D Euler states around the linear pass's acceptance: waves from well to badly
+    resolved, alone, with jumps, with constant pieces, nearly incompressible, supersonic."""
+    from paper_2004_07954_gb300 import inputs
+    x = (np.arange(n) + 0.5) * dx
+    g = np.random.default_rng(3)
+    wave = lambda m, a: a * np.sin(2 * np.pi * m * x / (n * dx) + g.uniform(0, 6.28))
+    m = {"waves": n // 200, "short waves": n // 20, "all waves": None}.get(kind, n // 100)
+    if m is None:                            # every resolution from 1000 to 4 cells a wave
+        rho = 1.0 + sum(wave(q, 0.02) for q in (n // 1000 + 1, n // 300, n // 100, n // 50, n // 30, n // 15, n // 4))
+        u, p = 0.3 + wave(n // 80, 0.05), 1.0 + wave(n // 60, 0.05)
+    else:
+        rho, u, p = 1.0 + wave(m, 0.2), 0.4 + wave(m + 1, 0.2), 1.0 + wave(m + 2, 0.2)
+    if kind == "jumps":
+        rho, p = rho + (x > 0.3 * n * dx) + 2.0 * (x > 0.7 * n * dx), p + 3.0 * ((x > 0.5 * n * dx) & (x < 0.9 * n * dx))
+    elif kind == "pieces":
+        rho, u, p = np.where(np.sin(3e-3 * np.arange(n)) > 0, rho, 1.0), np.where(np.sin(3e-3 * np.arange(n)) > 0, u, 0.0), 1.0 + 0 * p
+    elif kind == "entropy":
+        u, p = 0.7 + 0 * u, 1.0 + 0 * p
+    elif kind == "low Mach":
+        u = 1e-4 * u
+    elif kind == "supersonic":
+        u = u + 6.0
+    return np.ascontiguousarray(inputs.cons_from_prim(rho, u, p).reshape(3, 1, n))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["waves", "short waves", "all waves", "jumps", "pieces", "entropy", "low Mach", "supersonic"])
+def test_gpu_linear_pass(orc, kind):
+    """Lines long enough for the linear pass (2^17 + 13 cells; the same states at 900 cells take the
+    other kernels): the RHS against the oracle at the suite's 1e-12 of the flux scale over dx
+    that the differences of the fluxes can carry, and the 2D sweeps of a repeated line."""
+    import torch
+    from paper_2004_07954_gb300 import build, wenozn as W
+    build.build()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    for n in (900, 131085):
+        dx = 1.0 / 900
+        U = _smooth_line(kind, n, dx)
+        p = W.wenozn_problem_init(1, n, 1, dx, 1.0, bc_x=W.WENOZN_BC_PERIODIC)
+        got = W.Solver(p).rhs(dev(U)).cpu().numpy()
+        want = orc.rhs(orc.problem(1, n, 1, dx=dx, bc_x=W.WENOZN_BC_PERIODIC), U)
+        for k in range(3):
+            # (alpha U and, in the momentum's, the pressure) / dx, alpha < 10
+            flux = (np.abs(U[k]).max() * 10.0 + (np.abs(U[2]).max() if k == 1 else 0.0)) / dx
+            assert np.abs(got[k] - want[k]).max() <= 1e-14 * flux, (n, k)
+    # both sweeps in 2D (1100 cells along, the line repeated across): the same values as in 1D
+    n, m = 1100, 40
+    U1 = _smooth_line(kind, n, 1.0 / n)
+    p1 = W.wenozn_problem_init(1, n, 1, 1.0 / n, 1.0, bc_x=W.WENOZN_BC_PERIODIC)
+    L1 = W.Solver(p1).rhs(dev(U1)).cpu().numpy()[:, 0]
+    for axis in (0, 1):
+        U = np.zeros((4, m, n))
+        U[0], U[1 + axis], U[3] = U1[0], U1[1], U1[2]
+        U = np.ascontiguousarray(U if axis == 0 else U.transpose(0, 2, 1))
+        nx, ny = (n, m) if axis == 0 else (m, n)
+        p = W.wenozn_problem_init(2, nx, ny, 1.0 / n, 1.0 / n, bc_x=W.WENOZN_BC_PERIODIC, bc_y=W.WENOZN_BC_PERIODIC)
+        L = W.Solver(p).rhs(dev(U)).cpu().numpy()
+        L = L if axis == 0 else L.transpose(0, 2, 1)
+        for k, q in ((0, 0), (1 + axis, 1), (3, 2)):
+            flux = (np.abs(U1[q]).max() * 10.0 + (np.abs(U1[2]).max() if q == 1 else 0.0)) * n
+            assert np.abs(L[k] - L1[q]).max() <= 1e-14 * flux, (axis, k)
