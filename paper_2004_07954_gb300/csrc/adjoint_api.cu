@@ -21,6 +21,7 @@ VjpArgs vjp_args(const wenozn_problem& p, const Layout& L, void* ws) {
     v.gamma = p.gamma;
     v.eps4 = 4.0 * p.eps;
     v.kappa = zn_kappa(p.A);
+    v.wide = wide_const(p.eps, p.A);
     v.adv_speed = p.adv_speed;
     return v;
 }

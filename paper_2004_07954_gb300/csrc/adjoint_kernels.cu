@@ -14,7 +14,9 @@
 // at x = 0.
 #include <atomic>
 
+#include "euler_device.cuh"
 #include "launch.h"
+#include "speed_screen.cuh"
 
 namespace wz {
 
@@ -126,6 +128,9 @@ struct EulerSmem {
     double U[3][NC];
     double hp[3][NC], hm[3][NC];
     double u[NC], H[NC], sq[NC], r[NC], Ep[NC];
+    int64_t dp[3][NC], dm[3][NC];       // mantissas of the split fluxes' differences
+    uint32_t ex[4][NC];                 // and their exponents (CellPlanes)
+    unsigned char lin[WIDE ? 1 : 3][TI];   // per-field threads: the field's weights are the optimal ones
     double red[WIDE ? 1 : 3][WIDE ? 1 : 19][WIDE ? 1 : TI];   // per field: cotangents of its projected
                                         // h+ (5) and h- (5), half its left-eigenvector row (3), 6 Roe
                                         // scalars (the per-field threads' exchange)
@@ -171,7 +176,9 @@ constexpr int kTIWide = 64;             // interfaces a block of the one-thread-
 // instructions: no per-field copies of the Roe state, the fields' cotangents summed in
 // registers, 5 of 64 interfaces computed twice instead of 5 of 32); shorter ones need the
 // per-field kernel's three times as many warps to occupy the GPU.  Measured crossover:
-// 8192 cells 105 (per field) against 154 us per reverse step, 12288 cells 196 against 165.
+// 8192 cells 105 (per field) against 154 us per reverse step, 12288 cells 196 against 165 (before
+// the linear reverse below: now 103 us at 8192, 425 against 1153 us at 131071 cells of smooth data;
+// a launch of one wave still waits for the blocks that hold a nonlinear interface).
 constexpr int kWideMinCells = 10240;
 
 template <int TI, bool WIDE>
@@ -301,6 +308,9 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
     const double gm1 = a.gamma - 1.0;
     const unsigned long long abits = a.alpha_bits[0];
     const double alpha = __longlong_as_double((long long)abits), half_alpha = 0.5 * alpha;
+    // (truncated alpha times 1 - 2^-11, NaN where alpha has no float: every cell is then evaluated)
+    const float gg1 = wide_truncate(a.gamma * gm1);
+    const float af = wide_truncate(alpha) * kScreenKeep, alpha_keep = af == af ? af : -1.0f;
     // the record the next launch writes is no longer read by anyone: clear its argmax word
     if (b == 0 && tid == 0) a.ctl[(a.rec_out + 1) % kVjpRecs] = 0u;
     if (tid == 0) S.cand = n;
@@ -365,13 +375,13 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
             s[m] = a.U[int64_t(m) * n + src];
             sm.U[m][c] = s[m];
         }
-        const double rs = rsqrt(s[0]), r = rs * rs;   // 1/sqrt(rho) and 1/rho, as the forward cell phase
+        const double rs = inv_sqrt(s[0]), r = rs * rs;   // 1/sqrt(rho) and 1/rho, as the forward cell phase
         const double u = s[1] * r;
-        const double p = gm1 * (s[2] - 0.5 * s[1] * u);
+        const double p = gm1 * (s[2] - wide_half(s[1] * u));
         const double Ep = s[2] + p;
         const double F[3] = {s[1], fma(s[1], u, p), u * Ep};
         for (int m = 0; m < 3; ++m) {
-            const double hF = 0.5 * F[m];
+            const double hF = wide_half(F[m]);
             sm.hp[m][c] = fma(half_alpha, s[m], hF);
             sm.hm[m][c] = fma(-half_alpha, s[m], hF);
         }
@@ -381,9 +391,13 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         sm.sq[c] = s[0] * rs;
         sm.r[c] = r;
         if (g == src && c >= 5 && c < 5 + kOwn) {   // an owned grid cell: is it the LF argmax?
-            double sx, sy;
-            wave_speeds<3>(s, a.gamma, sx, sy);
-            if ((unsigned long long)__double_as_longlong(sx) == abits) atomicMin(&S.cand, g);
+            // (a speed estimate, within 1.8e-5 of the speed, rules nearly every cell out)
+            const SpeedEstimate est = estimate_speeds<3>(s, gg1);
+            if (!est.ok || est.sx >= alpha_keep) {
+                double sx, sy;
+                wave_speeds<3>(s, a.gamma, sx, sy);
+                if ((unsigned long long)__double_as_longlong(sx) == abits) atomicMin(&S.cand, g);
+            }
         }
     }
 #pragma unroll
@@ -418,6 +432,17 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         }
     }
     __syncthreads();
+    // the differences of neighbouring cells' split fluxes, for the linear check
+    CellPlanes<3> planes(nullptr, kCells);
+    planes.hp = &sm.hp[0][0];
+    planes.hm = &sm.hm[0][0];
+    planes.sr = sm.sq;
+    planes.un = sm.u;
+    planes.H = sm.H;
+    planes.dp = &sm.dp[0][0];
+    planes.dm = &sm.dm[0][0];
+    planes.ex = &sm.ex[0][0];
+    for (int c = tid; c < kCells - 1; c += kThreads) cell_diffs<3>(planes, c, 1);
     // the block's lowest candidate: offered for the global argmax (the lowest index on ties),
     // with d(|u| + c)/dU of its state left in the record (|x|' = 0 at 0)
     if (tid == kCand && S.cand < n) {
@@ -491,13 +516,28 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         }
         if (mm == 0) S.pcell[p][e] = cell;
     }
-    if (need) __syncthreads();
+    __syncthreads();
     const bool live = j >= 0 && j <= n;
     const bool owned = live && ((j >= c0 && j < c0 + kOwn) || (j == n && b == nb - 1));
     const int cl = i + 2, cr = i + 3;            // cells j-1, j
+    // Where every field's weights are the optimal ones to rounding, derivatives included
+    // (NearLinear), F^ = f^+ + f^- is one linear combination of the cells' split fluxes in every
+    // component, (2, -13, 47, 27, -3) / 60 of h+ at positions 0..4 and its mirror image of h-, and
+    // depends neither on the Roe state nor on the eigenvectors: its reverse is those
+    // coefficients times the flux cotangent.
+    bool lin = false;
+    if (WIDE) {
+        if (live) lin = NearLinear<3, true>(planes, i, 1, gm1, a.wide, 0, 3).ok;
+    } else {
+        if (live) sm.lin[k][i] = NearLinear<3, true>(planes, i, 1, gm1, a.wide, k, k + 1).ok;
+        __syncthreads();
+        if (live) lin = sm.lin[0][i] & sm.lin[1][i] & sm.lin[2][i];
+    }
     double ut = 0, Ht = 0, c = 0, rc = 0, b1 = 0, b2 = 0, wl = 0, wr = 0, rS = 0;
     double Fb[3] = {0.0, 0.0, 0.0};
-    if (live) {
+    if (live)
+        for (int m = 0; m < 3; ++m) Fb[m] = (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx;   // cells j, j - 1
+    if (live && !lin) {
         // Roe state (R[0][k] = 1) and the cotangents of the interface flux
         const double sl = sm.sq[cl], sr = sm.sq[cr];
         rS = rcp_nr(sl + sr);
@@ -510,13 +550,12 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         c = c2 * rc;
         b1 = gm1 * rc * rc;
         b2 = 0.5 * ut * ut * b1;
-        for (int m = 0; m < 3; ++m) Fb[m] = (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx;   // cells j, j - 1
     }
     double ab = 0.0;
     if constexpr (!WIDE) {
         // one thread per (interface, field k): the field's projection, both reconstructions
         // and their reverse; the fields' results meet in shared memory
-        if (live) {
+        if (live && !lin) {
             double L0, L1, L2, R1, R2;
             field_lr(k, ut, Ht, c, rc, b1, b2, L0, L1, L2, R1, R2);
             double fp[5], fm[5], fpb[5], fmb[5];
@@ -552,7 +591,24 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
 #pragma unroll
         for (int f = 0; f < 3; ++f)
 #pragma unroll
-            for (int m = 0; m < 3; ++m) hL[f][m] = live ? sm.red[f][10 + m][i] : 0.0;
+            for (int m = 0; m < 3; ++m) hL[f][m] = live && !lin ? sm.red[f][10 + m][i] : 0.0;
+        if (lin) {
+            // (hbar+ + hbar-)/2 = (2, -16, 74, 74, -16, 2)/120 Fb, (hbar+ - hbar-)/2 = (2, -10, 20,
+            // -20, 10, -2)/120 Fb at positions 0..5: this thread's are 2k and 2k + 1
+            const double f0 = k == 0 ? 2.0 / 120.0 : (k == 1 ? 74.0 / 120.0 : -16.0 / 120.0);
+            const double f1 = k == 0 ? -16.0 / 120.0 : (k == 1 ? 74.0 / 120.0 : 2.0 / 120.0);
+            const double d0 = k == 0 ? 2.0 / 120.0 : (k == 1 ? 20.0 / 120.0 : 10.0 / 120.0);
+            const double d1 = k == 0 ? -10.0 / 120.0 : (k == 1 ? -20.0 / 120.0 : -2.0 / 120.0);
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const double e0 = d0 * Fb[m], e1 = d1 * Fb[m];
+                S.cF[2 * k][m][i] = f0 * Fb[m];
+                S.cF[2 * k + 1][m][i] = f1 * Fb[m];
+                S.cD[2 * k][m][i] = e0;
+                S.cD[2 * k + 1][m][i] = e1;
+                if (owned) ab = fma(sm.U[m][i + 2 * k + 1], e1, fma(sm.U[m][i + 2 * k], e0, ab));
+            }
+        } else
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int s = 2 * k + t;
@@ -579,7 +635,7 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         if (k > 0) {
             // the Roe average reversed: warp 1 gives the left cell, warp 2 the right
             double Ub[3] = {0.0, 0.0, 0.0};
-            if (live) {
+            if (live && !lin) {
                 double sc[6];
 #pragma unroll
                 for (int q = 0; q < 6; ++q) sc[q] = (sm.red[0][13 + q][i] + sm.red[1][13 + q][i]) + sm.red[2][13 + q][i];
@@ -598,7 +654,7 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         for (int s = 0; s < 5; ++s)
 #pragma unroll
             for (int m = 0; m < 3; ++m) hpb[s][m] = hmb[s][m] = 0.0;
-        if (live) {
+        if (live && !lin) {
 #pragma unroll 1
             for (int kf = 0; kf < 3; ++kf) {
                 double L0, L1, L2, R1, R2;
@@ -631,6 +687,20 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
             }
         }
         // stencil positions 0..5, as above
+        if (lin) {
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const double f[3] = {(2.0 / 120.0) * Fb[m], (-16.0 / 120.0) * Fb[m], (74.0 / 120.0) * Fb[m]};
+                const double d[3] = {f[0], (-10.0 / 120.0) * Fb[m], (20.0 / 120.0) * Fb[m]};
+#pragma unroll
+                for (int s = 0; s < 3; ++s) {
+                    S.cF[s][m][i] = S.cF[5 - s][m][i] = f[s];
+                    S.cD[s][m][i] = d[s];
+                    S.cD[5 - s][m][i] = -d[s];
+                    if (owned) ab = fma(sm.U[m][i + s] - sm.U[m][i + 5 - s], d[s], ab);
+                }
+            }
+        } else
 #pragma unroll
         for (int s = 0; s < 6; ++s)
 #pragma unroll
@@ -643,7 +713,7 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
             }
         // the Roe average reversed to both input cells
         double Ul[3] = {0.0, 0.0, 0.0}, Ur[3] = {0.0, 0.0, 0.0};
-        if (live) {
+        if (live && !lin) {
             roe_reverse_cell(sc, ut, Ht, rc, b1, rS, gm1, a.gamma, wl, sm.u[cl], sm.H[cl], sm.r[cl], sm.sq[cl], Ul);
             roe_reverse_cell(sc, ut, Ht, rc, b1, rS, gm1, a.gamma, wr, sm.u[cr], sm.H[cr], sm.r[cr], sm.sq[cr], Ur);
         }

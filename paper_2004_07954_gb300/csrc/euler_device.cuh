@@ -47,18 +47,21 @@ struct CellPlanes {
 // per cell: the characteristic projection is linear, so the reconstructions' stencil
 // differences are projections of these (no cell difference is formed per interface and field).
 template <int NV>
+__device__ __forceinline__ void cell_diffs_side(const CellPlanes<NV>& s, int si, int stride, int side) {
+    const double* h = side == 0 ? s.hp : s.hm;
+    int64_t* d = side == 0 ? s.dp : s.dm;
+    int e[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        d[k * s.NC + si] = wide_unpack(h[k * s.NC + si] - h[k * s.NC + si + stride], e[k]);
+    s.ex[2 * side * s.NC + si] = uint32_t(e[0] | (e[1] << 16));
+    s.ex[(2 * side + 1) * s.NC + si] = uint32_t(e[2] | (e[3] << 16));
+}
+
+template <int NV>
 __device__ __forceinline__ void cell_diffs(const CellPlanes<NV>& s, int si, int stride) {
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        const double* h = side == 0 ? s.hp : s.hm;
-        int64_t* d = side == 0 ? s.dp : s.dm;
-        int e[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-            d[k * s.NC + si] = wide_unpack(h[k * s.NC + si] - h[k * s.NC + si + stride], e[k]);
-        s.ex[2 * side * s.NC + si] = uint32_t(e[0] | (e[1] << 16));
-        s.ex[(2 * side + 1) * s.NC + si] = uint32_t(e[2] | (e[3] << 16));
-    }
+    for (int side = 0; side < 2; ++side) cell_diffs_side<NV>(s, si, stride, side);
 }
 
 // 1/sqrt(x) in integer arithmetic (correctly rounded but for 0.6 % of a last place), CUDA's where
@@ -218,6 +221,7 @@ __device__ __forceinline__ void split_cell_gen(const double* Uc, int split, doub
 template <int NV>
 struct RoeState {
     double u, v, H, c, hrc, hq2, hb1, hb2;   // hrc = 1/(2c), hq2 = q^2/2, hb1 = b1/2, hb2 = b2/2
+    RoeState() = default;
     __device__ __forceinline__ RoeState(const CellPlanes<NV>& s, int cl, int cr, double gm1) {
         const double srl = s.sr[cl];
         const double wl = srl * wide_reciprocal(srl + s.sr[cr]);
@@ -305,6 +309,7 @@ struct WideProjection {
     // coefficients of h_0 (and of h_1) in Z/2 and B share an exponent
     Limbs z0, z1, z2, zE, p0, p1, w0;
     int e0, e1, e2, eE, ew;
+    __device__ __forceinline__ WideProjection() : z0(0), z1(0), z2(0), zE(0), p0(0), p1(0), w0(0), e0(0), e1(0), e2(0), eE(0), ew(0) {}
     __device__ __forceinline__ explicit WideProjection(const RoeState<NV>& R)
         : z0(0), z1(0), z2(0), zE(0), p0(0), p1(0), w0(0), e2(0), ew(0) {
         int a, b;
@@ -392,168 +397,200 @@ struct FieldMagnitudes {                     // sums of the projections' terms: 
     __device__ __forceinline__ float of(int k) const { return k == 0 || k == NV - 1 ? a : (k == 1 ? e : s); }
 };
 
+// The float evaluation behind it, for the fields k0 <= k < k1.  ADJ: whether the flux is the optimal
+// linear combination to rounding with all its first derivatives (the adjoint's use): Delta
+// below 2^-54 of the value and sum_i |d Delta / d D_i| below 2^-53, from
+//   |dr| <= r (2 |dQ/Q| + 2 |dT/T| + 2 |dh/h| + |db/b|), |dQ| <= 8, |dT| <= 100 F, |dh|, |db| <= 50 F
+// summed over the stencil, F its largest difference, in Delta's derivative 0.07 A |dr| + 2 r.
+template <int NV, bool ADJ>
+struct NearLinear {
+    int X[4], E;                               // the variables' exponents over both sides' vectors, the largest
+    int64_t S[NV];                             // 60 (lin(dh+) - lin(dh-)) per component, 2^(X_k - 1078)
+    float dl[NV];                              // 60 Delta of the fields, plus side - minus side, 2^(E - 1022)
+    float val[2];                              // 2^-57 of the fields' values in the same units
+    float u, v, H, c2, rc, hq2;
+    bool ok;
+
+    __device__ __forceinline__ NearLinear(const CellPlanes<NV>& s, int base, int stride, double gm1,
+                                          const WideConst& wc, int k0, int k1) {
+        const int NC = s.NC, cl = base + 2 * stride, cr = cl + stride;
+        // the variables' exponents over both sides' vectors
+        uint32_t xa = 0, xb = 0;
+#pragma unroll
+        for (int st = 0; st < 4; ++st) {
+            const int i = base + st * stride;
+            xa = __vimax3_u16x2(xa, s.ex[i], s.ex[2 * NC + i + stride]);
+            xb = __vimax3_u16x2(xb, s.ex[NC + i], s.ex[3 * NC + i + stride]);
+        }
+        X[0] = int(xa & 0xffffu);
+        X[1] = int(xa >> 16);
+        X[2] = int(xb & 0xffffu);
+        X[3] = int(xb >> 16);
+        E = max_i(max_i(X[0], X[1]), max_i(X[2], X[3]));
+        ok = E < kWideMaxExp;
+        // powers of two of the variables against the largest (0 for all-zero ones)
+        float sc[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int e = X[k] - E + 127;
+            sc[k] = bits_float(uint32_t(X[k] == 0 || e < 0 ? 0 : e) << 23);
+        }
+        // the Roe state in float
+        const float sl = wide_truncate(s.sr[cl]), wl = sl * float_rcp(sl + wide_truncate(s.sr[cr]));
+        const float ul = wide_truncate(s.un[cl]), ur = wide_truncate(s.un[cr]);
+        const float vl = NV == 4 ? wide_truncate(s.ut[cl]) : 0.0f, vr = NV == 4 ? wide_truncate(s.ut[cr]) : 0.0f;
+        const float Hl = wide_truncate(s.H[cl]), Hr = wide_truncate(s.H[cr]);
+        u = fmaf(wl, ul - ur, ur);
+        v = fmaf(wl, vl - vr, vr);
+        H = fmaf(wl, Hl - Hr, Hr);
+        const float um = fabsf(ul) + fabsf(ur), vm = fabsf(vl) + fabsf(vr);
+        const float g1 = wide_truncate(gm1);
+        hq2 = 0.5f * fmaf(u, u, v * v);
+        c2 = g1 * (H - hq2);
+        rc = rsqrtf(c2);
+        const float hrc = 0.5f * rc, hb1 = 0.5f * g1 * rc * rc, hb2 = hq2 * hb1;
+        const float rel = 0x1p-21f * fmaf(2.0f * hb1, fabsf(H), 4.0f);
+        // R in the units of the differences, 2^(E - 1022)
+        const int er = wc.eR - 57 - 2 * E;
+        const float R = wc.Rf * bits_float(uint32_t((er < -126 ? -126 : (er > 60 ? 60 : er)) + 127) << 23);
+        const int e0 = max_i(exponent_of(s.hp[cl]), exponent_of(s.hm[cr]));
+        const int ew = NV == 4 ? max_i(exponent_of(s.hp[2 * NC + cl]), exponent_of(s.ut[cl]) + e0 - 1024) : 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int ef = (q == 0 ? e0 - 2 : ew) - E + 126;
+            val[q] = 0x1p-57f * bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
+        }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            S[k] = 0;
+            dl[k] = 0.0f;
+        }
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const int64_t* pl = side == 0 ? s.dp : s.dm;
+            const uint32_t* ex = s.ex + 2 * side * NC;
+            const int step = side == 0 ? stride : -stride;
+            const int i0 = side == 0 ? base : base + 4 * stride;
+            // the vectors D2, D2 - D3, delta_0, delta_1 (floats, variable units against 2^E)
+            float w[4][NV];
+            uint32_t da[4], db[4];
+#pragma unroll
+            for (int st = 0; st < 4; ++st) {
+                da[st] = xa - ex[i0 + st * step];
+                db[st] = xb - ex[NC + i0 + st * step];
+            }
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                int64_t x[4];
+#pragma unroll
+                for (int st = 0; st < 4; ++st) {
+                    const uint32_t d = k < 2 ? da[st] : db[st];
+                    x[st] = shr_s64(pl[k * NC + i0 + st * step], int((k & 1) ? d >> 16 : d & 0xffffu) + 4);
+                }
+                const int64_t t = 2 * x[0] - 11 * x[1] - 24 * x[2] + 3 * x[3];
+                S[k] += side == 0 ? t : -t;
+                const int64_t s1 = x[1] - x[2], d0 = (x[0] - x[1]) - s1, d1 = s1 - (x[2] - x[3]);
+                w[0][k] = wide_float(x[1]) * sc[k];
+                w[1][k] = wide_float(s1) * sc[k];
+                w[2][k] = wide_float(d0) * sc[k];
+                w[3][k] = wide_float(d1) * sc[k];
+            }
+            float P[4][NV];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float* h = w[q];
+                const float W = fmaf(u, h[1], NV == 4 ? fmaf(v, h[2], -h[NV - 1]) : -h[NV - 1]);
+                const float Z = fmaf(hb2, h[0], -(hb1 * W)), B = hrc * fmaf(u, h[0], -h[1]);
+                P[q][0] = Z + B;
+                P[q][NV - 1] = Z - B;
+                P[q][1] = fmaf(-2.0f, Z, h[0]);
+                if (NV == 4) P[q][2] = fmaf(-v, h[0], h[2]);
+            }
+            // magnitudes of the projections' terms, of D2 and D3 and of the delta's
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                w[0][k] = 2.0f * fabsf(w[0][k]) + fabsf(w[1][k]);
+                w[2][k] = fabsf(w[2][k]) + fabsf(w[3][k]);
+            }
+            const FieldMagnitudes<NV> Mf(w[0], hb1, hrc, um, vm), Md(w[2], hb1, hrc, um, vm);
+            // (a rolled loop: the code of the interface phases is larger than the instruction cache's
+            // first level as it is)
+#pragma unroll 1
+            for (int k = k0; k < k1; ++k) {
+                float f2 = P[0][0], s1 = P[1][0], d0 = P[2][0], d1 = P[3][0];
+#pragma unroll
+                for (int m = 1; m < NV; ++m) {
+                    f2 = k == m ? P[0][m] : f2;
+                    s1 = k == m ? P[1][m] : s1;
+                    d0 = k == m ? P[2][m] : d0;
+                    d1 = k == m ? P[3][m] : d1;
+                }
+                const float f3 = f2 - s1, s0 = s1 + d0, s2 = s1 - d1, Q = d0 - d1;
+                const float A = fabsf(d0) + fabsf(d1), As = fabsf(s0) + fabsf(s2), Af = fabsf(f2) + fabsf(f3);
+                const float ef = rel * Mf.of(k), ed = fmaf(rel, Md.of(k), 0x1p-22f * A);
+                const float b0 = fmaf(4.0f * s0, s0, fmaf(3.0f * f2, f2 - s0, R)), b1 = fmaf(4.0f * s1, s1, fmaf(3.0f * f2, f3, R));
+                const float b2 = fmaf(4.0f * s2, s2, fmaf(3.0f * f3, f3 + s2, R));
+                const float T = fabsf(fmaf(4.0f * Q + 8.0f * d1, s0 + s2, 3.0f * fmaf(f3, d1, -(f2 * d0)))) + R;
+                const float ET = fmaf(ed, fmaf(8.0f, As + A, 6.0f * Af), 11.0f * A * ef);
+                // the b's smallest pair against the error of the differences in it
+                const float mn = fminf(fminf(fmaxf(fabsf(f2 + s0), fabsf(f2)), fmaxf(fabsf(f2), fabsf(f3))),
+                                       fmaxf(fabsf(f3), fabsf(f3 - s2)));
+                const float rho = 64.0f * ef * float_rcp(mn);                        // relative error of the b's
+                const float i0f = float_rcp(b0), i1f = float_rcp(b1), i2f = float_rcp(b2), im = fmaxf(fmaxf(i0f, i1f), i2f);
+                const float x = wc.Kf * float_rcp(fminf(b0, b2) - 0.5f * R);
+                const float q = x * Q * T, rr = q * q;
+                // r's error (x, im: b's and h to within rho < 1/8; d4 to within 2 ed)
+                const float qa = fabsf(q), qe = fabsf(x) * fmaf(fabsf(Q) + 2.0f * ed, ET, 2.0f * ed * T);
+                const float err = im * fmaf(qe, fmaf(2.0f, qa, qe), rr * fmaf(8.0f, rho, 0x1p-13f)) * 2.0f;
+                const float r0 = rr * i0f, r1 = 6.0f * rr * i1f, r2 = 3.0f * rr * i2f;
+                const float num = fmaf(r0, fmaf(18.0f, d0, -3.0f * d1),
+                                       fmaf(r1, fmaf(-2.0f, d0, -3.0f * d1), r2 * fmaf(-2.0f, d0, 7.0f * d1)));
+                const bool zero = Af + A == 0.0f && ef + ed == 0.0f;
+                const float del = zero ? 0.0f : num * float_rcp(10.0f + (r0 + r1 + r2));
+                // |error of Delta| <= 0.07 (A + 2 ed) min(err, 1) + rounding of Delta and of R Delta
+                const float bound = fmaf(0.125f * (A + 2.0f * ed), rho < 0.125f ? fminf(err, 1.0f) : 1.0f,
+                                         0x1p-22f * fabsf(del) + rel * fabsf(del));
+                const float vk = NV == 4 && k == 2 ? val[1] : val[0];
+                ok = ok && (zero || bound <= vk);
+                if (ADJ) {
+                    const float xb = 2.0f * fabsf(x) * (T + ET), qb = xb * (fabsf(Q) + 2.0f * ed), rb = 2.0f * qb * qb * im;
+                    const float F = Af + As + A, B = 0.07f * A * im * (xb * qb * 32.0f + qb * qb * F * 400.0f * float_rcp(T + ET) +
+                                                                       rb * F * 300.0f) + 2.0f * rb;
+                    ok = ok && (zero || (rho < 0.125f && B <= 0x1p-53f && fabsf(del) <= 480.0f * vk));
+                }
+                const float sd = side == 0 ? del : -del;
+#pragma unroll
+                for (int m = 0; m < NV; ++m) dl[m] += k == m ? sd : 0.0f;
+            }
+        }
+    }
+};
+
 template <int NV>
 __device__ __forceinline__ bool interface_linear(const CellPlanes<NV>& s, int base, int stride, double gm1,
                                                  const WideConst& wc, double* Fh) {
+    const NearLinear<NV, false> L(s, base, stride, gm1, wc, 0, NV);
+    if (!L.ok) return false;
     const int NC = s.NC, cl = base + 2 * stride, cr = cl + stride;
-    // the variables' exponents over both sides' vectors
-    uint32_t xa = 0, xb = 0;
-#pragma unroll
-    for (int st = 0; st < 4; ++st) {
-        const int i = base + st * stride;
-        xa = __vimax3_u16x2(xa, s.ex[i], s.ex[2 * NC + i + stride]);
-        xb = __vimax3_u16x2(xb, s.ex[NC + i], s.ex[3 * NC + i + stride]);
-    }
-    const int X[4] = {int(xa & 0xffffu), int(xa >> 16), int(xb & 0xffffu), int(xb >> 16)};
-    const int E = max_i(max_i(X[0], X[1]), max_i(X[2], X[3]));
-    if (E >= kWideMaxExp) return false;
-    // powers of two of the variables against the largest (0 for all-zero ones)
-    float sc[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const int e = X[k] - E + 127;
-        sc[k] = bits_float(uint32_t(X[k] == 0 || e < 0 ? 0 : e) << 23);
-    }
-    // the Roe state in float
-    const float sl = wide_truncate(s.sr[cl]), wl = sl * float_rcp(sl + wide_truncate(s.sr[cr]));
-    const float ul = wide_truncate(s.un[cl]), ur = wide_truncate(s.un[cr]);
-    const float vl = NV == 4 ? wide_truncate(s.ut[cl]) : 0.0f, vr = NV == 4 ? wide_truncate(s.ut[cr]) : 0.0f;
-    const float Hl = wide_truncate(s.H[cl]), Hr = wide_truncate(s.H[cr]);
-    const float u = fmaf(wl, ul - ur, ur), v = fmaf(wl, vl - vr, vr), H = fmaf(wl, Hl - Hr, Hr);
-    const float um = fabsf(ul) + fabsf(ur), vm = fabsf(vl) + fabsf(vr);
-    const float g1 = wide_truncate(gm1), hq2 = 0.5f * fmaf(u, u, v * v), c2 = g1 * (H - hq2);
-    const float rc = rsqrtf(c2);
-    const float hrc = 0.5f * rc, hb1 = 0.5f * g1 * rc * rc, hb2 = hq2 * hb1;
-    const float rel = 0x1p-21f * fmaf(2.0f * hb1, fabsf(H), 4.0f);
-    // R in the units of the differences, 2^(E - 1022)
-    const int er = wc.eR - 57 - 2 * E;
-    const float R = wc.Rf * bits_float(uint32_t((er < -126 ? -126 : (er > 60 ? 60 : er)) + 127) << 23);
-    const int e0 = max_i(exponent_of(s.hp[cl]), exponent_of(s.hm[cr]));
-    const int ew = NV == 4 ? max_i(exponent_of(s.hp[2 * NC + cl]), exponent_of(s.ut[cl]) + e0 - 1024) : 0;
-    float val[2];                              // the fields' values (as in interface_flux) in the same units
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int ef = (q == 0 ? e0 - 2 : ew) - E + 126;
-        val[q] = 0x1p-57f * bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
-    }
-    int64_t S[NV];
-    float dl[NV];                              // 60 Delta of the fields, plus side - minus side
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        S[k] = 0;
-        dl[k] = 0.0f;
-    }
-    bool ok = true;
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-        const int64_t* pl = side == 0 ? s.dp : s.dm;
-        const uint32_t* ex = s.ex + 2 * side * NC;
-        const int step = side == 0 ? stride : -stride;
-        const int i0 = side == 0 ? base : base + 4 * stride;
-        // the vectors D2, D2 - D3, delta_0, delta_1 (floats, variable units against 2^E)
-        float w[4][NV];
-        uint32_t da[4], db[4];
-#pragma unroll
-        for (int st = 0; st < 4; ++st) {
-            da[st] = xa - ex[i0 + st * step];
-            db[st] = xb - ex[NC + i0 + st * step];
-        }
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            int64_t x[4];
-#pragma unroll
-            for (int st = 0; st < 4; ++st) {
-                const uint32_t d = k < 2 ? da[st] : db[st];
-                x[st] = shr_s64(pl[k * NC + i0 + st * step], int((k & 1) ? d >> 16 : d & 0xffffu) + 4);
-            }
-            const int64_t t = 2 * x[0] - 11 * x[1] - 24 * x[2] + 3 * x[3];
-            S[k] += side == 0 ? t : -t;
-            const int64_t s1 = x[1] - x[2], d0 = (x[0] - x[1]) - s1, d1 = s1 - (x[2] - x[3]);
-            w[0][k] = wide_float(x[1]) * sc[k];
-            w[1][k] = wide_float(s1) * sc[k];
-            w[2][k] = wide_float(d0) * sc[k];
-            w[3][k] = wide_float(d1) * sc[k];
-        }
-        float P[4][NV];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float* h = w[q];
-            const float W = fmaf(u, h[1], NV == 4 ? fmaf(v, h[2], -h[NV - 1]) : -h[NV - 1]);
-            const float Z = fmaf(hb2, h[0], -(hb1 * W)), B = hrc * fmaf(u, h[0], -h[1]);
-            P[q][0] = Z + B;
-            P[q][NV - 1] = Z - B;
-            P[q][1] = fmaf(-2.0f, Z, h[0]);
-            if (NV == 4) P[q][2] = fmaf(-v, h[0], h[2]);
-        }
-        // magnitudes of the projections' terms, of D2 and D3 and of the delta's
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            w[0][k] = 2.0f * fabsf(w[0][k]) + fabsf(w[1][k]);
-            w[2][k] = fabsf(w[2][k]) + fabsf(w[3][k]);
-        }
-        const FieldMagnitudes<NV> Mf(w[0], hb1, hrc, um, vm), Md(w[2], hb1, hrc, um, vm);
-        // (a rolled loop, the fields' values moving up by one each turn: the code of the interface
-        // phases is larger than the instruction cache's first level as it is)
-#pragma unroll 1
-        for (int k = 0; k < NV; ++k) {
-            const float f2 = P[0][0], s1 = P[1][0], d0 = P[2][0], d1 = P[3][0];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int m = 0; m + 1 < NV; ++m) P[q][m] = P[q][m + 1];
-            const float f3 = f2 - s1, s0 = s1 + d0, s2 = s1 - d1, Q = d0 - d1;
-            const float A = fabsf(d0) + fabsf(d1), As = fabsf(s0) + fabsf(s2), Af = fabsf(f2) + fabsf(f3);
-            const float ef = rel * Mf.of(k), ed = fmaf(rel, Md.of(k), 0x1p-22f * A);
-            const float b0 = fmaf(4.0f * s0, s0, fmaf(3.0f * f2, f2 - s0, R)), b1 = fmaf(4.0f * s1, s1, fmaf(3.0f * f2, f3, R));
-            const float b2 = fmaf(4.0f * s2, s2, fmaf(3.0f * f3, f3 + s2, R));
-            const float T = fabsf(fmaf(4.0f * Q + 8.0f * d1, s0 + s2, 3.0f * fmaf(f3, d1, -(f2 * d0)))) + R;
-            const float ET = fmaf(ed, fmaf(8.0f, As + A, 6.0f * Af), 11.0f * A * ef);
-            // the b's smallest pair against the error of the differences in it
-            const float mn = fminf(fminf(fmaxf(fabsf(f2 + s0), fabsf(f2)), fmaxf(fabsf(f2), fabsf(f3))),
-                                   fmaxf(fabsf(f3), fabsf(f3 - s2)));
-            const float rho = 64.0f * ef * float_rcp(mn);                        // relative error of the b's
-            const float i0f = float_rcp(b0), i1f = float_rcp(b1), i2f = float_rcp(b2), im = fmaxf(fmaxf(i0f, i1f), i2f);
-            const float x = wc.Kf * float_rcp(fminf(b0, b2) - 0.5f * R);
-            const float q = x * Q * T, rr = q * q;
-            // r's error (x, im: b's and h to within rho < 1/8; d4 to within 2 ed)
-            const float qa = fabsf(q), qe = fabsf(x) * fmaf(fabsf(Q) + 2.0f * ed, ET, 2.0f * ed * T);
-            const float err = im * fmaf(qe, fmaf(2.0f, qa, qe), rr * fmaf(8.0f, rho, 0x1p-13f)) * 2.0f;
-            const float r0 = rr * i0f, r1 = 6.0f * rr * i1f, r2 = 3.0f * rr * i2f;
-            const float num = fmaf(r0, fmaf(18.0f, d0, -3.0f * d1),
-                                   fmaf(r1, fmaf(-2.0f, d0, -3.0f * d1), r2 * fmaf(-2.0f, d0, 7.0f * d1)));
-            const bool zero = Af + A == 0.0f && ef + ed == 0.0f;
-            const float del = zero ? 0.0f : num * float_rcp(10.0f + (r0 + r1 + r2));
-            // |error of Delta| <= 0.07 (A + 2 ed) min(err, 1) + rounding of Delta and of R Delta
-            const float bound = fmaf(0.125f * (A + 2.0f * ed), rho < 0.125f ? fminf(err, 1.0f) : 1.0f,
-                                     0x1p-22f * fabsf(del) + rel * fabsf(del));
-            ok = ok && (zero || bound <= (NV == 4 && k == 2 ? val[1] : val[0]));
-            const float sd = side == 0 ? del : -del;
-            const float total = dl[0] + sd;
-#pragma unroll
-            for (int m = 0; m + 1 < NV; ++m) dl[m] = dl[m + 1];
-            dl[NV - 1] = total;
-        }
-    }
-    if (!ok) return false;
 #pragma unroll
     for (int k = 0; k < NV; ++k)
-        Fh[k] = (s.hp[k * NC + cl] + s.hm[k * NC + cr]) + (X[k] == 0 ? 0.0 : wide_sixtieth(S[k], X[k]));
+        Fh[k] = (s.hp[k * NC + cl] + s.hm[k * NC + cr]) + (L.X[k] == 0 ? 0.0 : wide_sixtieth(L.S[k], L.X[k]));
     // R Delta, where it reaches the last places of the fluxes
     bool add = false;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) add = add || fabsf(dl[k]) > 2.0f * val[NV == 4 && k == 2 ? 1 : 0];
+    for (int k = 0; k < NV; ++k) add = add || fabsf(L.dl[k]) > 2.0f * L.val[NV == 4 && k == 2 ? 1 : 0];
     if (add) {
-        const float c = c2 * rc, t = dl[0] + dl[NV - 1], d = dl[NV - 1] - dl[0], f = t + dl[1];
+        const float c = L.c2 * L.rc, t = L.dl[0] + L.dl[NV - 1], d = L.dl[NV - 1] - L.dl[0], f = t + L.dl[1];
         float dF[NV];
         dF[0] = f;
-        dF[1] = fmaf(u, f, c * d);
-        if (NV == 4) dF[2] = fmaf(v, f, dl[2]);
-        dF[NV - 1] = fmaf(H, t, fmaf(u * c, d, fmaf(hq2, dl[1], NV == 4 ? v * dl[2] : 0.0f)));
+        dF[1] = fmaf(L.u, f, c * d);
+        if (NV == 4) dF[2] = fmaf(L.v, f, L.dl[2]);
+        dF[NV - 1] = fmaf(L.H, t, fmaf(L.u * c, d, fmaf(L.hq2, L.dl[1], NV == 4 ? L.v * L.dl[2] : 0.0f)));
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             // dF 2^(E - 1022) / 60 as a double, from the bits of dF/60
             const uint32_t b = float_bits(dF[k] * (1.0f / 60.0f)), e = (b >> 23) & 0xffu;
-            if (e != 0) Fh[k] += bits_double(join((b & 0x80000000u) | (((b & 0x7fffffu) >> 3) + (uint32_t(int(e) + E - 126) << 20)), b << 29));
+            if (e != 0) Fh[k] += bits_double(join((b & 0x80000000u) | (((b & 0x7fffffu) >> 3) + (uint32_t(int(e) + L.E - 126) << 20)), b << 29));
         }
     }
     return true;

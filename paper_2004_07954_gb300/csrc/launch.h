@@ -134,6 +134,7 @@ struct VjpArgs {
     double c1, c2, c3, d;
     int n, bc;
     double rdx, gamma, eps4, kappa, adv_speed;
+    WideConst wide;                        // the weights' constants for the linear check (wide_weights.cuh)
     int rec_out;                           // the record this launch writes
     int prec[kVjpPend];                    // records with corrections pending on the inputs (-1: none)
     int lam_slot;                          // index into prec of lam's record (-1: none)

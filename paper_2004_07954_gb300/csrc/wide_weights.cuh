@@ -134,6 +134,7 @@ WZ_HD uint64_t sqr_hi(uint64_t a) {
 // x = h 2^32 + l with a signed low limb, so that products of limbs are signed 32 x 32 ones
 struct Limbs {
     int32_t h, l;
+    WZ_HD Limbs(int32_t high, int32_t low) : h(high), l(low) {}
     WZ_HD explicit Limbs(int64_t x) {
         const uint32_t lo = uint32_t(x);
         l = int32_t(lo);
@@ -471,8 +472,8 @@ WZ_HD double wide_sixtieth(int64_t S, int G) {
     const int nq = clz_u32(uint32_t(q >> 32) | 1u);
     q <<= nq;
     const uint64_t r = ((q >> 10) + 1) >> 1;
-    const uint32_t ex = uint32_t(G + 2 - nt - (up ? 32 : 0) - nq) << 20;
-    return bits_double(N == 0 ? 0 : r + join(ex | sign, 0));
+    const int ex = G + 2 - nt - (up ? 32 : 0) - nq;           // (below 0: below the normal range)
+    return bits_double(N == 0 || ex < 0 ? 0 : r + join((uint32_t(ex) << 20) | sign, 0));
 }
 
 // A double to float by truncation of its bits; not a number outside [2^-126, 2^127) but for 0.
