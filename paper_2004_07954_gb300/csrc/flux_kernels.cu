@@ -164,6 +164,111 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMAL
                                    DIR == 0 ? blockIdx.y : blockIdx.x, smem);
 }
 
+// Short 1D Euler lines: too few interfaces to fill the GPU, so the time of a launch is the time of
+// one thread's chain of instructions.  Six warps share 32 interfaces: after the cells, warp 0
+// forms the Roe states and the projection's coefficients while the others difference the
+// cells, then warp (side, field) reconstructs one part of one field for each interface, and
+// three warps write a flux component each.  A step at 200 and 8192 cells: 39 and 47 us against 59
+// and 62 us with a thread per interface (64-thread blocks).
+constexpr int kLineTI = 32, kLineThreads = 192;
+constexpr int kLineMax = 24576;            // cells; 16384: 51 against 62 us a step, 30000: 74 against 69
+
+template <int GEN>
+__global__ void __launch_bounds__(kLineThreads) flux_line_kernel(FluxArgs a) {
+    constexpr int TI = kLineTI, NC = TI + 5, W = GEN == 0 ? 0 : -1;
+    __shared__ double s_planes[NC * CellPlanes<3>::kPerCellDefault];
+    __shared__ double s_R[8][TI], s_g[2][3][TI];
+    __shared__ int s_P[13][TI];
+    __shared__ int s_bad[TI];
+    const CellPlanes<3> sp(s_planes, NC);
+    pdl_wait();
+    const int tid = threadIdx.x, w = tid >> 5, i = tid & 31;
+    const int j0 = blockIdx.x * TI, n = a.nx;
+    const int cl_used = min(TI, n + 1 - j0) + 5;
+    const double alpha = __longlong_as_double((long long)a.alpha_bits[0]), gm1 = a.gamma - 1.0;
+    if (tid < cl_used) {
+        const int gi = j0 - 3 + tid, g = ghost_src(gi, n, a.bc);
+        double Uc[3] = {a.U[g], a.U[n + g], a.U[2 * int64_t(n) + g]};
+        if (a.bc == 2 && ghost_mirrored(gi, n, a.bc)) Uc[1] = -Uc[1];   // wall mirror image
+        if (GEN != 0) split_cell_gen<3>(Uc, a.split, alpha, a.adv_speed, a.gamma, sp, tid);
+        else split_cell<3>(Uc, alpha, a.adv_speed, gm1, sp, tid);
+    }
+    __syncthreads();
+    const bool live = j0 + i <= n;
+    if (w == 0) {
+        s_bad[i] = 0;
+        if (live) {
+            const RoeState<3> R(sp, i + 2, i + 3, gm1);
+            const WideProjection<3> P(R);
+            const double r[8] = {R.u, R.v, R.H, R.c, R.hrc, R.hq2, R.hb1, R.hb2};
+            const int q[13] = {P.z0.h, P.z0.l, P.z1.h, P.z1.l, P.zE.h, P.zE.l, P.p0.h, P.p0.l, P.p1.h, P.p1.l, P.e0, P.e1, P.eE};
+#pragma unroll
+            for (int m = 0; m < 8; ++m) s_R[m][i] = r[m];
+#pragma unroll
+            for (int m = 0; m < 13; ++m) s_P[m][i] = q[m];
+        }
+    } else {
+        for (int c = tid - 32; c < 2 * (cl_used - 1); c += kLineThreads - 32) {
+            const int side = c >= cl_used - 1;
+            cell_diffs_side<3>(sp, side ? c - (cl_used - 1) : c, 1, side);
+        }
+    }
+    __syncthreads();
+    const int side = w / 3, k = w % 3;
+    if (live) {
+        WideProjection<3> P;
+        P.z0 = Limbs(s_P[0][i], s_P[1][i]);
+        P.z1 = Limbs(s_P[2][i], s_P[3][i]);
+        P.zE = Limbs(s_P[4][i], s_P[5][i]);
+        P.p0 = Limbs(s_P[6][i], s_P[7][i]);
+        P.p1 = Limbs(s_P[8][i], s_P[9][i]);
+        P.e0 = s_P[10][i];
+        P.e1 = s_P[11][i];
+        P.eE = s_P[12][i];
+        // (the scale of the field's value as in interface_flux)
+        const int eb = (GEN == 0 ? exponent_of(sp.hp[i + 2]) : max_i(exponent_of(sp.hp[i + 2]), exponent_of(sp.hm[i + 3]))) - 2;
+        int64_t D[4];
+        int G[4];
+        uint32_t xm = 0;
+#pragma unroll
+        for (int st = 0; st < 4; ++st) {
+            int64_t d[3];
+            int g[3];
+            P.apply(side == 0 ? sp.dp : sp.dm, sp.ex + 2 * side * NC, NC, side == 0 ? i + st : i + 4 - st, d, g, xm);
+            D[st] = k == 0 ? d[0] : (k == 1 ? d[1] : d[2]);
+            G[st] = k == 0 ? g[0] : (k == 1 ? g[1] : g[2]);
+        }
+        double corr;
+        const bool ok = wide_correction<W>(D[0], D[1], D[2], D[3], G[0], G[1], G[2], G[3], eb, a.wide, a.weights, corr);
+        if (!ok || (xm & 0xffffu) == 2047u || (xm >> 16) == 2047u) s_bad[i] = 1;
+        s_g[side][k][i] = corr;
+    }
+    __syncthreads();
+    if (live && w < 3) {
+        RoeState<3> R;
+        R.u = s_R[0][i];
+        R.v = s_R[1][i];
+        R.H = s_R[2][i];
+        R.c = s_R[3][i];
+        R.hrc = s_R[4][i];
+        R.hq2 = s_R[5][i];
+        R.hb1 = s_R[6][i];
+        R.hb2 = s_R[7][i];
+        double gh[3], hc[3], Fh[3];
+        if (s_bad[i]) {
+            field_fluxes_double<3, GEN>(sp, R, i, 1, a.eps4, a.kappa, GEN == 0 ? 0 : a.weights, nullptr, gh);
+        } else {
+#pragma unroll
+            for (int m = 0; m < 3; ++m) gh[m] = s_g[0][m][i] - s_g[1][m][i];
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) hc[m] = sp.hp[m * NC + i + 2] + sp.hm[m * NC + i + 3];
+        R.back_project(gh, hc, Fh);
+        const int64_t j = j0 + i;
+        a.Fout[w * int64_t(n + 1) + j] = w == 0 ? Fh[0] : (w == 1 ? Fh[1] : Fh[2]);
+    }
+}
+
 // Both sweeps of a 2D stage in one grid, so that they share one tail: blocks [0, nbx) take
 // the x tiles (along the sweep fastest, as flux_kernel<4, 0>), the others the y tiles
 // (across the sweep fastest, as flux_kernel<4, 1>).
@@ -247,6 +352,9 @@ cudaError_t launch_flux_t(int system, int dir, const FluxArgs& a, cudaStream_t s
         const bool small = big_tiles < 2 * sm_count_cached();
         if (system == 0)
             return small ? launch_one<1, 0, true, GEN, false>(a, s) : launch_one<1, 0, false, GEN, false>(a, s);
+        if constexpr (GEN != 2)
+            if (a.nx < kLineMax)
+                return launch_pdl(flux_line_kernel<GEN>, dim3(unsigned((a.nx + kLineTI) / kLineTI)), dim3(kLineThreads), 0, s, a);
         if (small) return launch_one<3, 0, true, GEN, false>(a, s);
         if constexpr (GEN != 2)
             if (takes_linear(a, a.nx)) return launch_one<3, 0, false, GEN, true>(a, s);
