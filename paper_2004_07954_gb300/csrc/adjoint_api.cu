@@ -172,8 +172,6 @@ wenozn_status wenozn_rk3_step_vjp(const wenozn_problem* p, const double* U, doub
     const double* stage_in[2] = {U, u1};
     double* stage_out[2] = {u1, u2};
     for (int stage = 0; stage < 2 && e == cudaSuccess; ++stage) {
-        e = launch_fluxes(*p, stage_in[stage], ctrl->alpha[stage], nullptr, fx, nullptr, s);
-        if (e != cudaSuccess) break;
         UpdateArgs u = update_args(*p, ctrl, fx, nullptr);
         u.mode = stage + 1;
         u.Us = stage_in[stage];
@@ -181,7 +179,7 @@ wenozn_status wenozn_rk3_step_vjp(const wenozn_problem* p, const double* U, doub
         u.out = stage_out[stage];
         u.next_slot = euler ? stage + 1 : -1;
         u.dt_fixed = dt;
-        e = launch_update(p->system, u, s);
+        e = launch_stage(*p, stage_in[stage], ctrl->alpha[stage], nullptr, fx, nullptr, u, s);
     }
     if (e != cudaSuccess) return WENOZN_ECUDA;
     const unsigned long long* a = &ctrl->alpha[0][0];
@@ -235,8 +233,6 @@ wenozn_status wenozn_rk3_run_keep(const wenozn_problem* p, double* X, double* S1
         const double* in[3] = {Xk, S1 + k * ns, S2 + k * ns};
         double* out[3] = {S1 + k * ns, S2 + k * ns, Xk + ns};
         for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage) {
-            e = launch_fluxes(*p, in[stage], A + 3 * k + stage, nullptr, fx, nullptr, s);
-            if (e != cudaSuccess) break;
             UpdateArgs u = update_args(*p, ctrl, fx, nullptr);
             u.mode = stage + 1;
             u.Us = in[stage];
@@ -244,7 +240,7 @@ wenozn_status wenozn_rk3_run_keep(const wenozn_problem* p, double* X, double* S1
             u.out = out[stage];
             u.alpha_next = p->system != WENOZN_ADVECTION_1D ? A + 3 * k + stage + 1 : nullptr;
             u.dt_fixed = dt;
-            e = launch_update(p->system, u, s);
+            e = launch_stage(*p, in[stage], A + 3 * k + stage, nullptr, fx, nullptr, u, s);
         }
     }
     return cuda_status(e);

@@ -42,8 +42,6 @@ cudaError_t rk3_stages(const wenozn_problem& p, const Layout& lay, void* ws, con
     const double* stage_in[3] = {U, u1, u2};
     double* stage_out[3] = {u1, u2, U_out};
     for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage) {
-        e = launch_fluxes(p, stage_in[stage], ctrl->alpha[stage], &ctrl->alpha_f[stage][0][0], fx, gy, s);
-        if (e != cudaSuccess) break;
         UpdateArgs u = update_args(p, ctrl, fx, gy);
         u.mode = stage + 1;
         u.Us = stage_in[stage];
@@ -52,7 +50,7 @@ cudaError_t rk3_stages(const wenozn_problem& p, const Layout& lay, void* ws, con
         u.next_slot = (euler && stage < 2) ? stage + 1 : -1;
         u.dt_fixed = dt;
         u.t_remaining = t_remaining;
-        e = launch_update(p.system, u, s);
+        e = launch_stage(p, stage_in[stage], ctrl->alpha[stage], &ctrl->alpha_f[stage][0][0], fx, gy, u, s);
     }
     return e;
 }
@@ -179,12 +177,11 @@ wenozn_status wenozn_rhs(const wenozn_problem* p, const double* U, double* L, vo
     if (e == cudaSuccess)
         e = launch_max_wavespeed(p->system, U, int64_t(p->nx) * p->ny, p->gamma, p->adv_speed,
                                  ctrl->alpha[0], &ctrl->status, s, field_slot(*p, ctrl, 0));
-    if (e == cudaSuccess) e = launch_fluxes(*p, U, ctrl->alpha[0], &ctrl->alpha_f[0][0][0], fx, gy, s);
     if (e == cudaSuccess) {
         UpdateArgs u = update_args(*p, ctrl, fx, gy);
         u.mode = 0;
         u.out = L;
-        e = launch_update(p->system, u, s);
+        e = launch_stage(*p, U, ctrl->alpha[0], &ctrl->alpha_f[0][0][0], fx, gy, u, s);
     }
     note_status(stream, &ctrl->status);
     return cuda_status(e);
@@ -340,8 +337,6 @@ wenozn_status wenozn_rk3_run(const wenozn_problem* p, double* U, int64_t nsteps,
     double* stage_out[3] = {u1, u2, U};
     for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
         for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage) {
-            e = launch_fluxes(*p, stage_in[stage], ctrl->alpha[stage], &ctrl->alpha_f[stage][0][0], fx, gy, s);
-            if (e != cudaSuccess) break;
             UpdateArgs u = update_args(*p, ctrl, fx, gy);
             u.mode = stage + 1;
             u.Us = stage_in[stage];
@@ -350,7 +345,7 @@ wenozn_status wenozn_rk3_run(const wenozn_problem* p, double* U, int64_t nsteps,
             u.next_slot = euler ? (stage + 1) % 3 : -1;
             u.clear_slot = euler ? (stage + 2) % 3 : -1;
             u.dt_fixed = dt;
-            e = launch_update(p->system, u, s);
+            e = launch_stage(*p, stage_in[stage], ctrl->alpha[stage], &ctrl->alpha_f[stage][0][0], fx, gy, u, s);
         }
     }
     return cuda_status(e);

@@ -15,6 +15,7 @@
 
 #include "euler_device.cuh"
 #include "launch.h"
+#include "step_device.cuh"
 
 namespace wz {
 
@@ -164,108 +165,195 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMAL
                                    DIR == 0 ? blockIdx.y : blockIdx.x, smem);
 }
 
-// Short 1D Euler lines: too few interfaces to fill the GPU, so the time of a launch is the time of
-// one thread's chain of instructions.  Six warps share 32 interfaces: after the cells, warp 0
-// forms the Roe states and the projection's coefficients while the others difference the
-// cells, then warp (side, field) reconstructs one part of one field for each interface, and
-// three warps write a flux component each.  A step at 200 and 8192 cells: 39 and 47 us against 59
-// and 62 us with a thread per interface (64-thread blocks).
-constexpr int kLineTI = 32, kLineThreads = 192;
+// Short 1D lines: too few interfaces to fill the GPU, so the time of a launch is the time of one
+// thread's chain of instructions, and the launches themselves.  Euler: six warps share 32
+// interfaces; after the cells, warp 0 forms the Roe states and the projection's coefficients
+// while the others difference the cells, then warp (side, field) reconstructs one part of
+// one field for each interface, and three warps form a flux component each.  Advection: a warp
+// per part.  STAGE: the block goes on to the stage update of the cells between its
+// interfaces (31 of them: neighbouring blocks both compute the interface they share) and
+// their LF speeds, in the arithmetic of update_kernel, so that a stage is one launch.
+// A CFL step at 200 and 8192 cells: 59 and 62 us with a thread per interface (64-thread blocks) and
+// an update launch, 39 and 47 us with
+// this flux kernel and the update launch, 30 and 32 us as one; advection at 160 cells 13 -> 8.5 us.
+constexpr int kLineTI = 32;
 constexpr int kLineMax = 24576;            // cells; 16384: 51 against 62 us a step, 30000: 74 against 69
+template <int NV> constexpr int kLineThreads = NV == 3 ? 192 : 64;
 
-template <int GEN>
-__global__ void __launch_bounds__(kLineThreads) flux_line_kernel(FluxArgs a) {
-    constexpr int TI = kLineTI, NC = TI + 5, W = GEN == 0 ? 0 : -1;
-    __shared__ double s_planes[NC * CellPlanes<3>::kPerCellDefault];
-    __shared__ double s_R[8][TI], s_g[2][3][TI];
-    __shared__ int s_P[13][TI];
+template <int NV, int GEN, bool STAGE>
+__global__ void __launch_bounds__(kLineThreads<NV>) line_kernel(FluxArgs a, UpdateArgs u) {
+    constexpr int TI = kLineTI, NC = TI + 5, W = GEN == 0 ? 0 : -1, kThreads = kLineThreads<NV>;
+    __shared__ double s_planes[NC * CellPlanes<NV>::kPerCellDefault];
+    __shared__ double s_R[NV == 3 ? 8 : 1][TI], s_g[2][NV][TI];
+    __shared__ int s_P[NV == 3 ? 13 : 1][TI];
     __shared__ int s_bad[TI];
-    const CellPlanes<3> sp(s_planes, NC);
+    __shared__ double s_F[STAGE ? NV : 1][TI], s_dt;
+    const CellPlanes<NV> sp(s_planes, NC);
     pdl_wait();
     const int tid = threadIdx.x, w = tid >> 5, i = tid & 31;
-    const int j0 = blockIdx.x * TI, n = a.nx;
+    const int j0 = blockIdx.x * (STAGE ? TI - 1 : TI), n = a.nx;
     const int cl_used = min(TI, n + 1 - j0) + 5;
-    const double alpha = __longlong_as_double((long long)a.alpha_bits[0]), gm1 = a.gamma - 1.0;
+    const double alpha = NV == 1 ? fabs(a.adv_speed) : __longlong_as_double((long long)a.alpha_bits[0]);
+    const double gm1 = a.gamma - 1.0;
+    // the update's own inputs: component w of cell j0 + i
+    const bool mine = STAGE && w < NV && i < TI - 1 && j0 + i < n;
+    double us = 0.0, un = 0.0;
+    if (mine && u.mode != 0) {
+        us = u.Us[w * int64_t(n) + j0 + i];
+        if (u.mode > 1) un = u.Un[w * int64_t(n) + j0 + i];
+    }
     if (tid < cl_used) {
         const int gi = j0 - 3 + tid, g = ghost_src(gi, n, a.bc);
-        double Uc[3] = {a.U[g], a.U[n + g], a.U[2 * int64_t(n) + g]};
-        if (a.bc == 2 && ghost_mirrored(gi, n, a.bc)) Uc[1] = -Uc[1];   // wall mirror image
-        if (GEN != 0) split_cell_gen<3>(Uc, a.split, alpha, a.adv_speed, a.gamma, sp, tid);
-        else split_cell<3>(Uc, alpha, a.adv_speed, gm1, sp, tid);
+        double Uc[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) Uc[k] = a.U[k * int64_t(n) + g];
+        if (NV > 1 && a.bc == 2 && ghost_mirrored(gi, n, a.bc)) Uc[1] = -Uc[1];   // wall mirror image
+        if (GEN != 0) split_cell_gen<NV>(Uc, a.split, alpha, a.adv_speed, a.gamma, sp, tid);
+        else split_cell<NV>(Uc, alpha, a.adv_speed, gm1, sp, tid);
+    }
+    if (STAGE && tid == kThreads - 1) {
+        double dt = 0.0;
+        if (u.mode == 1) {
+            dt = step_dt(u, NV == 1 ? 0 : 1);
+            if (blockIdx.x == 0) u.ctrl->dt = dt;
+        } else if (u.mode > 1) {
+            dt = u.ctrl->dt;
+        }
+        s_dt = dt;
     }
     __syncthreads();
     const bool live = j0 + i <= n;
-    if (w == 0) {
-        s_bad[i] = 0;
+    double Fw = 0.0;                           // flux component w of interface i
+    if constexpr (NV == 1) {
         if (live) {
-            const RoeState<3> R(sp, i + 2, i + 3, gm1);
-            const WideProjection<3> P(R);
-            const double r[8] = {R.u, R.v, R.H, R.c, R.hrc, R.hq2, R.hb1, R.hb2};
-            const int q[13] = {P.z0.h, P.z0.l, P.z1.h, P.z1.l, P.zE.h, P.zE.l, P.p0.h, P.p0.l, P.p1.h, P.p1.l, P.e0, P.e1, P.eE};
-#pragma unroll
-            for (int m = 0; m < 8; ++m) s_R[m][i] = r[m];
-#pragma unroll
-            for (int m = 0; m < 13; ++m) s_P[m][i] = q[m];
+            const double* h = w == 0 ? sp.hp : sp.hm;
+            const int o = w == 0 ? i : i + 5, d = w == 0 ? 1 : -1;
+            const double h0 = h[o], h1 = h[o + d], h2 = h[o + 2 * d], h3 = h[o + 3 * d], h4 = h[o + 4 * d];
+            s_g[w][0][i] = zn_flux_wide<W>(h0 - h1, h1 - h2, h2 - h3, h3 - h4, h2, a.wide, a.eps4, a.kappa,
+                                           GEN == 0 ? 0 : a.weights);
         }
+        __syncthreads();
+        if (w == 0) Fw = s_g[0][0][i] + s_g[1][0][i];
     } else {
-        for (int c = tid - 32; c < 2 * (cl_used - 1); c += kLineThreads - 32) {
-            const int side = c >= cl_used - 1;
-            cell_diffs_side<3>(sp, side ? c - (cl_used - 1) : c, 1, side);
-        }
-    }
-    __syncthreads();
-    const int side = w / 3, k = w % 3;
-    if (live) {
-        WideProjection<3> P;
-        P.z0 = Limbs(s_P[0][i], s_P[1][i]);
-        P.z1 = Limbs(s_P[2][i], s_P[3][i]);
-        P.zE = Limbs(s_P[4][i], s_P[5][i]);
-        P.p0 = Limbs(s_P[6][i], s_P[7][i]);
-        P.p1 = Limbs(s_P[8][i], s_P[9][i]);
-        P.e0 = s_P[10][i];
-        P.e1 = s_P[11][i];
-        P.eE = s_P[12][i];
-        // (the scale of the field's value as in interface_flux)
-        const int eb = (GEN == 0 ? exponent_of(sp.hp[i + 2]) : max_i(exponent_of(sp.hp[i + 2]), exponent_of(sp.hm[i + 3]))) - 2;
-        int64_t D[4];
-        int G[4];
-        uint32_t xm = 0;
+        if (w == 0) {
+            s_bad[i] = 0;
+            if (live) {
+                const RoeState<3> R(sp, i + 2, i + 3, gm1);
+                const WideProjection<3> P(R);
+                const double r[8] = {R.u, R.v, R.H, R.c, R.hrc, R.hq2, R.hb1, R.hb2};
+                const int q[13] = {P.z0.h, P.z0.l, P.z1.h, P.z1.l, P.zE.h, P.zE.l, P.p0.h, P.p0.l, P.p1.h, P.p1.l, P.e0, P.e1, P.eE};
 #pragma unroll
-        for (int st = 0; st < 4; ++st) {
-            int64_t d[3];
-            int g[3];
-            P.apply(side == 0 ? sp.dp : sp.dm, sp.ex + 2 * side * NC, NC, side == 0 ? i + st : i + 4 - st, d, g, xm);
-            D[st] = k == 0 ? d[0] : (k == 1 ? d[1] : d[2]);
-            G[st] = k == 0 ? g[0] : (k == 1 ? g[1] : g[2]);
-        }
-        double corr;
-        const bool ok = wide_correction<W>(D[0], D[1], D[2], D[3], G[0], G[1], G[2], G[3], eb, a.wide, a.weights, corr);
-        if (!ok || (xm & 0xffffu) == 2047u || (xm >> 16) == 2047u) s_bad[i] = 1;
-        s_g[side][k][i] = corr;
-    }
-    __syncthreads();
-    if (live && w < 3) {
-        RoeState<3> R;
-        R.u = s_R[0][i];
-        R.v = s_R[1][i];
-        R.H = s_R[2][i];
-        R.c = s_R[3][i];
-        R.hrc = s_R[4][i];
-        R.hq2 = s_R[5][i];
-        R.hb1 = s_R[6][i];
-        R.hb2 = s_R[7][i];
-        double gh[3], hc[3], Fh[3];
-        if (s_bad[i]) {
-            field_fluxes_double<3, GEN>(sp, R, i, 1, a.eps4, a.kappa, GEN == 0 ? 0 : a.weights, nullptr, gh);
+                for (int m = 0; m < 8; ++m) s_R[m][i] = r[m];
+#pragma unroll
+                for (int m = 0; m < 13; ++m) s_P[m][i] = q[m];
+            }
         } else {
-#pragma unroll
-            for (int m = 0; m < 3; ++m) gh[m] = s_g[0][m][i] - s_g[1][m][i];
+            for (int c = tid - 32; c < 2 * (cl_used - 1); c += kThreads - 32) {
+                const int side = c >= cl_used - 1;
+                cell_diffs_side<NV>(sp, side ? c - (cl_used - 1) : c, 1, side);
+            }
         }
+        __syncthreads();
+        const int side = w / 3, k = w % 3;
+        if (live) {
+            WideProjection<3> P;
+            P.z0 = Limbs(s_P[0][i], s_P[1][i]);
+            P.z1 = Limbs(s_P[2][i], s_P[3][i]);
+            P.zE = Limbs(s_P[4][i], s_P[5][i]);
+            P.p0 = Limbs(s_P[6][i], s_P[7][i]);
+            P.p1 = Limbs(s_P[8][i], s_P[9][i]);
+            P.e0 = s_P[10][i];
+            P.e1 = s_P[11][i];
+            P.eE = s_P[12][i];
+            // (the scale of the field's value as in interface_flux)
+            const int eb = (GEN == 0 ? exponent_of(sp.hp[i + 2]) : max_i(exponent_of(sp.hp[i + 2]), exponent_of(sp.hm[i + 3]))) - 2;
+            int64_t D[4];
+            int G[4];
+            uint32_t xm = 0;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) hc[m] = sp.hp[m * NC + i + 2] + sp.hm[m * NC + i + 3];
-        R.back_project(gh, hc, Fh);
-        const int64_t j = j0 + i;
-        a.Fout[w * int64_t(n + 1) + j] = w == 0 ? Fh[0] : (w == 1 ? Fh[1] : Fh[2]);
+            for (int st = 0; st < 4; ++st) {
+                int64_t d[3];
+                int g[3];
+                P.apply(side == 0 ? sp.dp : sp.dm, sp.ex + 2 * side * NC, NC, side == 0 ? i + st : i + 4 - st, d, g, xm);
+                D[st] = k == 0 ? d[0] : (k == 1 ? d[1] : d[2]);
+                G[st] = k == 0 ? g[0] : (k == 1 ? g[1] : g[2]);
+            }
+            double corr;
+            const bool ok = wide_correction<W>(D[0], D[1], D[2], D[3], G[0], G[1], G[2], G[3], eb, a.wide, a.weights, corr);
+            if (!ok || (xm & 0xffffu) == 2047u || (xm >> 16) == 2047u) s_bad[i] = 1;
+            s_g[side][k][i] = corr;
+        }
+        __syncthreads();
+        if (live && w < 3) {
+            RoeState<3> R;
+            R.u = s_R[0][i];
+            R.v = s_R[1][i];
+            R.H = s_R[2][i];
+            R.c = s_R[3][i];
+            R.hrc = s_R[4][i];
+            R.hq2 = s_R[5][i];
+            R.hb1 = s_R[6][i];
+            R.hb2 = s_R[7][i];
+            double gh[3], hc[3], Fh[3];
+            if (s_bad[i]) {
+                field_fluxes_double<3, GEN>(sp, R, i, 1, a.eps4, a.kappa, GEN == 0 ? 0 : a.weights, nullptr, gh);
+            } else {
+#pragma unroll
+                for (int m = 0; m < 3; ++m) gh[m] = s_g[0][m][i] - s_g[1][m][i];
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) hc[m] = sp.hp[m * NC + i + 2] + sp.hm[m * NC + i + 3];
+            R.back_project(gh, hc, Fh);
+            Fw = w == 0 ? Fh[0] : (w == 1 ? Fh[1] : Fh[2]);
+        }
+    }
+    if (!STAGE) {
+        if (live && w < NV) a.Fout[w * int64_t(n + 1) + j0 + i] = Fw;
+        return;
+    }
+    if (w < NV) s_F[w][i] = Fw;
+    __syncthreads();
+    // the stage update, as update_kernel
+    bool bad = false;
+    double r = 0.0;
+    if (mine) {
+        const double dF = s_F[w][i + 1] - s_F[w][i];
+        if (u.mode == 0) {
+            r = -(dF * u.rdx);
+            bad = (__double2hiint(r) & 0x7ff00000) == 0x7ff00000;
+        } else {
+            const double wk = u.mode == 1 ? 1.0 : (u.mode == 2 ? 0.25 : 2.0 / 3.0);
+            const double kx = wk * s_dt * u.rdx;
+            double base = us;
+            if (u.mode == 2) base = fma(0.75, un, 0.25 * us);
+            else if (u.mode == 3) base = fma(1.0 / 3.0, un, (2.0 / 3.0) * us);
+            r = fma(-kx, dF, base);
+            if (NV == 1) bad = !isfinite(r);
+        }
+        u.out[w * int64_t(n) + j0 + i] = r;
+    }
+    if (NV == 3 && u.mode != 0 && (u.next_slot >= 0 || u.alpha_next || u.mode == 3)) {
+        // (s_g is free since the last barrier but one)
+        if (w < NV) s_g[0][w][i] = r;
+        __syncthreads();
+        if (w == 0) {
+            double sx = 0.0;
+            if (mine) {
+                const double st[3] = {s_g[0][0][i], s_g[0][1][i], s_g[0][2][i]};
+                double uu, vv, c;
+                const bool adm = wave_state<3>(st, u.gamma, uu, vv, c);
+                sx = __dadd_rn(fabs(uu), c);
+                bad = !(adm && isfinite(sx));
+            }
+            const double mx = warp_max(fmax(0.0, sx));
+            unsigned long long* dst = u.alpha_next ? u.alpha_next : (u.next_slot >= 0 ? u.ctrl->alpha[u.next_slot] : nullptr);
+            if (i == 0 && dst) atomicMax(dst, (unsigned long long)__double_as_longlong(mx));
+        }
+    }
+    if (bad) atomicOr(&u.ctrl->status, kStatusNonFinite);
+    if (u.clear_slot >= 0 && blockIdx.x == 0 && tid < 8) {
+        unsigned long long* z = tid < 2 ? &u.ctrl->alpha[u.clear_slot][tid] : &u.ctrl->alpha_f[u.clear_slot][0][tid - 2];
+        *z = 0ull;
     }
 }
 
@@ -354,7 +442,8 @@ cudaError_t launch_flux_t(int system, int dir, const FluxArgs& a, cudaStream_t s
             return small ? launch_one<1, 0, true, GEN, false>(a, s) : launch_one<1, 0, false, GEN, false>(a, s);
         if constexpr (GEN != 2)
             if (a.nx < kLineMax)
-                return launch_pdl(flux_line_kernel<GEN>, dim3(unsigned((a.nx + kLineTI) / kLineTI)), dim3(kLineThreads), 0, s, a);
+                return launch_pdl(line_kernel<3, GEN, false>, dim3(unsigned((a.nx + kLineTI) / kLineTI)),
+                                  dim3(kLineThreads<3>), 0, s, a, UpdateArgs{});
         if (small) return launch_one<3, 0, true, GEN, false>(a, s);
         if constexpr (GEN != 2)
             if (takes_linear(a, a.nx)) return launch_one<3, 0, false, GEN, true>(a, s);
@@ -373,6 +462,20 @@ cudaError_t launch_flux_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t 
     if (ax.weights == 0 && ax.split == 0) return lin ? launch_xy<0, true>(ax, ay, s) : launch_xy<0, false>(ax, ay, s);
     if (ax.split == 0 || ax.split == 3) return lin ? launch_xy<1, true>(ax, ay, s) : launch_xy<1, false>(ax, ay, s);
     return launch_xy<2, false>(ax, ay, s);
+}
+
+bool line_stage_applies(int system, const FluxArgs& a) {
+    return system != 2 && a.nx < kLineMax && (system == 0 || a.split == 0 || a.split == 3);
+}
+
+cudaError_t launch_line_stage(int system, const FluxArgs& a, const UpdateArgs& u, cudaStream_t s) {
+    const dim3 grid(unsigned((a.nx + kLineTI - 2) / (kLineTI - 1)));
+    const bool gen = a.weights != 0 || (system == 1 && a.split != 0);
+    if (system == 0)
+        return gen ? launch_pdl(line_kernel<1, 1, true>, grid, dim3(kLineThreads<1>), 0, s, a, u)
+                   : launch_pdl(line_kernel<1, 0, true>, grid, dim3(kLineThreads<1>), 0, s, a, u);
+    return gen ? launch_pdl(line_kernel<3, 1, true>, grid, dim3(kLineThreads<3>), 0, s, a, u)
+               : launch_pdl(line_kernel<3, 0, true>, grid, dim3(kLineThreads<3>), 0, s, a, u);
 }
 
 cudaError_t launch_flux(int system, int dir, const FluxArgs& a, cudaStream_t s) {

@@ -125,6 +125,17 @@ inline UpdateArgs update_args(const wenozn_problem& p, Ctrl* ctrl, const double*
     return u;
 }
 
+// One RK stage (or, mode 0, the RHS): the fluxes of stage input U and the update u, in one launch
+// for short lines.
+inline cudaError_t launch_stage(const wenozn_problem& p, const double* U, const unsigned long long* alpha_bits,
+                                const unsigned long long* alpha_f_bits, double* fx, double* gy, const UpdateArgs& u,
+                                cudaStream_t s) {
+    const FluxArgs fa = flux_args(p, U, alpha_bits, alpha_f_bits);
+    if (line_stage_applies(p.system, fa) && u.out != U) return launch_line_stage(p.system, fa, u, s);
+    const cudaError_t e = launch_fluxes(p, U, alpha_bits, alpha_f_bits, fx, gy, s);
+    return e == cudaSuccess ? launch_update(p.system, u, s) : e;
+}
+
 inline char* ws_base(void* ws) { return static_cast<char*>(ws); }
 
 // Clears every LF-speed slot (global and per-field) of the control block.

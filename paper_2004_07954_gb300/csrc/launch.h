@@ -71,6 +71,10 @@ struct UpdateArgs {
     double dt_fixed, t_remaining, cfl, dx, dy, gamma, adv_speed;
 };
 cudaError_t launch_update(int system, const UpdateArgs& a, cudaStream_t s);
+// Fluxes and update of a stage in one launch, for short 1D lines (fluxes not stored); the output
+// must not be the stage input.
+bool line_stage_applies(int system, const FluxArgs& a);
+cudaError_t launch_line_stage(int system, const FluxArgs& a, const UpdateArgs& u, cudaStream_t s);
 // ctrl->dt = the CFL step of the LF speeds in ctrl->alpha[0] (a.dt_fixed <= 0, no clipping
 // unless a.t_remaining > 0), in the update kernel's operation order.
 cudaError_t launch_cfl_dt(int system, const UpdateArgs& a, cudaStream_t s);

@@ -63,12 +63,11 @@ extern "C" wenozn_status wenozn_rhs_noalloc(const wenozn_problem* p, const doubl
     if (e == cudaSuccess)
         e = launch_max_wavespeed(p->system, U, int64_t(nx * ny), p->gamma, p->adv_speed, ctrl->alpha[0],
                                  &ctrl->status, s, field_slot(*p, ctrl, 0));
-    if (e == cudaSuccess) e = launch_fluxes(*p, U, ctrl->alpha[0], &ctrl->alpha_f[0][0][0], fx, gy, s);
     if (e == cudaSuccess) {
         UpdateArgs u = update_args(*p, ctrl, fx, gy);
         u.mode = 0;
         u.out = L;
-        e = launch_update(p->system, u, s);
+        e = launch_stage(*p, U, ctrl->alpha[0], &ctrl->alpha_f[0][0][0], fx, gy, u, s);
     }
     return cuda_status(e);
 }
