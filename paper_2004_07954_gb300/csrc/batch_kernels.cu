@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(THREADS, 2) batch_stage_kernel(BatchArgs a) {
         for (int q = threadIdx.x; q < count; q += THREADS) {
             const int jl = linear ? s_list[q] : q;
             double Fh[NV];
-            interface_flux<NV, 0, true>(sp, jl, 1, gm1, a.wide, a.eps4, a.kappa, 0, 0, nullptr, Fh);
+            interface_flux<NV, 0>(sp, jl, 1, gm1, a.wide, a.eps4, a.kappa, 0, 0, nullptr, Fh);
 #pragma unroll
             for (int k = 0; k < NV; ++k) sF[k * TI + jl] = Fh[k];
         }

@@ -30,19 +30,20 @@ namespace {
 // Both sweeps at 256^2 / 1024^2 / 4096^2, without the linear pass: 80 us / 0.54 / 7.5 ms with four
 // blocks (32 warps, 64 registers); three blocks 86 us / 0.53 / 7.5 ms, two 97 us / 0.71 / 9.2 ms,
 // 64 x 4 tiles 88 us / 0.58 / 7.55 ms, 128-thread blocks (eight) 84 us / 0.58 / 7.8 ms, a copy of the
-// code per sweep (128 x 2 and 32 x 8 tiles) 98 us / 0.63 / 7.85 ms.
-// The linear pass (LIN, interface_linear first, the rest compacted): 97 us / 0.47 / 5.75 ms with
-// three blocks, 97 us / 0.55 / 5.8 ms with four.  It pays where most interfaces pass, so lines of
-// kLinearMin cells and more take it; a single wave of blocks (short 1D lines) waits for its
-// slowest block, which pays for both passes, and does without (a rollout at 8192 cells 7.7 ms
-// without, 8.2 ms with).
+// code per sweep (128 x 2 and 32 x 8 tiles) 98 us / 0.63 / 7.85 ms; the loop over the fields rolled
+// (a quarter of the code): 77 us.
+// The linear pass (LIN, interface_linear first, the rest compacted) at 256^2 / 512^2 / 800^2 /
+// 1024^2 / 4096^2: 100 / 182 / 305 / 431 us / 5.2 ms with three blocks, 77 / 173 / 364 / 550 us / 7.5 ms
+// without it.  It pays where most interfaces pass, so lines of kLinearMin cells and more take
+// it; a single wave of blocks (short 1D lines) waits for its slowest block, which pays for both
+// passes, and does without (a rollout at 8192 cells 7.7 ms without, 8.2 ms with).
 // Long 1D lines use 251-interface tiles (256 cells with the halo: one full round of the cell
 // and difference passes; a 2^20-cell step 0.52 ms, without the linear pass 0.70 ms); short
 // ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
 // every SM gets work.  GEN = 2 projects F and U (twice the difference vectors a thread) and runs
 // best with two blocks and 128 registers (a 640 x 777 local-LF step 1.76 ms; three blocks 1.81,
 // four 1.85 ms).
-constexpr int kLinearMin = 1024;
+constexpr int kLinearMin = 640;
 template <int NV, bool SMALL = false> struct Tile { static constexpr int TI = 251, TA = 1, THREADS = 256; };
 template <int NV> struct Tile<NV, true> { static constexpr int TI = 64, TA = 1, THREADS = 64; };
 template <> struct Tile<4, false> { static constexpr int TI = 32, TA = 8, THREADS = 256; };
@@ -144,7 +145,7 @@ __device__ __forceinline__ void flux_tile(const FluxArgs& a, double* Fout, int b
         const int j = j0 + idx / TA, line = l0 + idx % TA;
         if (j >= nint || line >= nlines) continue;
         double Fh[NV];
-        interface_flux<NV, GEN, LIN>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
+        interface_flux<NV, GEN>(sp, idx, kStride, gm1, a.wide, a.eps4, a.kappa, a.weights, a.split, alpha_f, Fh);
         store(idx, Fh);
     }
 }
