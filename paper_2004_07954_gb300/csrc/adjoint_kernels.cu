@@ -101,13 +101,14 @@ __host__ __device__ __forceinline__ double zn_vjp(const double* f, double Wb, do
 // ---------------------------------------------------------------------------------------
 // Interface VJPs.  A block takes kTI consecutive interfaces and their kCells stencil cells,
 // whose split fluxes h+- (and, for Euler, u, H, sqrt(rho), 1/rho) it computes once into
-// shared memory.  For Euler each interface is then handled by three threads, one per
-// characteristic field k (warp k of the block): the Roe state, row k of the left and column
-// k of the right eigenvectors, the projection of the stencil onto field k, both WENO-ZN
-// reconstructions of that field and their reverse sweeps.  Each field leaves its projected
-// stencil's cotangents, half its left-eigenvector row and its Roe-quantity cotangents in
-// shared memory; the cotangents of the split fluxes are then the sums over the fields of
-// row m times the projected cotangents, and the Roe quantities' the sums of the fields'.
+// shared memory.  For Euler an interface whose weights are the optimal ones to rounding,
+// derivatives included, reverses as constant coefficients; each other one is handled by six
+// threads, one per characteristic field k and side: the Roe state, row k of the left and
+// column k of the right eigenvectors, the projection of the side's stencil onto field k, its
+// WENO-ZN reconstruction and the reverse sweep.  Each leaves its projected stencil's
+// cotangents, half its left-eigenvector row and its Roe-quantity cotangents in shared memory;
+// the cotangents of the split fluxes are then the sums over the fields of row m times the
+// projected cotangents, and the Roe quantities' the sums of the threads'.
 //
 // Per interface j and stencil position s = 0..5 (cell j - 3 + s) the results are
 //   (hbar+_{s,m} + hbar-_{s,m}) / 2  and  (hbar+_{s,m} - hbar-_{s,m}) / 2,  m = 0..NV-1,
@@ -116,12 +117,12 @@ __host__ __device__ __forceinline__ double zn_vjp(const double* f, double Wb, do
 // hbar+ dh+/dU + hbar- dh-/dU is J_F^T (hbar+ + hbar-)/2 + alpha (hbar+ - hbar-)/2: the
 // gather applies J_F^T once per cell to the summed first part.
 // ---------------------------------------------------------------------------------------
-constexpr int kTI = 32;                 // interfaces per block (one warp per field)
+constexpr int kTI = 32;                 // interfaces per block (one lane each)
 constexpr int kCells = kTI + 5;         // their stencil cells
 constexpr int kGather = 64;             // cells per advection gather block
 
 // The Euler stage kernel's tile: TI interfaces and their TI + 5 stencil cells; WIDE: one
-// thread per interface (all three fields), else one per (interface, field).
+// thread per interface (all three fields), else one per (interface, field, side).
 template <int TI, bool WIDE>
 struct EulerSmem {
     static constexpr int NC = TI + 5;
@@ -130,10 +131,13 @@ struct EulerSmem {
     double u[NC], H[NC], sq[NC], r[NC], Ep[NC];
     int64_t dp[3][NC], dm[3][NC];       // mantissas of the split fluxes' differences
     uint32_t ex[4][NC];                 // and their exponents (CellPlanes)
-    unsigned char lin[WIDE ? 1 : 3][TI];   // per-field threads: the field's weights are the optimal ones
-    double red[WIDE ? 1 : 3][WIDE ? 1 : 19][WIDE ? 1 : TI];   // per field: cotangents of its projected
-                                        // h+ (5) and h- (5), half its left-eigenvector row (3), 6 Roe
-                                        // scalars (the per-field threads' exchange)
+    // the six-warp form's: the field's weights are the optimal ones; each warp's copy of the
+    // remaining interfaces; their Roe states (u~, H~, 1/c, (gamma-1)/c^2, 1/(sqrt(rhoL) + sqrt(rhoR)));
+    // and the exchange between their threads, per field: cotangents of its projected h+ (5) and
+    // h- (5), half its left-eigenvector row (3), 6 Roe scalars of either side
+    unsigned char lin[WIDE ? 1 : 3][TI], list[WIDE ? 1 : 6][TI];
+    double roe[WIDE ? 1 : 5][WIDE ? 1 : TI];
+    double red[WIDE ? 1 : 3][WIDE ? 1 : 25][WIDE ? 1 : TI];
 };
 
 // ---------------------------------------------------------------------------------------
@@ -142,7 +146,7 @@ struct EulerSmem {
 // j = c0 - 2 .. c0 + kOwn + 2 (kTI of them), so that it can gather its own cells without
 // anything from other blocks; neighbouring blocks both compute the five interfaces they
 // share (5/kOwn more interface work, and no second launch).  Two forms: one thread per
-// (interface, characteristic field) with 32-interface tiles, which gives short lines three
+// (interface, characteristic field, side) with 32-interface tiles, which gives short lines six
 // times the warps, and one thread per interface with 64-interface tiles, which does less
 // work per interface and serves long lines (kWideMinCells).  What the tile cannot hold
 // crosses blocks through global memory:
@@ -168,17 +172,22 @@ struct EulerSmem {
 // and resets the argmax word and the counter.  Every sum has a fixed order, so the result
 // is deterministic and does not depend on which launches complete in place.
 // ---------------------------------------------------------------------------------------
-constexpr int kOwn = kTI - 5;           // cells owned by a block of the per-field kernel (the most blocks)
+constexpr int kOwn = kTI - 5;           // cells owned by a block of the short lines' kernel (the most blocks)
 constexpr int kGhostSlot = 6 * 9;       // 6 ghost cells x (flux, LF, Roe) x 3 components
 constexpr int kEnt = 7;                 // pending corrections of a record: 6 ghost targets + the argmax
 constexpr int kTIWide = 64;             // interfaces a block of the one-thread-per-interface kernel
-// Lines of at least this many cells take the one-thread-per-interface kernel (fewer FP64
-// instructions: no per-field copies of the Roe state, the fields' cotangents summed in
-// registers, 5 of 64 interfaces computed twice instead of 5 of 32); shorter ones need the
-// per-field kernel's three times as many warps to occupy the GPU.  Measured crossover:
-// 8192 cells 105 (per field) against 154 us per reverse step, 12288 cells 196 against 165 (before
-// the linear reverse below: now 103 us at 8192, 425 against 1153 us at 131071 cells of smooth data;
-// a launch of one wave still waits for the blocks that hold a nonlinear interface).
+// Lines of at least this many cells take the one-thread-per-interface kernel: fewer FP64
+// instructions where every interface is nonlinear (no copies of the Roe state, the fields'
+// cotangents summed in registers, 5 of 64 interfaces computed twice instead of 5 of 32);
+// shorter ones need the other kernel's six times as many warps, and its two blocks an SM end
+// with the slowest.  A reverse step (three launches) in us, six threads / one thread an interface:
+// smooth waves 8192 cells 85 / 164, 16384 118 / 166, 131071 514 / 406; random cells (every
+// interface nonlinear) 114 / 170 at 8192, 217 / 175 at 16384, 1629 / 1165 at 131071: the line lies
+// where neither kind of data loses.  With three threads an interface (both sides in turn, no
+// compaction) 8192 cells of smooth waves took 103.
+// Where the time of a block with nonlinear interfaces goes (200 cells, 45 thousand cycles): cells
+// 7, the linear check 2.5, the reverses 23 (two warps on the busiest sub-partition, 230 FP64
+// instructions of 64 cycles each), gathering their results 8, the rest 5; without any, 20 in all.
 constexpr int kWideMinCells = 10240;
 
 template <int TI, bool WIDE>
@@ -188,11 +197,11 @@ struct StageSmem {
     double cR[2][3][TI];                   // Roe-input cotangents (left cell, right cell)
     double sF[3][TI - 5];                  // gathered flux parts, exchanged between component threads
     double ghost[6][3][3];                 // ghost slots x (flux, LF, Roe) x component
-    double red[3];
+    double red[6];
     double lamw[3][TI + 1];                // the cotangent input on the window, corrections applied
     double pcq[kVjpPend][6][3];            // input records: ghost slots summed over the edge blocks,
     double pds[kVjpPend][3];               //   the argmax cell's speed derivative,
-    double pred[kVjpPend][3];              //   per-warp sums of the partials,
+    double pred[kVjpPend][6];              //   per-warp sums of the partials,
     double pa[kVjpPend][kEnt], pb[kVjpPend][kEnt][3];   // and their entries: x <- fma(pa, pb_m, x)
     int pcell[kVjpPend][kEnt];                           //   at cell pcell (-1: none)
     int last;                              // this block finished last
@@ -241,15 +250,14 @@ __device__ __forceinline__ double jft_row(int m, double F0, double F1, double F2
 // the Roe state (u~, H~, c, 1/c, b1 = (gamma-1)/c^2, b2 = u~^2 b1 / 2).
 __device__ __forceinline__ void field_lr(int k, double ut, double Ht, double c, double rc, double b1, double b2,
                                          double& L0, double& L1, double& L2, double& R1, double& R2) {
-    if (k == 0) {
-        L0 = 0.5 * fma(ut, rc, b2); L1 = -0.5 * fma(b1, ut, rc); L2 = 0.5 * b1;
-        R1 = ut - c; R2 = fma(-ut, c, Ht);
-    } else if (k == 1) {
+    if (k == 1) {
         L0 = 1.0 - b2; L1 = b1 * ut; L2 = -b1;
         R1 = ut; R2 = 0.5 * ut * ut;
     } else {
-        L0 = 0.5 * fma(-ut, rc, b2); L1 = -0.5 * fma(b1, ut, -rc); L2 = 0.5 * b1;
-        R1 = ut + c; R2 = fma(ut, c, Ht);
+        // (one path for k = 0 and 2, the signs of c and u~ apart: the lanes of a warp mix fields)
+        const double cs = k == 0 ? c : -c, rcs = k == 0 ? rc : -rc;
+        L0 = 0.5 * fma(ut, rcs, b2); L1 = -0.5 * fma(b1, ut, rcs); L2 = 0.5 * b1;
+        R1 = ut - cs; R2 = fma(-ut, cs, Ht);
     }
 }
 
@@ -257,15 +265,14 @@ __device__ __forceinline__ void field_lr(int k, double ut, double Ht, double c, 
 // of b2, b1, 1/c, u~, c and H~ (q[0..5]).
 __device__ __forceinline__ void field_lr_reverse(int k, const double* Lb, double Rb1, double Rb2, double ut, double c,
                                                  double rc, double b1, double* q) {
-    if (k == 0) {
-        q[0] = 0.5 * Lb[0]; q[1] = 0.5 * fma(-ut, Lb[1], Lb[2]); q[2] = 0.5 * fma(ut, Lb[0], -Lb[1]);
-        q[3] = 0.5 * fma(rc, Lb[0], -b1 * Lb[1]) + fma(-c, Rb2, Rb1); q[4] = fma(-ut, Rb2, -Rb1); q[5] = Rb2;
-    } else if (k == 1) {
+    if (k == 1) {
         q[0] = -Lb[0]; q[1] = fma(ut, Lb[1], -Lb[2]); q[2] = 0.0;
         q[3] = fma(b1, Lb[1], fma(ut, Rb2, Rb1)); q[4] = 0.0; q[5] = 0.0;
     } else {
-        q[0] = 0.5 * Lb[0]; q[1] = 0.5 * fma(-ut, Lb[1], Lb[2]); q[2] = 0.5 * fma(-ut, Lb[0], Lb[1]);
-        q[3] = -0.5 * fma(rc, Lb[0], b1 * Lb[1]) + fma(c, Rb2, Rb1); q[4] = fma(ut, Rb2, Rb1); q[5] = Rb2;
+        const double cs = k == 0 ? c : -c, rcs = k == 0 ? rc : -rc;
+        const double q2 = 0.5 * fma(ut, Lb[0], -Lb[1]), q4 = fma(-ut, Rb2, -Rb1);
+        q[0] = 0.5 * Lb[0]; q[1] = 0.5 * fma(-ut, Lb[1], Lb[2]); q[2] = k == 0 ? q2 : -q2;
+        q[3] = 0.5 * fma(rcs, Lb[0], -b1 * Lb[1]) + fma(-cs, Rb2, Rb1); q[4] = k == 0 ? q4 : -q4; q[5] = Rb2;
     }
 }
 
@@ -294,9 +301,10 @@ __device__ __forceinline__ void roe_reverse_cell(const double* sc, double ut, do
 }
 
 template <int TI, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a) {
+__global__ void __launch_bounds__(WIDE ? TI : 6 * TI, WIDE ? 1 : 2) vjp_stage_euler(VjpArgs a) {
     constexpr int kTI = TI, kOwn = TI - 5, kCells = TI + 5, kWin = TI + 1;   // (shadow the per-field values)
-    constexpr int kThreads = WIDE ? TI : 3 * TI, kWarps = kThreads / 32;
+    static_assert(WIDE || TI == 32, "one warp per (field, side)");
+    constexpr int kThreads = WIDE ? TI : 6 * TI, kWarps = kThreads / 32;
     constexpr int kLw = (3 * kWin + kThreads - 1) / kThreads;   // rounds of the window load
     constexpr int kCand = WIDE ? kThreads - 1 : 2 * kTI;        // the thread that offers the argmax candidate
     __shared__ StageSmem<TI, WIDE> S;
@@ -333,7 +341,7 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
     }
     // the input records' argmax words (uniform loads); where the argmax cell lies in the
     // window, its speed derivative and abar: the cotangent input's record sums its partials
-    // (the first 4 x 96 loaded now, used after the cell phase), the others were summed by
+    // (the first four a thread loaded now, used after the cell phase), the others were summed by
     // the launch that read them as its cotangent input, which left abar in the record
     int imp[kVjpPend];
     bool need = false;
@@ -460,7 +468,7 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
         slot[2] = kk * gm1;
     }
 
-    const int k = WIDE ? 0 : tid / kTI, i = WIDE ? tid : tid % kTI, j = j0 + i;
+    const int w = tid / kTI, i = tid % kTI, j = j0 + i;
     // ---- the corrections pending on the inputs (block-uniform branches) ------------------
     if (tid < kVjpPend * kEnt * 3) {
         // entry e of record p, component mm: e < 6 the first ghost slot of a target cell in the
@@ -529,125 +537,135 @@ __global__ void __launch_bounds__(WIDE ? TI : 3 * TI) vjp_stage_euler(VjpArgs a)
     if (WIDE) {
         if (live) lin = NearLinear<3, true>(planes, i, 1, gm1, a.wide, 0, 3).ok;
     } else {
-        if (live) sm.lin[k][i] = NearLinear<3, true>(planes, i, 1, gm1, a.wide, k, k + 1).ok;
+        if (live && w < 3) sm.lin[w][i] = NearLinear<3, true>(planes, i, 1, gm1, a.wide, w, w + 1).ok;
         __syncthreads();
         if (live) lin = sm.lin[0][i] & sm.lin[1][i] & sm.lin[2][i];
     }
-    double ut = 0, Ht = 0, c = 0, rc = 0, b1 = 0, b2 = 0, wl = 0, wr = 0, rS = 0;
     double Fb[3] = {0.0, 0.0, 0.0};
     if (live)
         for (int m = 0; m < 3; ++m) Fb[m] = (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx;   // cells j, j - 1
-    if (live && !lin) {
-        // Roe state (R[0][k] = 1) and the cotangents of the interface flux
-        const double sl = sm.sq[cl], sr = sm.sq[cr];
-        rS = rcp_nr(sl + sr);
-        wl = sl * rS;
-        wr = sr * rS;
-        ut = fma(wl, sm.u[cl], wr * sm.u[cr]);
-        Ht = fma(wl, sm.H[cl], wr * sm.H[cr]);
-        const double c2 = gm1 * fma(-0.5 * ut, ut, Ht);
-        rc = rsqrt(c2);
-        c = c2 * rc;
-        b1 = gm1 * rc * rc;
-        b2 = 0.5 * ut * ut * b1;
-    }
     double ab = 0.0;
     if constexpr (!WIDE) {
-        // one thread per (interface, field k): the field's projection, both reconstructions
-        // and their reverse; the fields' results meet in shared memory
-        if (live && !lin) {
-            double L0, L1, L2, R1, R2;
-            field_lr(k, ut, Ht, c, rc, b1, b2, L0, L1, L2, R1, R2);
-            double fp[5], fm[5], fpb[5], fmb[5];
+        // Six threads per remaining interface, one per (field, side): the field's projection,
+        // the reconstruction and its reverse; their results meet in shared memory.  The
+        // interfaces are compacted first, so a block with five of them or fewer (an extremum of a
+        // field) does them all in one warp, and a launch of a single wave, which lasts as long as
+        // its slowest block, waits for one reverse of a reconstruction instead of two.
+        const unsigned rest = __ballot_sync(0xffffffffu, live && !lin);   // the same in every warp
+        const int nrest = __popc(rest);
+        if (nrest > 0) {
+            if (live && !lin) sm.list[w][__popc(rest & ((1u << i) - 1u))] = (unsigned char)i;
+            __syncwarp();
+            if (tid < 6 * nrest) {
+                const int fs = tid / nrest, x = sm.list[w][tid - fs * nrest], k = fs >> 1, side = fs & 1;
+                const double sl = sm.sq[x + 2], sr = sm.sq[x + 3], rS = rcp_nr(sl + sr), wl = sl * rS, wr = sr * rS;
+                const double ut = fma(wl, sm.u[x + 2], wr * sm.u[x + 3]), Ht = fma(wl, sm.H[x + 2], wr * sm.H[x + 3]);
+                const double c2 = gm1 * fma(-0.5 * ut, ut, Ht), rc = inv_sqrt(c2), c = c2 * rc;
+                const double b1 = gm1 * rc * rc, b2 = 0.5 * ut * ut * b1;
+                double L0, L1, L2, R1, R2;
+                field_lr(k, ut, Ht, c, rc, b1, b2, L0, L1, L2, R1, R2);
+                double G[3];
 #pragma unroll
-            for (int s = 0; s < 5; ++s) {
-                fp[s] = fma(L2, sm.hp[2][i + s], fma(L1, sm.hp[1][i + s], L0 * sm.hp[0][i + s]));
-                fm[4 - s] = fma(L2, sm.hm[2][i + s + 1], fma(L1, sm.hm[1][i + s + 1], L0 * sm.hm[0][i + s + 1]));
+                for (int m = 0; m < 3; ++m) G[m] = (S.lamw[m][x + 1] - S.lamw[m][x]) * a.rdx;
+                // the five points in the order of the side's stencil
+                const double* h = side == 0 ? &sm.hp[0][x] : &sm.hm[0][x + 5];
+                const int step = side == 0 ? 1 : -1;
+                double f[5], fb[5];
+#pragma unroll
+                for (int s = 0; s < 5; ++s)
+                    f[s] = fma(L2, h[2 * kCells + s * step], fma(L1, h[kCells + s * step], L0 * h[s * step]));
+                const double ghb = fma(R2, G[2], fma(R1, G[1], G[0]));
+                const double gh = zn_vjp(f, ghb, a.eps4, a.kappa, fb);
+                double Lb[3] = {0, 0, 0};
+#pragma unroll
+                for (int s = 0; s < 5; ++s) {
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) Lb[m] = fma(fb[s], h[m * kCells + s * step], Lb[m]);
+                    sm.red[k][side == 0 ? s : 9 - s][x] = fb[s];     // of the projected h+_s, h-_{s+1}
+                }
+                if (side == 0) {
+                    sm.red[k][10][x] = 0.5 * L0; sm.red[k][11][x] = 0.5 * L1; sm.red[k][12][x] = 0.5 * L2;
+                }
+                if (fs == 0) {
+                    sm.roe[0][x] = ut; sm.roe[1][x] = Ht; sm.roe[2][x] = rc; sm.roe[3][x] = b1; sm.roe[4][x] = rS;
+                }
+                double q[6];
+                field_lr_reverse(k, Lb, G[1] * gh, G[2] * gh, ut, c, rc, b1, q);
+#pragma unroll
+                for (int t = 0; t < 6; ++t) sm.red[k][13 + 6 * side + t][x] = q[t];
             }
-            const double ghb = fma(R2, Fb[2], fma(R1, Fb[1], Fb[0]));
-            const double gh = zn_vjp(fp, ghb, a.eps4, a.kappa, fpb) +
-                              zn_vjp(fm, ghb, a.eps4, a.kappa, fmb);
-            double Lb[3] = {0, 0, 0};
-#pragma unroll
-            for (int s = 0; s < 5; ++s) {
-                const double gpb = fpb[s], gmb = fmb[4 - s];     // cotangents of the projected h+_s, h-_{s+1}
-#pragma unroll
-                for (int m = 0; m < 3; ++m) Lb[m] = fma(gpb, sm.hp[m][i + s], fma(gmb, sm.hm[m][i + s + 1], Lb[m]));
-                sm.red[k][s][i] = gpb;
-                sm.red[k][5 + s][i] = gmb;
-            }
-            sm.red[k][10][i] = 0.5 * L0; sm.red[k][11][i] = 0.5 * L1; sm.red[k][12][i] = 0.5 * L2;
-            double q[6];
-            field_lr_reverse(k, Lb, Fb[1] * gh, Fb[2] * gh, ut, c, rc, b1, q);
-#pragma unroll
-            for (int t = 0; t < 6; ++t) sm.red[k][13 + t][i] = q[t];
+            __syncthreads();
         }
-        __syncthreads();
-        // stencil positions 2k, 2k+1: the cotangents of h+- there, (hbar+ +- hbar-)/2 summed over
-        // the three fields (row m of each field's left eigenvector times its projected cotangent),
-        // and, for an owned interface, its share sum_s U_s . (hbar+ - hbar-)_s / 2 of the
-        // LF-speed cotangent
-        double hL[3][3];
-#pragma unroll
-        for (int f = 0; f < 3; ++f)
-#pragma unroll
-            for (int m = 0; m < 3; ++m) hL[f][m] = live && !lin ? sm.red[f][10 + m][i] : 0.0;
+        // stencil position w: the cotangents of h+- there, (hbar+ +- hbar-)/2 summed over the
+        // three fields (row m of each field's left eigenvector times its projected cotangent), and,
+        // for an owned interface, its share sum_s U_s . (hbar+ - hbar-)_s / 2 of the LF-speed cotangent
         if (lin) {
             // (hbar+ + hbar-)/2 = (2, -16, 74, 74, -16, 2)/120 Fb, (hbar+ - hbar-)/2 = (2, -10, 20,
-            // -20, 10, -2)/120 Fb at positions 0..5: this thread's are 2k and 2k + 1
-            const double f0 = k == 0 ? 2.0 / 120.0 : (k == 1 ? 74.0 / 120.0 : -16.0 / 120.0);
-            const double f1 = k == 0 ? -16.0 / 120.0 : (k == 1 ? 74.0 / 120.0 : 2.0 / 120.0);
-            const double d0 = k == 0 ? 2.0 / 120.0 : (k == 1 ? 20.0 / 120.0 : 10.0 / 120.0);
-            const double d1 = k == 0 ? -10.0 / 120.0 : (k == 1 ? -20.0 / 120.0 : -2.0 / 120.0);
+            // -20, 10, -2)/120 Fb at positions 0..5
+            const double f = w == 0 || w == 5 ? 2.0 / 120.0 : (w == 1 || w == 4 ? -16.0 / 120.0 : 74.0 / 120.0);
+            const double d0 = w == 0 || w == 5 ? 2.0 / 120.0 : (w == 1 || w == 4 ? -10.0 / 120.0 : 20.0 / 120.0);
+            const double d = w < 3 ? d0 : -d0;
 #pragma unroll
             for (int m = 0; m < 3; ++m) {
-                const double e0 = d0 * Fb[m], e1 = d1 * Fb[m];
-                S.cF[2 * k][m][i] = f0 * Fb[m];
-                S.cF[2 * k + 1][m][i] = f1 * Fb[m];
-                S.cD[2 * k][m][i] = e0;
-                S.cD[2 * k + 1][m][i] = e1;
-                if (owned) ab = fma(sm.U[m][i + 2 * k + 1], e1, fma(sm.U[m][i + 2 * k], e0, ab));
+                const double e = d * Fb[m];
+                S.cF[w][m][i] = f * Fb[m];
+                S.cD[w][m][i] = e;
+                if (owned) ab = fma(sm.U[m][i + w], e, ab);
             }
-        } else
+        } else {
+            double hL[3][3], gp[3], gm[3];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int s = 2 * k + t;
-            double gp[3] = {0.0, 0.0, 0.0}, gm[3] = {0.0, 0.0, 0.0};
-            if (live) {
-                if (s <= 4)
+            for (int f = 0; f < 3; ++f) {
 #pragma unroll
-                    for (int f = 0; f < 3; ++f) gp[f] = sm.red[f][s][i];
-                if (s >= 1)
-#pragma unroll
-                    for (int f = 0; f < 3; ++f) gm[f] = sm.red[f][4 + s][i];
-            }
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
+                for (int m = 0; m < 3; ++m) hL[f][m] = live ? sm.red[f][10 + m][i] : 0.0;
                 // (position 5 has no plus-side point, position 0 no minus-side one)
-                const double hpb = s <= 4 ? fma(gp[2], hL[2][m], fma(gp[1], hL[1][m], gp[0] * hL[0][m])) : 0.0;
-                const double hmb = s >= 1 ? fma(gm[2], hL[2][m], fma(gm[1], hL[1][m], gm[0] * hL[0][m])) : 0.0;
-                const double sumF = hpb + hmb, dh = hpb - hmb;
-                if (owned) ab = fma(sm.U[m][i + s], dh, ab);
-                S.cF[s][m][i] = sumF;
-                S.cD[s][m][i] = dh;
+                gp[f] = live && w <= 4 ? sm.red[f][w][i] : 0.0;
+                gm[f] = live && w >= 1 ? sm.red[f][4 + w][i] : 0.0;
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const double hpb = w <= 4 ? fma(gp[2], hL[2][m], fma(gp[1], hL[1][m], gp[0] * hL[0][m])) : 0.0;
+                const double hmb = w >= 1 ? fma(gm[2], hL[2][m], fma(gm[1], hL[1][m], gm[0] * hL[0][m])) : 0.0;
+                const double dh = hpb - hmb;
+                if (owned) ab = fma(sm.U[m][i + w], dh, ab);
+                S.cF[w][m][i] = hpb + hmb;
+                S.cD[w][m][i] = dh;
             }
         }
-        if (k > 0) {
-            // the Roe average reversed: warp 1 gives the left cell, warp 2 the right
+        if (w == 0 || w == 5) {
+            // the Roe average reversed: warp 0 gives the left cell, warp 5 the right
             double Ub[3] = {0.0, 0.0, 0.0};
             if (live && !lin) {
                 double sc[6];
 #pragma unroll
-                for (int q = 0; q < 6; ++q) sc[q] = (sm.red[0][13 + q][i] + sm.red[1][13 + q][i]) + sm.red[2][13 + q][i];
-                const int cc = k == 1 ? cl : cr;
-                roe_reverse_cell(sc, ut, Ht, rc, b1, rS, gm1, a.gamma, k == 1 ? wl : wr, sm.u[cc], sm.H[cc], sm.r[cc],
-                                 sm.sq[cc], Ub);
+                for (int q = 0; q < 6; ++q)
+                    sc[q] = ((sm.red[0][13 + q][i] + sm.red[0][19 + q][i]) + (sm.red[1][13 + q][i] + sm.red[1][19 + q][i])) +
+                            (sm.red[2][13 + q][i] + sm.red[2][19 + q][i]);
+                const int cc = w == 0 ? cl : cr;
+                const double rS = sm.roe[4][i];
+                roe_reverse_cell(sc, sm.roe[0][i], sm.roe[1][i], sm.roe[2][i], sm.roe[3][i], rS, gm1, a.gamma,
+                                 sm.sq[cc] * rS, sm.u[cc], sm.H[cc], sm.r[cc], sm.sq[cc], Ub);
             }
-            for (int m = 0; m < 3; ++m) S.cR[k - 1][m][i] = Ub[m];
+            for (int m = 0; m < 3; ++m) S.cR[w == 0 ? 0 : 1][m][i] = Ub[m];
         }
     } else {
         // one thread per interface: the three fields in turn, their cotangents summed in
-        // registers in the same order as the per-field threads sum them in shared memory
+        // registers
+        double ut = 0, Ht = 0, c = 0, rc = 0, b1 = 0, b2 = 0, wl = 0, wr = 0, rS = 0;
+        if (live && !lin) {
+            // Roe state (R[0][k] = 1)
+            const double sl = sm.sq[cl], sr = sm.sq[cr];
+            rS = rcp_nr(sl + sr);
+            wl = sl * rS;
+            wr = sr * rS;
+            ut = fma(wl, sm.u[cl], wr * sm.u[cr]);
+            Ht = fma(wl, sm.H[cl], wr * sm.H[cr]);
+            const double c2 = gm1 * fma(-0.5 * ut, ut, Ht);
+            rc = inv_sqrt(c2);
+            c = c2 * rc;
+            b1 = gm1 * rc * rc;
+            b2 = 0.5 * ut * ut * b1;
+        }
         double hpb[5][3], hmb[5][3];           // halved cotangents of h+ at cells i+s, of h- at cells i+s+1
         double sc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
@@ -956,7 +974,7 @@ __global__ void __launch_bounds__(kGather) vjp_gather_advection(VjpArgs a) {
 
 }  // namespace
 
-// The Euler stage kernel is FP64-bound and as fast as its busiest SM: the block scheduler
+// The short lines' stage kernel is as fast as its busiest SM: the block scheduler
 // balances it over empty SMs (two blocks per SM at the sizes where it matters), but
 // launched with programmatic dependent launch its blocks become resident (and wait) while
 // the previous launch drains, and would pile up on the SMs that launch leaves free first.
@@ -1011,7 +1029,7 @@ cudaError_t launch_vjp(int system, const VjpArgs& a, cudaStream_t s) {
     size_t pad = 0;
     cudaError_t e = euler_interface_pad(&pad);
     if (e == cudaSuccess)
-        e = launch_pdl(vjp_stage_euler<kTI, false>, dim3(unsigned((a.n + kOwn - 1) / kOwn)), dim3(3 * kTI), pad, s, a);
+        e = launch_pdl(vjp_stage_euler<kTI, false>, dim3(unsigned((a.n + kOwn - 1) / kOwn)), dim3(6 * kTI), pad, s, a);
     return e;
 }
 

@@ -314,3 +314,29 @@ def test_vjp_rejects_2d(wz):
     p = wz.wenozn_problem_init(wz.WENOZN_EULER_2D, 8, 8, 0.1, 0.1)
     with pytest.raises(wz.WenoznError):
         wz.wenozn_vjp_workspace_size(p)
+
+
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("kinks", [(), (13,), (0, 26, 27, 136), (40, 47, 55), tuple(range(137))])
+def test_rhs_vjp_with_few_nonlinear_interfaces(wz, orc, kinks, bc):
+    """Short lines compact the interfaces that need their reconstructions reversed, six threads
+    each: none of a block's 32, the seven around one kink (more than a warp's 32 lanes), kinks at the
+    tiles' and the grid's edges, two runs of them in one tile, all.  On a constant state the
+    others reverse as constant coefficients.  The tolerance is that of
+    test_rhs_vjp_dot_product: the terms' rounding, summed."""
+    n = 137
+    p, P = _problem(wz, orc, 1, n, 10.0 / n, bc)
+    g = np.random.default_rng(7)
+    rho, u, pr = np.full(n, 1.0), np.full(n, 0.4), np.full(n, 1.1)
+    for c in kinks:                          # (two cells: about one alone IS_0 = IS_2, where |.| has no derivative)
+        for q in (rho, u, pr):
+            q[c:c + 2] += g.uniform(-0.1, 0.1, size=len(q[c:c + 2]))
+    U = np.ascontiguousarray(inputs.cons_from_prim(rho, u, pr).reshape(3, 1, n))
+    ws = wz.vjp_workspace(p)
+    for _ in range(3):
+        v, lam = g.normal(size=U.shape), g.normal(size=U.shape)
+        _, Jv = orc.rhs_jvp_quad(P, U, v)
+        out = torch.empty_like(dev(U))
+        wz.wenozn_rhs_vjp(p, dev(U), dev(lam), out, ws)
+        a, b = float(np.sum(lam * Jv)), float(np.sum(out.cpu().numpy() * v))
+        assert b == pytest.approx(a, rel=1e-10, abs=1e-12 * np.abs(lam).sum() * np.abs(Jv).max())
