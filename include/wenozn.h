@@ -22,11 +22,11 @@
  *    anything.  Launch failures return WENOZN_ECUDA.  Conditions detected on the device
  *    (non-finite values, rho <= 0 or p <= 0) set bits in the workspace status word, read
  *    with wenozn_workspace_status; the kernels never trap.
- *  - Range of the reconstruction.  The weights are evaluated division-free (their common
- *    denominator is a fifth-degree product of the smoothness indicators).  When that
- *    product leaves the double range (stencil differences above about 1e26, or data far
- *    below the scale of eps), the weights are evaluated again on the stencil scaled by an
- *    exact power of two, which is exact algebra.  With the admissible constants
+ *  - Range of the reconstruction.  The weights are evaluated in integer arithmetic whose
+ *    exponents neither overflow nor underflow; stencils it does not take (values near the ends of
+ *    the double range, infinities, NaN) are evaluated division-free in double, on the stencil
+ *    scaled by an exact power of two where the common denominator (a fifth-degree product of
+ *    the smoothness indicators) would leave the double range.  With the admissible constants
  *    (1e-60 <= eps <= 1, 1e-6 <= A <= 1e6; other values return WENOZN_EINVAL) every
  *    reconstruction is therefore finite and accurate to rounding for stencils whose first
  *    differences stay below 2^440 (about 2.8e132) in magnitude; for Euler these are the

@@ -1,5 +1,6 @@
 // Interface-flux kernels: global Lax-Friedrichs splitting, Roe-averaged characteristic
-// projection and WENO-ZN reconstruction of both split parts, one thread per interface.
+// projection and WENO-ZN reconstruction of both split parts, one thread per interface (short
+// 1D Euler lines: one per interface, field and side, the stage update in the same launch).
 // The generic instantiations (GEN = 1: splittings that project the cell split fluxes, global
 // LF and Steger-Warming; GEN = 2: those that split per field after the projection, per-field
 // and local LF) take the weight function and the flux splitting at run
@@ -10,7 +11,8 @@
 // first computes, once per cell of the tile plus its 3+2 halo cells, the split fluxes
 // h+- = (F +- alpha U)/2 and the Roe-average ingredients (sqrt(rho), velocities, H) into
 // shared memory; then every thread turns the six cells around its interface into
-// F^_{i-1/2} = R (g^+ + g^-).  No interface is computed twice.
+// F^_{i-1/2} = R (g^+ + g^-).  No interface is computed twice (but by line_kernel, whose blocks
+// share the interfaces at their edges).
 #include <atomic>
 
 #include "euler_device.cuh"

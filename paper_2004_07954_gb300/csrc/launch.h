@@ -38,7 +38,7 @@ struct FluxArgs {
     const unsigned long long* alpha_f_bits;  // per-field speeds [dir][3] (split 1 only)
     int nx, ny, bc;                        // bc of the sweep direction (0 periodic, 1 outflow, 2 reflective)
     int weights, split;                    // weight function and flux splitting (wenozn.h enums)
-    double eps4, kappa, gamma, adv_speed;  // eps4 = 4 eps, kappa = 2 / sqrt(A) (see zn_parts)
+    double eps4, kappa, gamma, adv_speed;  // eps4 = 4 eps, kappa = 2 / sqrt(A) (see zn_num_den)
     WideConst wide;                        // the same constants for the integer evaluation
 };
 // Admissible constants of the weights: with 1e-60 <= eps <= 1 and 1e-6 <= A <= 1e6 the

@@ -4,7 +4,9 @@
 // resource: constants are folded, the three un-normalised weights are brought to a common
 // denominator so that one division per reconstruction remains, and comparisons of
 // non-negative indicators run on the integer pipe.  Every rearrangement is exact algebra;
-// only the rounding differs from the plain evaluation order.
+// only the rounding differs from the plain evaluation order.  The kernels evaluate the weights
+// in 64-bit integers first (wide_weights.cuh); the double evaluation here serves the stencils
+// that refuses (infinities, NaN and exponents outside its range) and the adjoint.
 #pragma once
 
 #include <cmath>
@@ -47,7 +49,7 @@ namespace wz {
 //    division per reconstruction.  The fourth difference is d4 = t0 + t2.
 //
 // Range.  The a_k are fifth powers of the indicators, so for stencils whose differences
-// exceed about 2^88 they overflow, and for data far below the scale of eps (differences
+// exceed about 2^88 they overflow in double, and for data far below the scale of eps (differences
 // under about sqrt(eps) times 1e-100) the numerator underflows.  Every quantity above is
 // homogeneous once eps is scaled with the data: with the first differences multiplied by s
 // and eps by s^2, each b_k scales by s^2, each a_k by s^10 and num/den by s.  So the fast
@@ -223,16 +225,6 @@ __host__ __device__ __forceinline__ double zn_correction_rescaled(double D1, dou
 // Newton reciprocal applies.
 // base + (f^ - c) from the stencil's first differences D1..D4 (f^ - c depends on nothing
 // else), so that a caller holding the differences and several centre values adds them once.
-__host__ __device__ __forceinline__ double zn_flux_d(double D1, double D2, double D3, double D4, double base,
-                                                     double eps4, double kappa) {
-    double num, den;
-    zn_num_den(D1, D2, D3, D4, eps4, kappa, num, den);
-    if (zn_out_of_range(num, den, D1, D2, D3, D4))
-        return base + zn_correction_rescaled(D1, D2, D3, D4, eps4, kappa, 0);
-    return fma(num, rcp_nr(den), base);
-}
-
-// zn_flux_d with the weight function chosen at run time
 __host__ __device__ __forceinline__ double zn_flux_w_d(double D1, double D2, double D3, double D4, double base,
                                                        double eps4, double kappa, int weights) {
     double num, den;

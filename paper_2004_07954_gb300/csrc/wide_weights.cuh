@@ -7,8 +7,8 @@
 // multiply-add ones, on pipes that otherwise idle; where the weights hardly differ from the
 // optimal ones (wide_linear) about 150 in all.  Measured with the FP64 weights before and these
 // after (with the integer projection of euler_device.cuh in the solver): wenozn_reconstruct
-// 1.24 -> 0.24 ms per side of 2^24 points, the 2D Euler step 99.9 -> 25.6 ms at 4096^2 and 6.5 ->
-// 1.85 ms at 1024^2, the 1D step 2.63 -> 0.66 ms at 2^20 cells.
+// 1.24 -> 0.24 ms per side of 2^24 points, the 2D Euler step 99.9 -> 18.9 ms at 4096^2 and 6.5 ->
+// 1.53 ms at 1024^2, the 1D step 2.63 -> 0.52 ms at 2^20 cells.
 //
 // Precision.  Every quantity carries a 64-bit mantissa (block floating point: integers with a
 // common exponent), every truncation stays below that of a 53-bit one, so the result is
