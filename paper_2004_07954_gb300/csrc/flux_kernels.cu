@@ -177,10 +177,14 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMAL
 // interfaces (31 of them: neighbouring blocks both compute the interface they share) and
 // their LF speeds, in the arithmetic of update_kernel, so that a stage is one launch.
 // A CFL step at 200 and 8192 cells: 59 and 62 us with a thread per interface (64-thread blocks) and
-// an update launch, 39 and 47 us with
-// this flux kernel and the update launch, 30 and 32 us as one; advection at 160 cells 13 -> 8.5 us.
+// an update launch, 39 and 47 us with this flux kernel and the update launch, 29 and 32 us as one;
+// advection at 160 cells 13 -> 7.6 us.
+// Up to which length: as long as the blocks are one wave, six an SM (56 registers) for the default
+// scheme, five (64) for the generic ones.  A step as one launch a stage / by the 64-thread flux
+// kernel and the update: 28,000 cells 52 / 82 us, 32,768 76 / 72, 36,864 81 / 71, 60,000 118 / 101;
+// Steger-Warming 22,000 cells 60 / 90, 24,000 91 / 86; WENO-Z 45 / 72 and 73 / 70.
 constexpr int kLineTI = 32;
-constexpr int kLineMax = 24576;            // cells; 16384: 51 against 62 us a step, 30000: 74 against 69
+constexpr int line_max(bool gen) { return (gen ? 5 : 6) * 152 * (kLineTI - 1); }
 template <int NV> constexpr int kLineThreads = NV == 3 ? 192 : 64;
 
 template <int NV, int GEN, bool STAGE>
@@ -444,7 +448,7 @@ cudaError_t launch_flux_t(int system, int dir, const FluxArgs& a, cudaStream_t s
         if (system == 0)
             return small ? launch_one<1, 0, true, GEN, false>(a, s) : launch_one<1, 0, false, GEN, false>(a, s);
         if constexpr (GEN != 2)
-            if (a.nx < kLineMax)
+            if (a.nx < line_max(GEN != 0))
                 return launch_pdl(line_kernel<3, GEN, false>, dim3(unsigned((a.nx + kLineTI) / kLineTI)),
                                   dim3(kLineThreads<3>), 0, s, a, UpdateArgs{});
         if (small) return launch_one<3, 0, true, GEN, false>(a, s);
@@ -468,7 +472,8 @@ cudaError_t launch_flux_xy(const FluxArgs& ax, const FluxArgs& ay, cudaStream_t 
 }
 
 bool line_stage_applies(int system, const FluxArgs& a) {
-    return system != 2 && a.nx < kLineMax && (system == 0 || a.split == 0 || a.split == 3);
+    const bool gen = a.weights != 0 || (system == 1 && a.split != 0);
+    return system != 2 && a.nx < line_max(gen) && (system == 0 || a.split == 0 || a.split == 3);
 }
 
 cudaError_t launch_line_stage(int system, const FluxArgs& a, const UpdateArgs& u, cudaStream_t s) {

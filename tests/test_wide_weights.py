@@ -244,3 +244,21 @@ def test_gpu_linear_pass(orc, kind):
         for k, q in ((0, 0), (1 + axis, 1), (3, 2)):
             flux = (np.abs(U1[q]).max() * 10.0 + (np.abs(U1[2]).max() if q == 1 else 0.0)) * n
             assert np.abs(L[k] - L1[q]).max() <= 1e-14 * flux, (axis, k)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("split,weights,n", [(0, 0, 28271), (0, 0, 28272), (3, 0, 23559), (3, 0, 23560), (0, 1, 23559), (0, 1, 23560)])
+def test_gpu_line_kernel_limits(orc, split, weights, n):
+    """The longest lines of the one-launch stage kernel and the shortest beyond it: the RHS against
+    the oracle, at the tolerance of test_gpu_linear_pass."""
+    import torch
+    from paper_2004_07954_gb300 import build, inputs, wenozn as W
+    build.build()
+    dx = 10.0 / n
+    U = inputs.euler1d_ic(n, seed=5)
+    p = W.wenozn_problem_init(1, n, 1, dx, 1.0, split=split, weights=weights)
+    got = W.Solver(p).rhs(torch.from_numpy(U).cuda()).cpu().numpy()
+    want = orc.rhs(orc.problem(1, n, 1, dx=dx, split=split, weights=weights), U)
+    for k in range(3):
+        flux = (np.abs(U[k]).max() * 10.0 + (np.abs(U[2]).max() if k == 1 else 0.0)) / dx
+        assert np.abs(got[k] - want[k]).max() <= 1e-14 * flux, k
