@@ -374,7 +374,7 @@ struct WideProjection {
 // is not shown.  With the optimal weights the reconstruction is the same linear combination
 // in every field, and R L = 1 takes the projection out: F^ = h+_2 + h-_3 + lin(dh+) - lin(dh-)
 // per component, lin = (2 D1 - 11 D2 - 24 D3 + 3 D4)/60, sums of integers here, without an FP64
-// Roe state.  What the fields add to it, R times the sum of their
+// What the fields add to it, R times the sum of their
 //   Delta = sum c_k r_k (g_k - lin) / (1 + sum c_k r_k)   (wide_linear),
 // is evaluated in float with float eigenvectors: each field's D2, D3, their difference, the
 // second differences delta_0, delta_1 and d4 are projections of vectors differenced exactly in
@@ -382,6 +382,16 @@ struct WideProjection {
 // from the coefficients: 2^-19, more where c^2 is a small difference of H and u^2/2).  The
 // errors of r and of Delta follow from these, and the interface is accepted if they stay below
 // 2^-57 of every field's value.  Smooth data of some 40 cells a wave pass.
+//
+// Units.  Velocities are taken in units of 2^q, 2^(2q) the scale of H, and a difference of the
+// momenta's fluxes in units 2^q, of the energy's 2^(2q) times larger than the mass flux's, so
+// u, c, H and every field are of order one or less whatever the units of the data.  A small
+// float counts as proof only where nothing it came from can have been rounded away: variables
+// more than 2^126 below the largest enter with their scale raised to that (an error below 2^-120
+// in every magnitude), and a field's r is used only where every 1/b_k is below 2^84, with 2^-62
+// added to its error: products that fall below the float range then move r by less, and so does
+// R, held at 2^100 from there on (r < 4 (K d4)^2 / R there).  Elsewhere Delta counts as
+// unknown, |Delta| <= 0.34 (|delta_0| + |delta_1|) whatever the weights.
 template <int NV>
 struct FieldMagnitudes {                     // sums of the projections' terms: acoustic, entropy, shear
     float a, e, s;
@@ -404,11 +414,11 @@ struct FieldMagnitudes {                     // sums of the projections' terms: 
 // summed over the stencil, F its largest difference, in Delta's derivative 0.07 A |dr| + 2 r.
 template <int NV, bool ADJ>
 struct NearLinear {
-    int X[4], E;                               // the variables' exponents over both sides' vectors, the largest
+    int X[4], E, q;                            // the variables' exponents over both sides' vectors; the units' (below)
     int64_t S[NV];                             // 60 (lin(dh+) - lin(dh-)) per component, 2^(X_k - 1078)
-    float dl[NV];                              // 60 Delta of the fields, plus side - minus side, 2^(E - 1022)
+    float dl[NV];                              // 60 Delta of the fields, plus side - minus side, 2^(E - 1022) (shear: times 2^q)
     float val[2];                              // 2^-57 of the fields' values in the same units
-    float u, v, H, c2, rc, hq2;
+    float u, v, H, c2, rc, hq2;                // the Roe state in units of 2^q
     bool ok;
 
     __device__ __forceinline__ NearLinear(const CellPlanes<NV>& s, int base, int stride, double gm1,
@@ -426,20 +436,27 @@ struct NearLinear {
         X[1] = int(xa >> 16);
         X[2] = int(xb & 0xffffu);
         X[3] = int(xb >> 16);
-        E = max_i(max_i(X[0], X[1]), max_i(X[2], X[3]));
-        ok = E < kWideMaxExp;
-        // powers of two of the variables against the largest (0 for all-zero ones)
-        float sc[NV];
+        // the unit of velocity 2^q from the larger H; variables' exponents in units of 1, 2^q, 2^(2q)
+        q = (max_i(exponent_of(s.H[cl]), exponent_of(s.H[cr])) - 1023) >> 1;
+        ok = unsigned(q + 400) < 800u;
+        int Y[NV];
+        E = -4096;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const int e = X[k] - E + 127;
-            sc[k] = bits_float(uint32_t(X[k] == 0 || e < 0 ? 0 : e) << 23);
+            Y[k] = X[k] == 0 ? -8192 : X[k] - (k == 0 ? 0 : (k == NV - 1 ? 2 * q : q));
+            E = max_i(E, Y[k]);
+            // (infinities, NaN; differences whose linear part would leave the normal range)
+            ok = ok && (X[k] == 0 || unsigned(X[k] - 64) < unsigned(kWideMaxExp - 64));
         }
+        // powers of two of the variables against the largest
+        float sc[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) sc[k] = bits_float(uint32_t(max_i(Y[k] - E + 127, 1)) << 23);
         // the Roe state in float
         const float sl = wide_truncate(s.sr[cl]), wl = sl * float_rcp(sl + wide_truncate(s.sr[cr]));
-        const float ul = wide_truncate(s.un[cl]), ur = wide_truncate(s.un[cr]);
-        const float vl = NV == 4 ? wide_truncate(s.ut[cl]) : 0.0f, vr = NV == 4 ? wide_truncate(s.ut[cr]) : 0.0f;
-        const float Hl = wide_truncate(s.H[cl]), Hr = wide_truncate(s.H[cr]);
+        const float ul = wide_scaled(s.un[cl], q), ur = wide_scaled(s.un[cr], q);
+        const float vl = NV == 4 ? wide_scaled(s.ut[cl], q) : 0.0f, vr = NV == 4 ? wide_scaled(s.ut[cr], q) : 0.0f;
+        const float Hl = wide_scaled(s.H[cl], 2 * q), Hr = wide_scaled(s.H[cr], 2 * q);
         u = fmaf(wl, ul - ur, ur);
         v = fmaf(wl, vl - vr, vr);
         H = fmaf(wl, Hl - Hr, Hr);
@@ -450,15 +467,19 @@ struct NearLinear {
         rc = rsqrtf(c2);
         const float hrc = 0.5f * rc, hb1 = 0.5f * g1 * rc * rc, hb2 = hq2 * hb1;
         const float rel = 0x1p-21f * fmaf(2.0f * hb1, fabsf(H), 4.0f);
-        // R in the units of the differences, 2^(E - 1022)
-        const int er = wc.eR - 57 - 2 * E;
-        const float R = wc.Rf * bits_float(uint32_t((er < -126 ? -126 : (er > 60 ? 60 : er)) + 127) << 23);
-        const int e0 = max_i(exponent_of(s.hp[cl]), exponent_of(s.hm[cr]));
-        const int ew = NV == 4 ? max_i(exponent_of(s.hp[2 * NC + cl]), exponent_of(s.ut[cl]) + e0 - 1024) : 0;
+        // R in the units of the fields' squares (density's and shear's), 0 below 2^-126
+        float R[2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int ef = (q == 0 ? e0 - 2 : ew) - E + 126;
-            val[q] = 0x1p-57f * bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
+        for (int m = 0; m < 2; ++m) {
+            const int er = wc.eR - 57 - 2 * (m == 0 ? E : E + q);
+            R[m] = er < -126 ? 0.0f : wc.Rf * bits_float(uint32_t((er > 100 ? 100 : er) + 127) << 23);
+        }
+        const int e0 = max_i(exponent_of(s.hp[cl]), exponent_of(s.hm[cr]));
+        const int ew = NV == 4 ? max_i(exponent_of(s.hp[2 * NC + cl]), exponent_of(s.ut[cl]) + e0 - 1024) - q : 0;
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int ef = (m == 0 ? e0 - 2 : ew) - E + 126;
+            val[m] = 0x1p-57f * bits_float(uint32_t(ef < 0 ? 0 : (ef > 250 ? 250 : ef)) << 23);
         }
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
@@ -528,10 +549,13 @@ struct NearLinear {
                 }
                 const float f3 = f2 - s1, s0 = s1 + d0, s2 = s1 - d1, Q = d0 - d1;
                 const float A = fabsf(d0) + fabsf(d1), As = fabsf(s0) + fabsf(s2), Af = fabsf(f2) + fabsf(f3);
-                const float ef = rel * Mf.of(k), es = fmaf(rel, Ms.of(k), 0x1p-22f * Af), ed = fmaf(rel, Md.of(k), 0x1p-22f * A);
-                const float b0 = fmaf(4.0f * s0, s0, fmaf(3.0f * f2, f2 - s0, R)), b1 = fmaf(4.0f * s1, s1, fmaf(3.0f * f2, f3, R));
-                const float b2 = fmaf(4.0f * s2, s2, fmaf(3.0f * f3, f3 + s2, R));
-                const float T = fabsf(fmaf(4.0f * Q + 8.0f * d1, s0 + s2, 3.0f * fmaf(f3, d1, -(f2 * d0)))) + R;
+                const float ef = fmaf(rel, Mf.of(k), 0x1p-120f);
+                const float es = fmaf(rel, Ms.of(k), fmaf(0x1p-22f, Af, 0x1p-120f));
+                const float ed = fmaf(rel, Md.of(k), fmaf(0x1p-22f, A, 0x1p-120f));
+                const float Rk = R[NV == 4 && k == 2 ? 1 : 0];
+                const float b0 = fmaf(4.0f * s0, s0, fmaf(3.0f * f2, f2 - s0, Rk)), b1 = fmaf(4.0f * s1, s1, fmaf(3.0f * f2, f3, Rk));
+                const float b2 = fmaf(4.0f * s2, s2, fmaf(3.0f * f3, f3 + s2, Rk));
+                const float T = fabsf(fmaf(4.0f * Q + 8.0f * d1, s0 + s2, 3.0f * fmaf(f3, d1, -(f2 * d0)))) + Rk;
                 // (an error common to D2 and D3 enters f3 delta_1 - f2 delta_0 with delta_1 - delta_0 only)
                 const float ET = fmaf(ed, fmaf(8.0f, As + A, 6.0f * Af), fmaf(3.0f * ef, fabsf(Q) + ed, 11.0f * A * es));
                 const float i0f = float_rcp(b0), i1f = float_rcp(b1), i2f = float_rcp(b2), im = fmaxf(fmaxf(i0f, i1f), i2f);
@@ -541,18 +565,19 @@ struct NearLinear {
                 const float g1 = (fabsf(fmaf(8.0f, f2, -5.0f * f3)) + fabsf(fmaf(8.0f, f3, -5.0f * f2))) * i1f;
                 const float g2 = (fabsf(fmaf(20.0f, f3, -11.0f * F4)) + fabsf(fmaf(8.0f, F4, -11.0f * f3))) * i2f;
                 const float rho = 2.0f * (ef + es + ed) * fmaxf(fmaxf(g0, g1), g2);
-                const float x = wc.Kf * float_rcp(fminf(b0, b2) - 0.5f * R);
-                const float q = x * Q * T, rr = q * q;
+                const float x = wc.Kf * float_rcp(fminf(b0, b2) - 0.5f * Rk);
+                const float z = x * Q * T, rr = z * z;
                 // r's error (x, im: b's and h to within rho < 1/8; d4 to within 2 ed)
-                const float qa = fabsf(q), qe = fabsf(x) * fmaf(fabsf(Q) + 2.0f * ed, ET, 2.0f * ed * T);
-                const float err = im * fmaf(qe, fmaf(2.0f, qa, qe), rr * fmaf(8.0f, rho, 0x1p-13f)) * 2.0f;
+                const float za = fabsf(z), ze = fabsf(x) * fmaf(fabsf(Q) + 2.0f * ed, ET, 2.0f * ed * T);
+                const float err = fmaf(2.0f * im, fmaf(ze, fmaf(2.0f, za, ze), rr * fmaf(8.0f, rho, 0x1p-13f)), 0x1p-62f);
+                const bool known = rho < 0.125f && im <= 0x1p84f;
                 const float r0 = rr * i0f, r1 = 6.0f * rr * i1f, r2 = 3.0f * rr * i2f;
                 const float num = fmaf(r0, fmaf(18.0f, d0, -3.0f * d1),
                                        fmaf(r1, fmaf(-2.0f, d0, -3.0f * d1), r2 * fmaf(-2.0f, d0, 7.0f * d1)));
-                const bool zero = Af + A == 0.0f && ef + ed == 0.0f;
-                const float del = zero ? 0.0f : num * float_rcp(10.0f + (r0 + r1 + r2));
-                // |error of Delta| <= 0.07 (A + 2 ed) min(err, 1) + rounding of Delta and of R Delta
-                const float bound = fmaf(0.125f * (A + 2.0f * ed), rho < 0.125f ? fminf(err, 1.0f) : 1.0f,
+                const bool zero = Mf.of(k) + Md.of(k) == 0.0f;
+                const float del = zero || !known ? 0.0f : num * float_rcp(10.0f + (r0 + r1 + r2));
+                // |error of Delta| <= 0.07 (A + 2 ed) err + rounding of Delta and of R Delta
+                const float bound = fmaf(A + 2.0f * ed, known ? fminf(0.125f * err, 0.34f) : 0.34f,
                                          0x1p-22f * fabsf(del) + rel * fabsf(del));
                 const float vk = NV == 4 && k == 2 ? val[1] : val[0];
                 ok = ok && (zero || bound <= vk);
@@ -560,7 +585,7 @@ struct NearLinear {
                     const float xb = 2.0f * fabsf(x) * (T + ET), qb = xb * (fabsf(Q) + 2.0f * ed), rb = 2.0f * qb * qb * im;
                     const float F = Af + As + A, B = 0.07f * A * im * (xb * qb * 32.0f + qb * qb * F * 400.0f * float_rcp(T + ET) +
                                                                        rb * F * 300.0f) + 2.0f * rb;
-                    ok = ok && (zero || (rho < 0.125f && B <= 0x1p-53f && fabsf(del) <= 480.0f * vk));
+                    ok = ok && (zero || (known && B <= 0x1p-53f && fabsf(del) <= 480.0f * vk));
                 }
                 const float sd = side == 0 ? del : -del;
 #pragma unroll
@@ -592,9 +617,11 @@ __device__ __forceinline__ bool interface_linear(const CellPlanes<NV>& s, int ba
         dF[NV - 1] = fmaf(L.H, t, fmaf(L.u * c, d, fmaf(L.hq2, L.dl[1], NV == 4 ? L.v * L.dl[2] : 0.0f)));
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            // dF 2^(E - 1022) / 60 as a double, from the bits of dF/60
-            const uint32_t b = float_bits(dF[k] * (1.0f / 60.0f)), e = (b >> 23) & 0xffu;
-            if (e != 0) Fh[k] += bits_double(join((b & 0x80000000u) | (((b & 0x7fffffu) >> 3) + (uint32_t(int(e) + L.E - 126) << 20)), b << 29));
+            // dF 2^(E - 1022) / 60 in the variable's units as a double, from the bits of dF/60
+            const uint32_t b = float_bits(dF[k] * (1.0f / 60.0f));
+            const int e = int((b >> 23) & 0xffu), ex = e + L.E - 126 + (k == 0 ? 0 : (k == NV - 1 ? 2 * L.q : L.q));
+            if (e != 0 && unsigned(ex - 1) < 2046u)
+                Fh[k] += bits_double(join((b & 0x80000000u) | (((b & 0x7fffffu) >> 3) + (uint32_t(ex) << 20)), b << 29));
         }
     }
     return true;

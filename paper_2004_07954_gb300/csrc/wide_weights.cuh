@@ -484,6 +484,14 @@ WZ_HD float wide_truncate(double v) {
     return bits_float(a < (253u << 20) ? f : ((u << 1) == 0 ? 0u : 0x7fffffffu));
 }
 
+// v 2^-n as a float by truncation, |n| < 897; 0 below 2^-126, not a number from 2^127 on
+WZ_HD float wide_scaled(double v, int n) {
+    const uint64_t u = double_bits(v);
+    const uint32_t hi = uint32_t(u >> 32), a = (hi & 0x7fffffffu) - (uint32_t(897 + n) << 20);
+    const uint32_t f = funnel_l(uint32_t(u), a + (1u << 20), 3) | (hi & 0x80000000u);
+    return bits_float(a < (253u << 20) ? f : (int32_t(a) < 0 ? 0u : 0x7fffffffu));
+}
+
 // f^ - c where the weights hardly differ from the optimal ones; false where that is not shown.
 // With r_k = (K d4 T)^2 / (h^2 b_k) the weights are c_k (1 + r_k) (the other weight functions alike
 // with their own r_k), so f^ - c is the optimal
