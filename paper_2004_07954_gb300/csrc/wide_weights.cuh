@@ -256,28 +256,31 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
         f1 = eS - 2 * n1;
         f2 = eS - 2 * n2;
     } else {
-        // T = |b_0 - b_2| (+ R) with the larger's exponent, normalised
+        // T = |b_0 - b_2|, normalised (zero: exponent far below), then + R: R at its own scale, since
+        // on a tie T is R alone
         const bool lt = n0 < n2 || (n0 == n2 && b0 < b2);
         const uint64_t mx = lt ? b2 : b0, mn = lt ? b0 : b2;
         const int nx = lt ? n2 : n0, nn = lt ? n0 : n2;
-        uint64_t T = mx - shr_u64(mn, nx - nn) + (weights == 0 ? shr_u64(c.RM, nx - c.eR) : 0);
-        int eT = nx;
-        if ((T >> 32) == 0) {
-            T <<= 32;
-            eT -= 32;
-        }
+        uint64_t T = mx - shr_u64(mn, nx - nn);
+        const bool lowT = (T >> 32) == 0;
+        T = lowT ? T << 32 : T;
         const int nT = clz_u32(uint32_t(T >> 32) | 1u);
+        int eT = T == 0 ? -(1 << 20) : nx - (lowT ? 32 : 0) - nT;
         T <<= nT;
-        eT -= nT;
+        if (weights == 0) {
+            const int e = max_i(eT, c.eR) + 1;
+            T = shr_u64(T, e - eT) + shr_u64(c.RM, e - c.eR);
+            eT = e;
+        }
         uint64_t Y;
         int eY;
         if (weights == 1) {
             X = mul_hi(b01, b2);
             eX = 128;
             Y = T;
-            eY = T == 0 ? -(1 << 20) : eT + 128;
+            eY = eT + 128;
         } else {
-            // z = K |d4| T from normalised factors (both may have lost their leading bits);
+            // z = K |d4| T from normalised factors (T to within a bit);
             // X = h^2 b_0 b_1 b_2 with h = min - R/2, Y = z^2
             const int64_t c1 = shr_s64(x0, E - e0), c2 = shr_s64(x1, E - e1), c3 = shr_s64(x2, E - e2),
                           c4 = shr_s64(x3, E - e3);

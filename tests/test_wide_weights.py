@@ -103,6 +103,19 @@ def test_integer_evaluation_of_the_other_weights(wide, orc, name, weights, eps):
         assert np.all(np.abs(got - ref) <= _bound(f, ref, side)), side
 
 
+@pytest.mark.parametrize("eps,A", [(1e-40, 10.0), (1e-6, 1e-6), (1.0, 1e-6), (1e-6, 0.1)])
+def test_a_tie_leaves_eps_alone_in_the_weights(wide, orc, eps, A):
+    """b_0 = b_2 far above eps: tau5 + eps is eps, which has to keep its own precision (the module's
+    bound), for every size of the differences."""
+    for x in 10.0 ** np.arange(-12.0, 13.0):
+        for f in ([-x, 0.0, 0.0, 0.0, -x, 0.0], [-x, 0.0, 0.0, 0.0, -x, 0.4 * x], [3.0 * x, x, 0.0, x, 3.0 * x, 0.0]):
+            for side in (1, -1):
+                g = np.array(f if side > 0 else f[::-1])
+                got, refused = wide(g, side, eps, A)
+                ref = orc.reconstruct_quad(g, side, eps=eps, A=A)
+                assert refused == 0 and abs(got[0] - ref[0]) <= _bound(g, ref, side)[0], (x, f, side)
+
+
 def test_constant_data_are_exact_and_other_values_refused(wide):
     for c in (0.0, -0.0, 0.1, -3.7e200):
         got, refused = wide(np.full(40, c), 1)
