@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMAL
 // an update launch, 39 and 47 us with this flux kernel and the update launch, 29 and 32 us as one;
 // advection at 160 cells 13 -> 7.6 us.
 // Up to which length: as long as the blocks are one wave, six an SM (56 registers) for the default
-// scheme, five (64) for the generic ones.  A step as one launch a stage / by the 64-thread flux
+// scheme, five (64) for the generic ones (the launch bounds hold them there).  A step as one launch a stage / by the 64-thread flux
 // kernel and the update: 28,000 cells 52 / 82 us, 32,768 76 / 72, 36,864 81 / 71, 60,000 118 / 101;
 // Steger-Warming 22,000 cells 60 / 90, 24,000 91 / 86; WENO-Z 45 / 72 and 73 / 70.
 constexpr int kLineTI = 32;
@@ -188,7 +188,7 @@ constexpr int line_max(bool gen) { return (gen ? 5 : 6) * 152 * (kLineTI - 1); }
 template <int NV> constexpr int kLineThreads = NV == 3 ? 192 : 64;
 
 template <int NV, int GEN, bool STAGE>
-__global__ void __launch_bounds__(kLineThreads<NV>) line_kernel(FluxArgs a, UpdateArgs u) {
+__global__ void __launch_bounds__(kLineThreads<NV>, NV == 3 ? (GEN == 0 ? 6 : 5) : 1) line_kernel(FluxArgs a, UpdateArgs u) {
     constexpr int TI = kLineTI, NC = TI + 5, W = GEN == 0 ? 0 : -1, kThreads = kLineThreads<NV>;
     __shared__ double s_planes[NC * CellPlanes<NV>::kPerCellDefault];
     __shared__ double s_R[NV == 3 ? 8 : 1][TI], s_g[2][NV][TI];

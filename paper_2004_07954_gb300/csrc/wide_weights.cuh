@@ -28,6 +28,11 @@
 // and f^ - c = (a_0 g_0 + 6 a_1 g_1 + 3 a_2 g_2) / (6 (a_0 + 6 a_1 + 3 a_2)) with
 //   g_0 = 2 D1 - 5 D2,  g_1 = -(D2 + 2 D3),  g_2 = D4 - 4 D3.
 //
+// Signs.  f^ - c is odd in the differences and every step here is exactly odd or even in them:
+// shifts and products drop the low bits of magnitudes, never of two's complement values.  So a
+// stencil mirrored about its centre cell (D4 = -D1, D3 = -D2) has b_0 = b_2 to the last bit and
+// tau5 = 0 exactly: near a flat top a last bit of tau5 alone would decide the weights.
+//
 // Scales.  Each D_i comes with an exponent of its own.  A sub-stencil's pair takes the scale of
 // its larger difference, each weight a_k and each product a_k g_k an exponent of its own too,
 // so a flat sub-stencil beside a jump keeps its full relative accuracy (the result there is
@@ -92,6 +97,15 @@ WZ_HD int64_t shr_s64(int64_t x, int n) {            // n >= 0, the sign from 63
 #endif
 }
 
+// x, or ~|x| of a negative x, so that shifting drops bits of the magnitude; and x >> n from it,
+// toward zero
+WZ_HD int64_t ones(int64_t x) { return x - int64_t(uint64_t(x) >> 63); }
+
+WZ_HD int64_t shr_ones(int64_t o, int n) {
+    const int64_t r = shr_s64(o, n);
+    return r + int64_t(uint64_t(r) >> 63);
+}
+
 WZ_HD int clz_u32(uint32_t x) {                      // x > 0
 #ifdef __CUDA_ARCH__
     int r;
@@ -112,9 +126,9 @@ WZ_HD uint32_t funnel_l(uint32_t lo, uint32_t hi, int n) {      // high word of 
 
 WZ_HD int max_i(int a, int b) { return a > b ? a : b; }
 
-WZ_HD int leading_zeros6(uint64_t x) {               // of x, at most 6
+WZ_HD int leading_zeros4(uint64_t x) {               // of x, at most 4
     const int n = clz_u32(uint32_t(x >> 32) | 1u);
-    return n < 6 ? n : 6;
+    return n < 4 ? n : 4;
 }
 
 WZ_HD uint64_t join(uint32_t hi, uint32_t lo) { return (uint64_t(hi) << 32) | lo; }
@@ -144,13 +158,22 @@ struct Limbs {
 
 WZ_HD int64_t wide_mul(int32_t a, int32_t b) { return int64_t(a) * b; }
 
+WZ_HD int32_t wide_mul_hi(int32_t a, int32_t b) {    // floor(a b / 2^32)
+#ifdef __CUDA_ARCH__
+    return __mulhi(a, b);
+#else
+    return int32_t((int64_t(a) * b) >> 32);
+#endif
+}
+
 // b_k = beta_k + R of a sub-stencil: its second difference s and the factors p w of beta's
 // other part (beta = 4 s^2 + 3 p w) at the pair's scale, e its exponent: |2 s| <= 2^62,
-// |3 p|, |w| <= 3 2^60.  B in [2^63, 2^64), b = B 2^eb.
+// |3 p|, |w| <= 3 2^60.  B in [2^63, 2^64), b = B 2^eb.  (The low limbs' product counts with its
+// floor, so that the sum does not depend on which way p and w were split: it is even in them.)
 WZ_HD uint64_t wide_indicator(int64_t s, int64_t p, int64_t w, int e, const WideConst& c, int& eb) {
     const Limbs S(s + s), P(p + p + p), Wl(w);
     const int64_t main = wide_mul(S.h, S.h) + wide_mul(P.h, Wl.h);
-    const int64_t cross = wide_mul(S.h, S.l) + wide_mul(S.h, S.l) + wide_mul(P.h, Wl.l) + wide_mul(P.l, Wl.h);
+    const int64_t cross = wide_mul(S.h, S.l) + wide_mul(S.h, S.l) + wide_mul(P.h, Wl.l) + wide_mul(P.l, Wl.h) + wide_mul_hi(P.l, Wl.l);
     const uint64_t m = uint64_t(main + (cross >> 32)) + shr_u64(c.RM, 64 + 2 * e - c.eR);
     const int n = clz_u32(uint32_t(m >> 32));
     eb = 2 * e + 64 - n;
@@ -175,8 +198,9 @@ WZ_HD uint64_t wide_rcp(uint64_t d) {
 }
 
 // A double as a signed mantissa x, |x| in [2^59, 2^60), and its biased exponent e: the value is
-// x 2^(e - 1082).  Zeros and subnormals have e = 0 (a zero x = 0).
-WZ_HD int64_t wide_unpack(double v, int& e) {
+// x 2^(e - 1082).  Zeros and subnormals have e = 0 (a zero x = 0).  wide_unpack_ones gives ones(x)
+// (of -0.0: -1, which every shift takes to 0).
+WZ_HD int64_t wide_unpack_ones(double v, int& e) {
 #ifdef __CUDA_ARCH__
     const uint64_t u = uint64_t(__double_as_longlong(v));
 #else
@@ -186,7 +210,12 @@ WZ_HD int64_t wide_unpack(double v, int& e) {
     const uint32_t hi = uint32_t(u >> 32), sg = uint32_t(int32_t(hi) >> 31);
     e = int((hi >> 20) & 0x7ffu);
     const uint64_t m = join((hi & 0xfffffu) | (e ? 0x100000u : 0u), uint32_t(u)) << 7;
-    return int64_t((m ^ join(sg, sg)) - join(sg, sg));
+    return int64_t(m ^ join(sg, sg));
+}
+
+WZ_HD int64_t wide_unpack(double v, int& e) {
+    const int64_t o = wide_unpack_ones(v, e);
+    return o + int64_t(uint64_t(o) >> 63);
 }
 
 WZ_HD int64_t shl_s64(int64_t x, int n) {            // 0 <= n < 64
@@ -208,17 +237,18 @@ WZ_HD int64_t wide_normalise(int64_t D, int G, int& e) {
     return shl_s64(D, n);
 }
 
-// f^ - c from the differences x_i 2^(e_i - 1082), |x_i| in [2^59, 2^60] (or x_i = 0, e_i = 0).
+// f^ - c from the differences x_i 2^(e_i - 1082), |x_i| in [2^59, 2^60] (or x_i = 0, e_i = 0),
+// given as o_i = ones(x_i).
 // weights: 0 WENO-ZN, as above; 1 WENO-Z (q = 1), a_k = b_0 b_1 b_2 + |b_0 - b_2| b_i b_j; 3
 // Jiang-Shu, a_k = (b_i b_j)^2 (the linear weights, 2, are wide_linear's).
-WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e0, int e1, int e2, int e3,
+WZ_HD double wide_weighted(int64_t o0, int64_t o1, int64_t o2, int64_t o3, int e0, int e1, int e2, int e3,
                            const WideConst& c, int weights) {
     // the sub-stencils' pairs at their own scales
     const int g01 = max_i(e0, e1), g12 = max_i(e1, e2), g23 = max_i(e2, e3);
     const int E = max_i(g01, g23);
-    const int64_t p0 = shr_s64(x0, g01 - e0), q0 = shr_s64(x1, g01 - e1);
-    const int64_t p1 = shr_s64(x1, g12 - e1), q1 = shr_s64(x2, g12 - e2);
-    const int64_t p2 = shr_s64(x2, g23 - e2), q2 = shr_s64(x3, g23 - e3);
+    const int64_t p0 = shr_ones(o0, g01 - e0), q0 = shr_ones(o1, g01 - e1);
+    const int64_t p1 = shr_ones(o1, g12 - e1), q1 = shr_ones(o2, g12 - e2);
+    const int64_t p2 = shr_ones(o2, g23 - e2), q2 = shr_ones(o3, g23 - e3);
 
     // the indicators; a pair below the scale of eps enters at that scale (b_k is then R to
     // within rounding, and never loses its leading bits)
@@ -231,12 +261,12 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
             h01 = max_i(g01, c.e_min);
             h12 = max_i(g12, c.e_min);
             h23 = max_i(g23, c.e_min);
-            u0 = shr_s64(u0, h01 - g01);
-            v0 = shr_s64(v0, h01 - g01);
-            u1 = shr_s64(u1, h12 - g12);
-            v1 = shr_s64(v1, h12 - g12);
-            u2 = shr_s64(u2, h23 - g23);
-            v2 = shr_s64(v2, h23 - g23);
+            u0 = shr_ones(ones(u0), h01 - g01);
+            v0 = shr_ones(ones(v0), h01 - g01);
+            u1 = shr_ones(ones(u1), h12 - g12);
+            v1 = shr_ones(ones(v1), h12 - g12);
+            u2 = shr_ones(ones(u2), h23 - g23);
+            v2 = shr_ones(ones(v2), h23 - g23);
         }
         b0 = wide_indicator(u0 - v0, v0, v0 + v0 - u0, h01, c, n0);
         b1 = wide_indicator(u1 - v1, u1, v1, h12, c, n1);
@@ -282,8 +312,8 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
         } else {
             // z = K |d4| T from normalised factors (T to within a bit);
             // X = h^2 b_0 b_1 b_2 with h = min - R/2, Y = z^2
-            const int64_t c1 = shr_s64(x0, E - e0), c2 = shr_s64(x1, E - e1), c3 = shr_s64(x2, E - e2),
-                          c4 = shr_s64(x3, E - e3);
+            const int64_t c1 = shr_ones(o0, E - e0), c2 = shr_ones(o1, E - e1), c3 = shr_ones(o2, E - e2),
+                          c4 = shr_ones(o3, E - e3);
             const int64_t d23 = c2 - c3;
             const int64_t d4 = (c1 - c4) - (d23 + d23 + d23);
             uint64_t ad = uint64_t(d4 < 0 ? -d4 : d4);
@@ -308,31 +338,29 @@ WZ_HD double wide_weighted(int64_t x0, int64_t x1, int64_t x2, int64_t x3, int e
         f1 = eY - n1;
         f2 = eY - n2;
     }
-    // a_k below 2^59 with the exponent of its larger term's leading bit (at most six zeros counted)
-    const int tX = eX - leading_zeros6(X);
-    const int m0 = max_i(tX, f0 - leading_zeros6(Y0)) + 6;
-    const int m1 = max_i(tX, f1 - leading_zeros6(Y1)) + 6;
-    const int m2 = max_i(tX, f2 - leading_zeros6(Y2)) + 6;
+    // a_k below 2^61 with the exponent of its larger term's leading bit (at most four zeros counted)
+    const int tX = eX - leading_zeros4(X);
+    const int m0 = max_i(tX, f0 - leading_zeros4(Y0)) + 4;
+    const int m1 = max_i(tX, f1 - leading_zeros4(Y1)) + 4;
+    const int m2 = max_i(tX, f2 - leading_zeros4(Y2)) + 4;
     // with the optimal weights 1 : 6 : 3
     const uint64_t a0 = shr_u64(X, m0 - eX) + shr_u64(Y0, m0 - f0);
     const uint64_t a1 = (shr_u64(X, m1 - eX) + shr_u64(Y1, m1 - f1)) * 6;
     const uint64_t a2 = (shr_u64(X, m2 - eX) + shr_u64(Y2, m2 - f2)) * 3;
 
-    // numerator: products a_k g_k / 2^62, |.| < 2^61.3, each with its own exponent, summed at the
-    // largest (g_k: |p|, |q| <= 2^60; limbs |A_h| < 2^30, |G_h| < 2^31)
-    auto product = [](uint64_t a, int64_t g) {
-        const Limbs A{int64_t(a)}, G(g);
-        const int64_t cross = wide_mul(A.h, G.l) + wide_mul(A.l, G.h);
-        const int64_t top = wide_mul(A.h, G.h) + (cross >> 32);
-        return int64_t(join(funnel_l(uint32_t(top), uint32_t(uint64_t(top) >> 32), 2),
-                            funnel_l(uint32_t(cross), uint32_t(top), 2)));
+    // numerator: products a_k g_k / 2^64, each with its own exponent, summed at the largest
+    // (|g_k| <= 7 2^60, 3 2^60, 5 2^60: the sum stays below 2^62.4)
+    auto product = [](uint64_t a, int64_t g, int n) {
+        const int32_t s = int32_t(uint64_t(g) >> 32) >> 31;
+        const int64_t m = int64_t(shr_u64(mul_hi(a, uint64_t((g + s) ^ s)), n));
+        return (m ^ s) - s;
     };
     const int k0 = m0 + g01, k1 = m1 + g12, k2 = m2 + g23, km = max_i(max_i(k0, k1), k2);
-    const int64_t S = shr_s64(product(a0, p0 + p0 - 5 * q0), km - k0) - shr_s64(product(a1, p1 + q1 + q1), km - k1) +
-                      shr_s64(product(a2, q2 - 4 * p2), km - k2);
+    const int64_t S = product(a0, p0 + p0 - 5 * q0, km - k0) - product(a1, p1 + q1 + q1, km - k1) +
+                      product(a2, q2 - 4 * p2, km - k2);
     // denominator
     const int dm = max_i(max_i(m0, m1), m2);
-    uint64_t d = (shr_u64(a0, dm - m0) + shr_u64(a1, dm - m1) + shr_u64(a2, dm - m2)) * 3;
+    uint64_t d = (shr_u64(a0, dm + 2 - m0) + shr_u64(a1, dm + 2 - m1) + shr_u64(a2, dm + 2 - m2)) * 3;
     const int nd = clz_u32(uint32_t(d >> 32));
     d <<= nd;
     // |S|, normalised, times the reciprocal
@@ -509,13 +537,16 @@ WZ_HD float wide_scaled(double v, int n) {
 // data and differences at the rounding level of the value itself.  2^(eb - 1023) bounds that
 // value from below (eb <= 0: nothing is known of it).
 // About 150 instructions instead of 600 for a warp whose lanes are all accepted.
-WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
-                       const WideConst& c, int weights, double& corr) {
+// ODD: the differences come as ones(D_i), as wide_weighted's, for a result exactly odd in them;
+// else as D_i, rounded down (the bound holds either way).
+template <bool ODD>
+WZ_HD bool wide_linear(int64_t o1, int64_t o2, int64_t o3, int64_t o4, int G1, int G2, int G3, int G4, int eb, const WideConst& c, int weights, double& corr) {
     const int G = max_i(max_i(G1, G2), max_i(G3, G4));
-    const int64_t c1 = shr_s64(D1, G - G1 + 4), c2 = shr_s64(D2, G - G2 + 4);      // |c_i| <= 2^56
-    const int64_t c3 = shr_s64(D3, G - G3 + 4), c4 = shr_s64(D4, G - G4 + 4);
-    const int64_t s0 = c1 - c2, s1 = c2 - c3, s2 = c3 - c4, d0 = s0 - s1, d1 = s1 - s2;
-    const float f2 = wide_float(c2), f3 = wide_float(c3), S1 = wide_float(s1), E0 = wide_float(d0),
+    auto shifted = [](int64_t o, int n) { return ODD ? shr_ones(o, n) : shr_s64(o, n); };
+    const int64_t c1 = shifted(o1, G - G1 + 4), c2 = shifted(o2, G - G2 + 4);      // |c_i| <= 2^56
+    const int64_t c3 = shifted(o3, G - G3 + 4), c4 = shifted(o4, G - G4 + 4);
+    const int64_t c12 = c1 - c2, c23 = c2 - c3, c34 = c3 - c4, d0 = c12 - c23, d1 = c23 - c34;
+    const float f2 = wide_float(c2), f3 = wide_float(c3), S1 = wide_float(c23), E0 = wide_float(d0),
                 E1 = wide_float(d1), Q = wide_float(d0 - d1);
     const float S0 = S1 + E0, S2 = S1 - E1;
     const int er = c.eR - 57 - 2 * G;                         // R in the floats' units
@@ -572,6 +603,10 @@ WZ_HD bool wide_linear(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, i
 
 // The weighted evaluation as a call of its own: the warps of smooth data pass it by, and one copy
 // of its code serves every field (inlined four times it does not fit the instruction cache).
+// The projected differences of a stencil mirrored about its centre cell (a plateau of three cells
+// between equal neighbours) are so but for their truncations, five of the last places of
+// D_i: within eight (2^-57 of the projection's terms, its accuracy) they are made so exactly, or
+// tau5 would be noise where it is zero, and decide the weights ("Signs" above).
 // W: the weight function, -1 for the run-time value.
 template <int W>
 #ifdef __CUDACC__
@@ -581,10 +616,14 @@ inline
 #endif
 double wide_weighted_call(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, WideConst c,
                           int weights) {
+    if (G1 == G4 && G2 == G3 && uint64_t(D1 + D4 + 8) <= 16 && uint64_t(D2 + D3 + 8) <= 16) {
+        D4 = -D1;
+        D3 = -D2;
+    }
     int e0, e1, e2, e3;
     const int64_t x0 = wide_normalise(D1, G1, e0), x1 = wide_normalise(D2, G2, e1), x2 = wide_normalise(D3, G3, e2),
                   x3 = wide_normalise(D4, G4, e3);
-    return wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c, W < 0 ? weights : W);
+    return wide_weighted(ones(x0), ones(x1), ones(x2), ones(x3), e0, e1, e2, e3, c, W < 0 ? weights : W);
 }
 
 // Whether the largest difference lies in the range of the integer evaluation (E its exponent).
@@ -596,7 +635,7 @@ WZ_HD bool wide_in_range(int E) { return unsigned(E - kWideMinExp) < unsigned(kW
 template <int W>
 WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G1, int G2, int G3, int G4, int eb,
                            const WideConst& c, int weights, double& corr) {
-    if (wide_linear(D1, D2, D3, D4, G1, G2, G3, G4, eb, c, W < 0 ? weights : W, corr)) return true;
+    if (wide_linear<false>(D1, D2, D3, D4, G1, G2, G3, G4, eb, c, W < 0 ? weights : W, corr)) return true;
     corr = 0.0;
     int e0, e1, e2, e3;
     wide_normalise(D1, G1, e0);
@@ -614,14 +653,14 @@ template <int W>
 WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, int eb, const WideConst& c, int weights,
                            double& corr) {
     int e0, e1, e2, e3;
-    const int64_t x0 = wide_unpack(D1, e0), x1 = wide_unpack(D2, e1), x2 = wide_unpack(D3, e2),
-                  x3 = wide_unpack(D4, e3);
+    const int64_t o0 = wide_unpack_ones(D1, e0), o1 = wide_unpack_ones(D2, e1), o2 = wide_unpack_ones(D3, e2),
+                  o3 = wide_unpack_ones(D4, e3);
     const int E = max_i(max_i(e0, e1), max_i(e2, e3));
     corr = 0.0;
     if (!wide_in_range(E)) return E == 0;
-    if (wide_linear(x0, x1, x2, x3, e0, e1, e2, e3, eb, c, W < 0 ? weights : W, corr)) return true;
+    if (wide_linear<true>(o0, o1, o2, o3, e0, e1, e2, e3, eb, c, W < 0 ? weights : W, corr)) return true;
     if (W < 0 && weights == 2) return false;
-    corr = wide_weighted(x0, x1, x2, x3, e0, e1, e2, e3, c, W < 0 ? weights : W);
+    corr = wide_weighted(o0, o1, o2, o3, e0, e1, e2, e3, c, W < 0 ? weights : W);
     return true;
 }
 

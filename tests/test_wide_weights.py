@@ -116,6 +116,33 @@ def test_a_tie_leaves_eps_alone_in_the_weights(wide, orc, eps, A):
                 assert refused == 0 and abs(got[0] - ref[0]) <= _bound(g, ref, side)[0], (x, f, side)
 
 
+@pytest.mark.parametrize("A", [10.0, 1e-6])
+def test_stencils_mirrored_about_their_centre(wide, orc, A):
+    """D4 = -D1, D3 = -D2: tau5 = 0 exactly, however flat the top is (the module's bound)."""
+    y = np.concatenate([10.0 ** -np.arange(1.0, 17.0), 2.0 ** -np.arange(1.0, 50.0), [0.0]])
+    for D1, D2 in ((y - 1.0, y), (-np.ones_like(y), y), (1.0 + y, -y)):
+        for sixth in (0.0, 0.3):
+            for a, b in zip(D1, D2):
+                f = np.array([a + b, b, 0.0, b, a + b, sixth])
+                for side in (1, -1):
+                    g = f if side > 0 else f[::-1].copy()
+                    got, refused = wide(g, side, 1e-40, A)
+                    ref = orc.reconstruct_quad(g, side, eps=1e-40, A=A)
+                    assert refused == 0 and abs(got[0] - ref[0]) <= _bound(g, ref, side)[0], (a, b, side)
+
+
+@pytest.mark.parametrize("weights", [0, 1, 2, 3])
+@pytest.mark.parametrize("name", list(_lines()) + ["single precision"])
+def test_odd_in_the_data_and_mirrored_between_the_sides(wide, name, weights):
+    """f^(-f) = -f^(f), and the plus side is the minus side of the reversed line, bit for bit."""
+    f = _lines()[name] if name in _lines() else np.random.default_rng(3).normal(size=3006).astype(np.float32).astype(np.float64)
+    for scale in (1.0, 2.0 ** -100):
+        g = np.ascontiguousarray(f * scale)
+        got = wide(g, 1, weights=weights)[0]
+        assert np.array_equal(wide(-g, 1, weights=weights)[0], -got)
+        assert np.array_equal(wide(g[::-1].copy(), -1, weights=weights)[0][::-1], got)
+
+
 def test_constant_data_are_exact_and_other_values_refused(wide):
     for c in (0.0, -0.0, 0.1, -3.7e200):
         got, refused = wide(np.full(40, c), 1)
