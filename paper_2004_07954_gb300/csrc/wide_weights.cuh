@@ -643,7 +643,8 @@ WZ_HD bool wide_correction(int64_t D1, int64_t D2, int64_t D3, int64_t D4, int G
     wide_normalise(D3, G3, e2);
     wide_normalise(D4, G4, e3);
     const int E = max_i(max_i(e0, e1), max_i(e2, e3));
-    if (!wide_in_range(E) || (W < 0 && weights == 2)) return E == 0;
+    // (constant data; other differences below 2^-1022 are not zero)
+    if (!wide_in_range(E) || (W < 0 && weights == 2)) return (D1 | D2 | D3 | D4) == 0;
     corr = wide_weighted_call<W>(D1, D2, D3, D4, G1, G2, G3, G4, c, weights);
     return true;
 }
@@ -657,7 +658,7 @@ WZ_HD bool wide_correction(double D1, double D2, double D3, double D4, int eb, c
                   o3 = wide_unpack_ones(D4, e3);
     const int E = max_i(max_i(e0, e1), max_i(e2, e3));
     corr = 0.0;
-    if (!wide_in_range(E)) return E == 0;
+    if (!wide_in_range(E)) return ((double_bits(D1) | double_bits(D2) | double_bits(D3) | double_bits(D4)) << 1) == 0;
     if (wide_linear<true>(o0, o1, o2, o3, e0, e1, e2, e3, eb, c, W < 0 ? weights : W, corr)) return true;
     if (W < 0 && weights == 2) return false;
     corr = wide_weighted(o0, o1, o2, o3, e0, e1, e2, e3, c, W < 0 ? weights : W);

@@ -153,6 +153,31 @@ def test_constant_data_are_exact_and_other_values_refused(wide):
         assert wide(f, 1)[1] > 0
 
 
+def test_differences_below_the_normal_range_are_refused(wide):
+    """They are no zeros: the double evaluation has to take them."""
+    f = np.random.default_rng(1).integers(-2 ** 40, 2 ** 40, size=46) * 5e-324
+    for side in (1, -1):
+        assert wide(f, side)[1] == 41
+        assert wide(np.where(np.arange(46) < 23, f, f[22]), side)[1] < 41
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("weights", [0, 1, 2, 3])
+def test_gpu_reconstruction_of_subnormal_data(orc, weights):
+    """Against the binary128 evaluation, to the last places of the subnormal range: the double
+    evaluation's differences are exact there, its weights off by 1e-12 at most."""
+    import torch
+    from paper_2004_07954_gb300 import build, wenozn as W
+    build.build()
+    f = np.random.default_rng(1).integers(-2 ** 50, 2 ** 50, size=606) * 5e-324
+    out = torch.empty(601, dtype=torch.float64, device="cuda")
+    for side in (1, -1):
+        W.wenozn_reconstruct_weights(torch.from_numpy(f).cuda(), out, side, weights)
+        ref = orc.reconstruct_quad(f, side, kind=weights)
+        # (in units of the smallest double, which 1e-12 of the data is about a thousandth of)
+        assert np.abs((out.cpu().numpy() - ref) / 5e-324).max() <= 4 + 1e-12 * 2 ** 50
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("k", [-320, -301, -300, -299, 0, 398, 399, 400])
 def test_gpu_reconstruction_across_the_range_switch(orc, k):
