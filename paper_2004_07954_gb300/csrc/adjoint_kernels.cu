@@ -132,11 +132,11 @@ struct EulerSmem {
     int64_t dp[3][NC], dm[3][NC];       // mantissas of the split fluxes' differences
     uint32_t ex[4][NC];                 // and their exponents (CellPlanes)
     // the six-warp form's: the field's weights are the optimal ones; each warp's copy of the
-    // remaining interfaces; their Roe states (u~, H~, 1/c, (gamma-1)/c^2, 1/(sqrt(rhoL) + sqrt(rhoR)));
-    // and the exchange between their threads, per field: cotangents of its projected h+ (5) and
+    // remaining interfaces; every interface's Roe state (u~, H~, 1/c, (gamma-1)/c^2,
+    // 1/(sqrt(rhoL) + sqrt(rhoR)), c, u~^2 (gamma-1)/(2 c^2)) and flux cotangent; and the exchange between their threads, per field: cotangents of its projected h+ (5) and
     // h- (5), half its left-eigenvector row (3), 6 Roe scalars of either side
     unsigned char lin[WIDE ? 1 : 3][TI], list[WIDE ? 1 : 6][TI];
-    double roe[WIDE ? 1 : 5][WIDE ? 1 : TI];
+    double roe[WIDE ? 1 : 7][WIDE ? 1 : TI], Fb[WIDE ? 1 : 3][WIDE ? 1 : TI];
     double red[WIDE ? 1 : 3][WIDE ? 1 : 25][WIDE ? 1 : TI];
 };
 
@@ -177,17 +177,18 @@ constexpr int kGhostSlot = 6 * 9;       // 6 ghost cells x (flux, LF, Roe) x 3 c
 constexpr int kEnt = 7;                 // pending corrections of a record: 6 ghost targets + the argmax
 constexpr int kTIWide = 64;             // interfaces a block of the one-thread-per-interface kernel
 // Lines of at least this many cells take the one-thread-per-interface kernel: fewer FP64
-// instructions where every interface is nonlinear (no copies of the Roe state, the fields'
-// cotangents summed in registers, 5 of 64 interfaces computed twice instead of 5 of 32);
-// shorter ones need the other kernel's six times as many warps, and its two blocks an SM end
-// with the slowest.  A reverse step (three launches) in us, six threads / one thread an interface:
-// smooth waves 8192 cells 85 / 164, 16384 118 / 166, 131071 514 / 406; random cells (every
-// interface nonlinear) 114 / 170 at 8192, 217 / 175 at 16384, 1629 / 1165 at 131071: the line lies
-// where neither kind of data loses.  With three threads an interface (both sides in turn, no
-// compaction) 8192 cells of smooth waves took 103.
-// Where the time of a block with nonlinear interfaces goes (200 cells, 45 thousand cycles): cells
-// 7, the linear check 2.5, the reverses 23 (two warps on the busiest sub-partition, 230 FP64
-// instructions of 64 cycles each), gathering their results 8, the rest 5; without any, 20 in all.
+// instructions where every interface is nonlinear (the fields' cotangents summed in registers, 5 of
+// 64 interfaces computed twice instead of 5 of 32); shorter ones need the other kernel's six
+// times as many warps, and its two blocks an SM end with the slowest.  A reverse step (three
+// launches) in us, six threads / one thread an interface: random cells (every interface
+// nonlinear) 10240 cells 161 / 168, 12288 195 / 169, 16384 199 / 170, 131071 1629 / 1156; smooth
+// waves 101 / 168, 132 / 168, 133 / 170, 514 / 431: the line lies where neither kind of data
+// loses.  At 8192 cells 106 on random cells, 103 on smooth waves (an FP64 kernel without the
+// check, three threads an interface: 107 on either).
+// The one-thread kernel makes the linear check only where its blocks are more than one wave, two
+// an SM: a single wave waits for the blocks that hold a nonlinear interface, and pays for the
+// check as well.  With / without it: smooth waves 16384 cells 175 / 171, 20000 180 / 299, 65536
+// 364 / 584; random cells 173 / 170, 299 / 295, 593 / 584.
 constexpr int kWideMinCells = 10240;
 
 template <int TI, bool WIDE>
@@ -450,7 +451,8 @@ __global__ void __launch_bounds__(WIDE ? TI : 6 * TI, WIDE ? 1 : 2) vjp_stage_eu
     planes.dp = &sm.dp[0][0];
     planes.dm = &sm.dm[0][0];
     planes.ex = &sm.ex[0][0];
-    for (int c = tid; c < kCells - 1; c += kThreads) cell_diffs<3>(planes, c, 1);
+    if (!WIDE || a.check)
+        for (int c = tid; c < kCells - 1; c += kThreads) cell_diffs<3>(planes, c, 1);
     // the block's lowest candidate: offered for the global argmax (the lowest index on ties),
     // with d(|u| + c)/dU of its state left in the record (|x|' = 0 at 0)
     if (tid == kCand && S.cand < n) {
@@ -535,15 +537,34 @@ __global__ void __launch_bounds__(WIDE ? TI : 6 * TI, WIDE ? 1 : 2) vjp_stage_eu
     // coefficients times the flux cotangent.
     bool lin = false;
     if (WIDE) {
-        if (live) lin = NearLinear<3, true>(planes, i, 1, gm1, a.wide, 0, 3).ok;
+        if (live && a.check) lin = NearLinear<3, true>(planes, i, 1, gm1, a.wide, 0, 3).ok;
     } else {
-        if (live && w < 3) sm.lin[w][i] = NearLinear<3, true>(planes, i, 1, gm1, a.wide, w, w + 1).ok;
+        // (a field's check per warp; meanwhile the others form the Roe states and the flux
+        // cotangents once: in each of an interface's six threads they were 32 of 213 FP64 instructions)
+        if (live) {
+            if (w < 3) {
+                sm.lin[w][i] = NearLinear<3, true>(planes, i, 1, gm1, a.wide, w, w + 1).ok;
+            } else if (w == 3) {
+                const double sl = sm.sq[cl], rS = rcp_nr(sl + sm.sq[cr]), wl = sl * rS, wr = sm.sq[cr] * rS;
+                const double ut = fma(wl, sm.u[cl], wr * sm.u[cr]), Ht = fma(wl, sm.H[cl], wr * sm.H[cr]);
+                const double c2 = gm1 * fma(-0.5 * ut, ut, Ht), rc = inv_sqrt(c2), b1 = gm1 * rc * rc;
+                sm.roe[0][i] = ut;
+                sm.roe[1][i] = Ht;
+                sm.roe[2][i] = rc;
+                sm.roe[3][i] = b1;
+                sm.roe[4][i] = rS;
+                sm.roe[5][i] = c2 * rc;
+                sm.roe[6][i] = 0.5 * ut * ut * b1;
+            } else if (w == 4) {
+                for (int m = 0; m < 3; ++m) sm.Fb[m][i] = (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx;   // cells j, j - 1
+            }
+        }
         __syncthreads();
         if (live) lin = sm.lin[0][i] & sm.lin[1][i] & sm.lin[2][i];
     }
     double Fb[3] = {0.0, 0.0, 0.0};
     if (live)
-        for (int m = 0; m < 3; ++m) Fb[m] = (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx;   // cells j, j - 1
+        for (int m = 0; m < 3; ++m) Fb[m] = WIDE ? (S.lamw[m][i + 1] - S.lamw[m][i]) * a.rdx : sm.Fb[m][i];
     double ab = 0.0;
     if constexpr (!WIDE) {
         // Six threads per remaining interface, one per (field, side): the field's projection,
@@ -558,15 +579,10 @@ __global__ void __launch_bounds__(WIDE ? TI : 6 * TI, WIDE ? 1 : 2) vjp_stage_eu
             __syncwarp();
             if (tid < 6 * nrest) {
                 const int fs = tid / nrest, x = sm.list[w][tid - fs * nrest], k = fs >> 1, side = fs & 1;
-                const double sl = sm.sq[x + 2], sr = sm.sq[x + 3], rS = rcp_nr(sl + sr), wl = sl * rS, wr = sr * rS;
-                const double ut = fma(wl, sm.u[x + 2], wr * sm.u[x + 3]), Ht = fma(wl, sm.H[x + 2], wr * sm.H[x + 3]);
-                const double c2 = gm1 * fma(-0.5 * ut, ut, Ht), rc = inv_sqrt(c2), c = c2 * rc;
-                const double b1 = gm1 * rc * rc, b2 = 0.5 * ut * ut * b1;
+                const double ut = sm.roe[0][x], Ht = sm.roe[1][x], rc = sm.roe[2][x], b1 = sm.roe[3][x], c = sm.roe[5][x];
                 double L0, L1, L2, R1, R2;
-                field_lr(k, ut, Ht, c, rc, b1, b2, L0, L1, L2, R1, R2);
-                double G[3];
-#pragma unroll
-                for (int m = 0; m < 3; ++m) G[m] = (S.lamw[m][x + 1] - S.lamw[m][x]) * a.rdx;
+                field_lr(k, ut, Ht, c, rc, b1, sm.roe[6][x], L0, L1, L2, R1, R2);
+                const double G[3] = {sm.Fb[0][x], sm.Fb[1][x], sm.Fb[2][x]};
                 // the five points in the order of the side's stencil
                 const double* h = side == 0 ? &sm.hp[0][x] : &sm.hm[0][x + 5];
                 const int step = side == 0 ? 1 : -1;
@@ -585,9 +601,6 @@ __global__ void __launch_bounds__(WIDE ? TI : 6 * TI, WIDE ? 1 : 2) vjp_stage_eu
                 }
                 if (side == 0) {
                     sm.red[k][10][x] = 0.5 * L0; sm.red[k][11][x] = 0.5 * L1; sm.red[k][12][x] = 0.5 * L2;
-                }
-                if (fs == 0) {
-                    sm.roe[0][x] = ut; sm.roe[1][x] = Ht; sm.roe[2][x] = rc; sm.roe[3][x] = b1; sm.roe[4][x] = rS;
                 }
                 double q[6];
                 field_lr_reverse(k, Lb, G[1] * gh, G[2] * gh, ut, c, rc, b1, q);
@@ -1023,9 +1036,12 @@ cudaError_t launch_vjp(int system, const VjpArgs& a, cudaStream_t s) {
         if (e == cudaSuccess) e = launch_pdl(vjp_gather_advection, dim3(gc), dim3(kGather), 0, s, a);
         return e;
     }
-    if (a.n >= kWideMinCells)
-        return launch_pdl(vjp_stage_euler<kTIWide, true>, dim3(unsigned((a.n + kTIWide - 6) / (kTIWide - 5))),
-                          dim3(kTIWide), 0, s, a);
+    if (a.n >= kWideMinCells) {
+        VjpArgs w = a;
+        const int blocks = (a.n + kTIWide - 6) / (kTIWide - 5);
+        w.check = blocks > 2 * sm_count_cached();
+        return launch_pdl(vjp_stage_euler<kTIWide, true>, dim3(unsigned(blocks)), dim3(kTIWide), 0, s, w);
+    }
     size_t pad = 0;
     cudaError_t e = euler_interface_pad(&pad);
     if (e == cudaSuccess)

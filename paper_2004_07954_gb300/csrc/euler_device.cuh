@@ -486,8 +486,9 @@ struct NearLinear {
             S[k] = 0;
             dl[k] = 0.0f;
         }
+        // (a thread whose interface is refused is done: warps at fronts and in rough data leave early)
 #pragma unroll 1
-        for (int side = 0; side < 2; ++side) {
+        for (int side = 0; side < 2 && ok; ++side) {
             const int64_t* pl = side == 0 ? s.dp : s.dm;
             const uint32_t* ex = s.ex + 2 * side * NC;
             const int step = side == 0 ? stride : -stride;
@@ -538,7 +539,7 @@ struct NearLinear {
             // (a rolled loop: the code of the interface phases is larger than the instruction cache's
             // first level as it is)
 #pragma unroll 1
-            for (int k = k0; k < k1; ++k) {
+            for (int k = k0; k < k1 && ok; ++k) {
                 float f2 = P[0][0], s1 = P[1][0], d0 = P[2][0], d1 = P[3][0];
 #pragma unroll
                 for (int m = 1; m < NV; ++m) {

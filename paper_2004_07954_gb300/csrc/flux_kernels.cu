@@ -429,16 +429,6 @@ cudaError_t launch_one(const FluxArgs& a, cudaStream_t s) {
     return launch_pdl(flux_kernel<NV, DIR, SMALL, GEN, LIN>, grid, dim3(Tile<NV, SMALL>::THREADS), smem, s, a);
 }
 
-int sm_count_cached() {
-    static int sms = 0;
-    if (sms > 0) return sms;
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-        sms = v;
-    return sms > 0 ? sms : 152;
-}
-
 template <int GEN>
 cudaError_t launch_flux_t(int system, int dir, const FluxArgs& a, cudaStream_t s) {
     if (system != 2) {

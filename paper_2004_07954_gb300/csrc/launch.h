@@ -122,6 +122,17 @@ cudaError_t launch_batch_stage(int shape, const BatchArgs& a, int sms, cudaStrea
 constexpr int kVjpRecs = 5;
 constexpr int kVjpPend = 3;
 
+// SMs of the device (the same on every GB300; looked up once).
+inline int sm_count_cached() {
+    static int sms = 0;
+    if (sms > 0) return sms;
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
+        sms = v;
+    return sms > 0 ? sms : 152;
+}
+
 struct VjpArgs {
     const double* U;                       // stage input, [nv][n]
     const double* lam;                     // cotangent of L(U), [nv][n]
@@ -139,6 +150,7 @@ struct VjpArgs {
     int n, bc;
     double rdx, gamma, eps4, kappa, adv_speed;
     WideConst wide;                        // the weights' constants for the linear check (wide_weights.cuh)
+    int check;                             // long lines: whether the check is made (set by launch_vjp)
     int rec_out;                           // the record this launch writes
     int prec[kVjpPend];                    // records with corrections pending on the inputs (-1: none)
     int lam_slot;                          // index into prec of lam's record (-1: none)

@@ -340,3 +340,22 @@ def test_rhs_vjp_with_few_nonlinear_interfaces(wz, orc, kinks, bc):
         wz.wenozn_rhs_vjp(p, dev(U), dev(lam), out, ws)
         a, b = float(np.sum(lam * Jv)), float(np.sum(out.cpu().numpy() * v))
         assert b == pytest.approx(a, rel=1e-10, abs=1e-12 * np.abs(lam).sum() * np.abs(Jv).max())
+
+
+@pytest.mark.parametrize("n", [10239, 10240, 17936, 17937])
+@pytest.mark.parametrize("rough", [False, True])
+def test_rhs_vjp_at_the_limits_of_the_stage_kernels(wz, orc, n, rough):
+    """Six threads an interface, one thread without the linear check (its blocks a single wave, 304 of
+    59 cells), one thread with it; the tolerance of test_rhs_vjp_dot_product."""
+    p, P = _problem(wz, orc, 1, n, 10.0 / n, 0)
+    g = np.random.default_rng(8)
+    U = inputs.adjoint_ic(n, 1)
+    if rough:
+        U = U * (1.0 + 0.01 * g.random(U.shape))
+    ws = wz.vjp_workspace(p)
+    v, lam = g.normal(size=U.shape), g.normal(size=U.shape)
+    _, Jv = orc.rhs_jvp_quad(P, U, v)
+    out = torch.empty_like(dev(U))
+    wz.wenozn_rhs_vjp(p, dev(U), dev(lam), out, ws)
+    a, b = float(np.sum(lam * Jv)), float(np.sum(out.cpu().numpy() * v))
+    assert b == pytest.approx(a, rel=1e-10, abs=1e-12 * np.abs(lam).sum() * np.abs(Jv).max())
