@@ -116,6 +116,23 @@ def test_a_tie_leaves_eps_alone_in_the_weights(wide, orc, eps, A):
                 assert refused == 0 and abs(got[0] - ref[0]) <= _bound(g, ref, side)[0], (x, f, side)
 
 
+@pytest.mark.parametrize("scale", [2.0 ** -320, 2.0 ** -300, 2.0 ** -290, 1.0, 2.0 ** 390, 2.0 ** 399])
+@pytest.mark.parametrize("name", list(_lines()))
+def test_every_stencil_is_right_or_refused_by_its_range(wide, orc, name, scale):
+    """Stencil by stencil: refused exactly where the largest difference leaves [2^-300, 2^400), unless
+    all are zero; every other one within the bound."""
+    f = np.ascontiguousarray(_lines()[name] * scale)
+    for side in (1, -1):
+        ref = orc.reconstruct_quad(f, side)
+        bound = _bound(f, ref, side)
+        d = np.abs(np.diff(f))
+        for j in range(ref.size):
+            dmax = d[j:j + 4].max() if side > 0 else d[j + 1:j + 5].max()
+            got, refused = wide(f[j:j + 6].copy(), side)
+            assert bool(refused) == (dmax != 0.0 and not 2.0 ** -300 <= dmax < 2.0 ** 400), (j, side)
+            assert refused or abs(got[0] - ref[j]) <= bound[j], (j, side)
+
+
 @pytest.mark.parametrize("A", [10.0, 1e-6])
 def test_stencils_mirrored_about_their_centre(wide, orc, A):
     """D4 = -D1, D3 = -D2: tau5 = 0 exactly, however flat the top is (the module's bound)."""
@@ -159,6 +176,43 @@ def test_differences_below_the_normal_range_are_refused(wide):
     for side in (1, -1):
         assert wide(f, side)[1] == 41
         assert wide(np.where(np.arange(46) < 23, f, f[22]), side)[1] < 41
+
+
+def test_integer_reciprocal_square_root_and_halves(tmp_path):
+    """wide_reciprocal and wide_rsqrt to 0.506 of a last place over their ranges (the comments' figure,
+    with the host's seeds), wide_half and wide_truncate to the bit."""
+    src, so = str(tmp_path / "f.cpp"), str(tmp_path / "f.so")
+    with open(src, "w") as fh:
+        fh.write("""#include "wide_weights.cuh"
+extern "C" void f(const double* x, long n, double* r, double* q, double* h, float* t) {
+    bool ok;
+    for (long i = 0; i < n; ++i) {
+        r[i] = wz::wide_reciprocal(x[i]);
+        q[i] = wz::wide_rsqrt(x[i], ok);
+        h[i] = wz::wide_half(x[i]);
+        t[i] = wz::wide_truncate(x[i]);
+    }
+}""")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
+    g = np.random.default_rng(2)
+    p = 2.0 ** np.arange(-1000.0, 1001.0)
+    x = np.concatenate([p, np.nextafter(p, 0), np.nextafter(p, np.inf), g.uniform(1, 4, 20000) * 2.0 ** g.integers(-1000, 999, 20000)])
+    r, q, h, t = np.empty_like(x), np.empty_like(x), np.empty_like(x), np.empty(x.size, np.float32)
+    P = ctypes.c_void_p
+    L = ctypes.CDLL(so)
+    L.f.argtypes = [P, ctypes.c_long, P, P, P, P]
+    L.f(x.ctypes.data, x.size, r.ctypes.data, q.ctypes.data, h.ctypes.data, t.ctypes.data)
+    from fractions import Fraction as F
+    for xi, ri, qi in zip(x[::7].tolist(), r[::7].tolist(), q[::7].tolist()):
+        ulp = F(float(np.spacing(ri)))
+        assert abs(F(ri) - 1 / F(xi)) <= F(506, 1000) * ulp, xi
+        # |q - 1/sqrt(x)| <= e  <=>  (q - e)^2 x <= 1 <= (q + e)^2 x
+        e = F(506, 1000) * F(float(np.spacing(qi)))
+        assert (F(qi) - e) ** 2 * F(xi) <= 1 <= (F(qi) + e) ** 2 * F(xi), xi
+    assert np.array_equal(h, 0.5 * x)
+    y = (x.view(np.uint64) & np.uint64(0xFFFFFFFFE0000000)).view(np.float64)          # 24 bits kept
+    inside = (x >= 2.0 ** -126) & (x < 2.0 ** 127)
+    assert np.array_equal(t[inside].astype(np.float64), y[inside]) and np.all(np.isnan(t[~inside]))
 
 
 @pytest.mark.gpu
