@@ -183,8 +183,10 @@ __global__ void __launch_bounds__(Tile<NV, SMALL>::THREADS, (min_blocks<NV, SMAL
 // scheme, five (64) for the generic ones (the launch bounds hold them there).  A step as one launch a stage / by the 64-thread flux
 // kernel and the update: 28,000 cells 52 / 82 us, 32,768 76 / 72, 36,864 81 / 71, 60,000 118 / 101;
 // Steger-Warming 22,000 cells 60 / 90, 24,000 91 / 86; WENO-Z 45 / 72 and 73 / 70.
+// (Those are 152 SMs.)  Advection's blocks hold 64 threads and more of them fit; it takes the
+// same limit, on whose near side the one launch wins as well (28,000 cells 15.1 / 18.9 us).
 constexpr int kLineTI = 32;
-constexpr int line_max(bool gen) { return (gen ? 5 : 6) * 152 * (kLineTI - 1); }
+int line_max(bool gen) { return (gen ? 5 : 6) * sm_count_cached() * (kLineTI - 1); }
 template <int NV> constexpr int kLineThreads = NV == 3 ? 192 : 64;
 
 template <int NV, int GEN, bool STAGE>

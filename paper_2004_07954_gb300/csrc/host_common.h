@@ -126,7 +126,7 @@ inline UpdateArgs update_args(const wenozn_problem& p, Ctrl* ctrl, const double*
 }
 
 // One RK stage (or, mode 0, the RHS): the fluxes of stage input U and the update u, in one launch
-// for short lines.
+// for short lines (never in place, where the pair still is right: wenozn_rk3_run_keep with S1 = S2).
 inline cudaError_t launch_stage(const wenozn_problem& p, const double* U, const unsigned long long* alpha_bits,
                                 const unsigned long long* alpha_f_bits, double* fx, double* gy, const UpdateArgs& u,
                                 cudaStream_t s) {

@@ -467,9 +467,10 @@ WZ_HD double wide_reciprocal(double x) {
 }
 
 // 1 / sqrt(x) of a positive normal x: the float approximation Y0 of y = 1/sqrt(t), t in [1/4, 1)
-// the mantissa with an even exponent, and one step of y = y0 (1 + h/2 + 3/8 h^2 + ...),
-// h = 1 - t y0^2 < 2^-19 in units of 2^-62, so the truncated terms are below 2^-59 and the result
-// is within 2^-59 before its rounding to 53 bits.  Where x is not positive and normal: ok = false.
+// the mantissa with an even exponent, and one step of Householder's third-order iteration,
+// y = y0 (1 + h/2 + 3/8 h^2 + ...), h = 1 - t y0^2 < 2^-19 in units of 2^-62, so the truncated terms
+// are below 2^-59 and the result is within 2^-59 before its rounding to 53 bits.  Where x is not
+// positive and normal: ok = false.
 WZ_HD double wide_rsqrt(double x, bool& ok) {
     const uint64_t u = double_bits(x);
     const int e = int(u >> 52);                                // the sign included
