@@ -33,18 +33,23 @@ namespace {
 // blocks (32 warps, 64 registers); three blocks 86 us / 0.53 / 7.5 ms, two 97 us / 0.71 / 9.2 ms,
 // 64 x 4 tiles 88 us / 0.58 / 7.55 ms, 128-thread blocks (eight) 84 us / 0.58 / 7.8 ms, a copy of the
 // code per sweep (128 x 2 and 32 x 8 tiles) 98 us / 0.63 / 7.85 ms; the loop over the fields rolled
-// (a quarter of the code): 77 us.
-// The linear pass (LIN, interface_linear first, the rest compacted) at 256^2 / 512^2 / 800^2 /
-// 1024^2 / 4096^2: 100 / 182 / 305 / 431 us / 5.2 ms with three blocks, 77 / 173 / 364 / 550 us / 7.5 ms
-// without it.  It pays where most interfaces pass, so lines of kLinearMin cells and more take
-// it; a single wave of blocks (short 1D lines) waits for its slowest block, which pays for both
-// passes, and does without (a rollout at 8192 cells 7.7 ms without, 8.2 ms with).
+// (a quarter of the code): 77 us.  (Compared before the weights were made exactly odd and the
+// linear pass unit-free; the chosen shape takes 80 us / 0.60 / 8.8 ms since.)
+// The linear pass (LIN, interface_linear first, the rest compacted, three blocks): both sweeps at
+// 800^2 / 1024^2 / 4096^2 310 / 440 us / 5.2 ms with it, 376 / 597 us / 8.8 ms without, on smooth
+// waves and jumps; at 256^2 / 512^2 100 / 182 against 78 / 179 us.  A step of a developed flow (400
+// steps on): 700^2 1.22 / 1.15 ms, 1024^2 2.01 / 2.16.  On random cells, where nearly every
+// interface takes both, 1024^2 2.98 / 2.89 ms, 4096^2 45.3 / 43.3, 2^20 cells of 1D 1.13 / 1.04
+// (smooth 0.50 / 0.69).  So lines of kLinearMin cells and more take it, where most interfaces of a
+// resolved flow pass and the others lose 3 to 9 %; a single wave of blocks (short 1D lines) waits
+// for its slowest block, which pays for both passes, and does without (a rollout at 8192 cells
+// 7.7 ms without, 8.2 ms with).
 // Long 1D lines use 251-interface tiles (256 cells with the halo: one full round of the cell
-// and difference passes; a 2^20-cell step 0.52 ms, without the linear pass 0.70 ms); short
+// and difference passes; a 2^20-cell step 0.50 ms, without the linear pass 0.69 ms); short
 // ones (fewer tiles than twice the SM count) use 64-interface tiles of 64 threads so that
 // every SM gets work.  GEN = 2 projects F and U (twice the difference vectors a thread) and runs
-// best with two blocks and 128 registers (a 640 x 777 local-LF step 1.76 ms; three blocks 1.81,
-// four 1.85 ms).
+// best with two blocks and 128 registers (a 640 x 777 local-LF step 1.76 ms, 1.80 since the
+// weights are exactly odd; three blocks 1.81, four 1.85 ms).
 constexpr int kLinearMin = 640;
 template <int NV, bool SMALL = false> struct Tile { static constexpr int TI = 251, TA = 1, THREADS = 256; };
 template <int NV> struct Tile<NV, true> { static constexpr int TI = 64, TA = 1, THREADS = 64; };

@@ -3,19 +3,20 @@
 // Why.  GB300 issues one FP64 instruction per SM sub-partition every 64 cycles, and its 32-bit
 // integer and FMA pipes one every 2: a 64 x 64-bit product of which only the top half is kept
 // is three 32 x 32 multiply-adds, an addition two instructions.  A reconstruction is 46 FP64
-// instructions (2,944 cycles of a sub-partition's FP64 unit) or about 325 ALU and 270
-// multiply-add ones, on pipes that otherwise idle; where the weights hardly differ from the
+// instructions (2,944 cycles of a sub-partition's FP64 unit) or some 650 ALU and multiply-add
+// ones, on pipes that otherwise idle; where the weights hardly differ from the
 // optimal ones (wide_linear) about 150 in all.  Measured with the FP64 weights before and these
 // after (with the integer projection of euler_device.cuh in the solver): wenozn_reconstruct
-// 1.24 -> 0.24 ms per side of 2^24 points, the 2D Euler step 99.9 -> 18.9 ms at 4096^2 and 6.5 ->
-// 1.53 ms at 1024^2, the 1D step 2.63 -> 0.52 ms at 2^20 cells.
+// 1.24 -> 0.24 ms per side of 2^24 points, the 2D Euler step 99.9 -> 19.0 ms at 4096^2 and 6.5 ->
+// 1.54 ms at 1024^2, the 1D step 2.63 -> 0.50 ms at 2^20 cells.
 //
 // Precision.  Every quantity carries a 64-bit mantissa (block floating point: integers with a
 // common exponent), every truncation stays below that of a 53-bit one, so the result is
 // closer to the exact value than the double evaluation's: against binary128, over 3 10^5
-// stencils each, the rms error of f^ - c relative to the largest difference is 1.3e-17 on random
-// data (double 2.9e-17), 2.4e-17 on smooth data (5.0e-17), the largest 6.9e-17 and 5.9e-17
-// (2.4e-16, 2.3e-16).  Nothing overflows or underflows: the exponents are integers of their own.
+// stencils each, the rms error of f^ - c relative to the largest difference is 6.3e-18 on random
+// differences (double 3.3e-17), 4.7e-18 on smooth data (4.7e-17), the largest 1.3e-16 and 1.1e-16
+// (3.4e-16, 2.3e-16).  Nothing overflows or underflows on the way: the exponents are integers of
+// their own (a result below the normal range becomes 0).
 //
 // Derivation, from the first differences D1..D4 of the stencil (see wenozn_device.cuh for
 // the scheme).  With s_k the second differences, 3 IS_k is a binary form in the two differences
