@@ -327,3 +327,23 @@ def test_gpu_plateaus_in_a_batch(orc):
         P = orc.problem(1, n, 1, dx=0.01)
         want, _ = orc.rollout_jvp_quad(P, a, a, orc.cfl_dt(P, a), 1)
         assert np.abs(got[:, o:o + n] - want[:, 0]).max() <= 1e-12 * np.abs(want).max()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [2000, 20001])
+@pytest.mark.parametrize("f", [2.0 ** 20, 2.0 ** 36, 2.0 ** 40])
+def test_gpu_adjoint_in_velocity_units(n, f):
+    """The reverse makes the same check, in both its kernels: with S = diag(1, f, f^2) the RHS of S U is
+    f S L(U), so J(S U)^T S^-1 lam = f S^-1 J(U)^T lam, to 1e-10 (the adjoint tests' figure)."""
+    import torch
+    from paper_2004_07954_gb300 import build, wenozn as W
+    build.build()
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    p = W.wenozn_problem_init(W.WENOZN_EULER_1D, n, dx=1e-3, bc_x=W.WENOZN_BC_PERIODIC)
+    ws, S = W.vjp_workspace(p), np.array([1.0, f, f * f])[:, None, None]
+    U, lam = _line(n)[:, None], np.random.default_rng(3).normal(size=(3, 1, n))
+    one, big = torch.empty_like(dev(U)), torch.empty_like(dev(U))
+    W.wenozn_rhs_vjp(p, dev(U), dev(lam), one, ws)
+    W.wenozn_rhs_vjp(p, dev(U * S), dev(lam / S), big, ws)
+    got, want = big.cpu().numpy() * S / f, one.cpu().numpy()
+    assert np.abs(got - want).max() <= 1e-10 * np.abs(want).max()
